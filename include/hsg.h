@@ -81,8 +81,8 @@ enum {
                           * spins and bonds (28 N bytes) exceed three quarters of
                           * the device's L2, so that the sweep streams much of it
                           * from HBM; else GLOBAL */
-  HSG_KERNEL_GLOBAL = 1, /* one thread per site, neighbours through L1/L2 (heat-bath:
-                          * one thread per six-plane column, carrying its column's
+  HSG_KERNEL_GLOBAL = 1, /* one thread per one to four sites of a column, neighbours through L1/L2 (heat-bath from
+                          * L = 224: one thread per six-plane column, carrying its column's
                           * neighbours; the same results) */
   HSG_KERNEL_SLAB = 2,   /* z-marching tiles: other colour staged in shared memory */
   /* Temporally blocked over-relaxation: each over-relaxation sweep

@@ -269,31 +269,6 @@ __device__ __forceinline__ float4 renorm_spin(float4 v) {
   return v;
 }
 
-// The spins of one colour: float4 per site, or three component arrays
-// (packed layout).  Both hand the site code the same float4 values, so the
-// arithmetic -- and the result -- is the same in either layout.
-struct SpinsF4 {
-  float4* p;
-  __device__ __forceinline__ float4 ldg(uint32_t q) const { return __ldg(p + q); }
-  __device__ __forceinline__ float4 ld(uint32_t q) const { return p[q]; }
-  __device__ __forceinline__ void st(uint32_t q, float4 v) const { p[q] = v; }
-};
-struct SpinsSoA {
-  float* p;       // component 0; components 1 and 2 at + stride, + 2 stride
-  size_t stride;  // N/2
-  __device__ __forceinline__ float4 ldg(uint32_t q) const {
-    return make_float4(__ldg(p + q), __ldg(p + stride + q), __ldg(p + 2 * stride + q), 0.0f);
-  }
-  __device__ __forceinline__ float4 ld(uint32_t q) const {
-    return make_float4(p[q], p[stride + q], p[2 * stride + q], 0.0f);
-  }
-  __device__ __forceinline__ void st(uint32_t q, float4 v) const {
-    p[q] = v.x;
-    p[stride + q] = v.y;
-    p[2 * stride + q] = v.z;
-  }
-};
-
 // What one site of a half-sweep reads: its six other-colour neighbours and
 // bonds, its own spin, its index q and its Philox site number.
 struct SiteInputs {
@@ -303,8 +278,6 @@ struct SiteInputs {
   uint32_t q, site;
 };
 
-// Gather the inputs of site (x = 2 xh + p, y, z) of colour `colour` (layout
-// at the top of this file).  Indices are 32-bit: q < N/2 <= 1624^3/2 < 2^31.
 // Indices a site of colour `colour` at (x = 2 xh + p, y, z) reads: its own
 // q, its six other-colour neighbours (periodic wrap by compare-and-select,
 // no power-of-2 assumption) and its Philox site number x + y L + z L^2.
@@ -330,36 +303,7 @@ __host__ __device__ __forceinline__ SiteIndex site_index(uint32_t xh, uint32_t y
   return i;
 }
 
-template <int U, class Spins>
-__device__ __forceinline__ void gather_site_in(SiteInputs& in, Spins own, Spins oth, const float* __restrict__ jx_own,
-                                               const float* __restrict__ jy_own, const float* __restrict__ jz_own,
-                                               const float* __restrict__ jx_oth, const float* __restrict__ jy_oth,
-                                               const float* __restrict__ jz_oth, uint32_t xh, uint32_t y, uint32_t z,
-                                               uint32_t L, uint32_t Lh, uint32_t colour) {
-  const SiteIndex ix = site_index(xh, y, z, L, Lh, colour);
-  const uint32_t q = ix.q, q_xp = ix.q_xp, q_xm = ix.q_xm, q_yp = ix.q_yp, q_ym = ix.q_ym, q_zp = ix.q_zp,
-                 q_zm = ix.q_zm;
-  in.sxp = oth.ldg(q_xp);
-  in.sxm = oth.ldg(q_xm);
-  in.syp = oth.ldg(q_yp);
-  in.sym = oth.ldg(q_ym);
-  in.szp = oth.ldg(q_zp);
-  in.szm = oth.ldg(q_zm);
-  in.jxp = __ldg(jx_own + q);
-  in.jxm = __ldg(jx_oth + q_xm);
-  in.jyp = __ldg(jy_own + q);
-  in.jym = __ldg(jy_oth + q_ym);
-  in.jzp = __ldg(jz_own + q);
-  in.jzm = __ldg(jz_oth + q_zm);
-  in.s = make_float3(0.0f, 0.0f, 0.0f);
-  if constexpr (U != U_HB) {
-    const float4 o = own.ld(q);
-    in.s = make_float3(o.x, o.y, o.z);
-  }
-  in.q = q;
-  in.site = ix.site;
-}
-
+// The inputs of one site from float4 spins.
 template <int U>
 __device__ __forceinline__ void gather_site(SiteInputs& in, const float4* __restrict__ own,
                                             const float4* __restrict__ oth, const float* __restrict__ jx_own,
@@ -367,8 +311,26 @@ __device__ __forceinline__ void gather_site(SiteInputs& in, const float4* __rest
                                             const float* __restrict__ jx_oth, const float* __restrict__ jy_oth,
                                             const float* __restrict__ jz_oth, uint32_t xh, uint32_t y, uint32_t z,
                                             uint32_t L, uint32_t Lh, uint32_t colour) {
-  gather_site_in<U>(in, SpinsF4{const_cast<float4*>(own)}, SpinsF4{const_cast<float4*>(oth)}, jx_own, jy_own, jz_own,
-                    jx_oth, jy_oth, jz_oth, xh, y, z, L, Lh, colour);
+  const SiteIndex ix = site_index(xh, y, z, L, Lh, colour);
+  in.sxp = __ldg(oth + ix.q_xp);
+  in.sxm = __ldg(oth + ix.q_xm);
+  in.syp = __ldg(oth + ix.q_yp);
+  in.sym = __ldg(oth + ix.q_ym);
+  in.szp = __ldg(oth + ix.q_zp);
+  in.szm = __ldg(oth + ix.q_zm);
+  in.jxp = __ldg(jx_own + ix.q);
+  in.jxm = __ldg(jx_oth + ix.q_xm);
+  in.jyp = __ldg(jy_own + ix.q);
+  in.jym = __ldg(jy_oth + ix.q_ym);
+  in.jzp = __ldg(jz_own + ix.q);
+  in.jzm = __ldg(jz_oth + ix.q_zm);
+  in.s = make_float3(0.0f, 0.0f, 0.0f);
+  if constexpr (U != U_HB) {
+    const float4 o = own[ix.q];
+    in.s = make_float3(o.x, o.y, o.z);
+  }
+  in.q = ix.q;
+  in.site = ix.site;
 }
 
 // Form h (Eq. 2) and apply update U: the site's new spin.
@@ -406,20 +368,111 @@ __device__ __forceinline__ void half_sweep_site(float4* __restrict__ own, const 
   finish_site<U>(in, own, colour, sweep_lo, sweep_hi, k0, k1, beta, step, hits, hit0);
 }
 
-// One site of a half-sweep in the packed layout (same arithmetic).
-template <int U>
-__device__ __forceinline__ void half_sweep_site_packed(SpinsSoA own, SpinsSoA oth, const float* __restrict__ jx_own,
-                                                       const float* __restrict__ jy_own,
-                                                       const float* __restrict__ jz_own,
-                                                       const float* __restrict__ jx_oth,
-                                                       const float* __restrict__ jy_oth,
-                                                       const float* __restrict__ jz_oth, uint32_t xh, uint32_t y,
-                                                       uint32_t z, uint32_t L, uint32_t Lh, uint32_t colour,
-                                                       uint32_t sweep_lo, uint32_t sweep_hi, uint32_t k0, uint32_t k1,
-                                                       float beta, float step, int hits) {
-  SiteInputs in;
-  gather_site_in<U>(in, own, oth, jx_own, jy_own, jz_own, jx_oth, jy_oth, jz_oth, xh, y, z, L, Lh, colour);
-  own.st(in.q, site_result<U>(in, colour, sweep_lo, sweep_hi, k0, k1, beta, step, hits));
+// Element q of array b: the byte offset is formed in Off -- 32 bits where
+// every offset fits, which the load and store instructions then add to the
+// array's base themselves (no 64-bit address arithmetic per access).
+template <class Off, class T>
+__device__ __forceinline__ T* elem(T* b, uint32_t q) {
+  return reinterpret_cast<T*>(reinterpret_cast<char*>(b) + (Off)q * (Off)sizeof(T));
+}
+template <class Off, class T>
+__device__ __forceinline__ const T* elem(const T* b, uint32_t q) {
+  return reinterpret_cast<const T*>(reinterpret_cast<const char*>(b) + (Off)q * (Off)sizeof(T));
+}
+
+// One colour of a lattice as update_rows sees it, in either spin layout
+// (float4 per spin, or three component arrays `stride` floats apart: both
+// hand the site code the same values, so the results are the same).
+template <bool PACKED>
+struct RowLattice {
+  float4* own;        // packed: component 0, as are the other colour's
+  const float4* oth;
+  const float *jx_own, *jy_own, *jz_own, *jx_oth, *jy_oth, *jz_oth;
+  size_t stride;
+  uint32_t L, Lh, colour;
+  template <class Off>
+  __device__ __forceinline__ float4 other(uint32_t q) const {
+    if constexpr (PACKED) {
+      const float* b = reinterpret_cast<const float*>(oth);
+      return make_float4(__ldg(elem<Off>(b, q)), __ldg(elem<Off>(b + stride, q)), __ldg(elem<Off>(b + 2 * stride, q)),
+                         0.0f);
+    } else {
+      return __ldg(elem<Off>(oth, q));
+    }
+  }
+  template <class Off>
+  __device__ __forceinline__ float3 old(uint32_t q) const {
+    if constexpr (PACKED) {
+      const float* b = reinterpret_cast<const float*>(own);
+      return make_float3(*elem<Off>(b, q), *elem<Off>(b + stride, q), *elem<Off>(b + 2 * stride, q));
+    } else {
+      const float4 v = *elem<Off>(own, q);
+      return make_float3(v.x, v.y, v.z);
+    }
+  }
+  template <class Off>
+  __device__ __forceinline__ void put(uint32_t q, float4 v) const {
+    if constexpr (PACKED) {
+      float* b = reinterpret_cast<float*>(own);
+      *elem<Off>(b, q) = v.x;
+      *elem<Off>(b + stride, q) = v.y;
+      *elem<Off>(b + 2 * stride, q) = v.z;
+    } else {
+      *elem<Off>(own, q) = v;
+    }
+  }
+};
+
+// What the random updates draw from.
+struct DrawArgs {
+  uint32_t sweep_lo, sweep_hi, k0, k1;
+  float beta, step;
+  int hits, hit0;
+};
+
+// Update U on the R sites of colour a.colour in column xh of plane z, rows
+// y0 .. y0 + R - 1 (R divides L, y0 is a multiple of R); p0 = (colour + y0 + z)
+// mod 2, a constant at the call where R is even.  The indices are those of
+// site_index: the column's other-colour spin of row y is the y neighbour of
+// rows y - 1 and y + 1 and one of row y's x neighbours, and is loaded once.
+template <int U, int R, class Off, bool PACKED>
+__device__ __forceinline__ void update_rows(const RowLattice<PACKED>& a, uint32_t xh, uint32_t y0, uint32_t z,
+                                            uint32_t p0, const DrawArgs& d) {
+  const uint32_t L = a.L, Lh = a.Lh, plane = L * Lh;
+  const uint32_t zo = z * plane, zpo = z + 1 == L ? 0u : zo + plane, zmo = z == 0 ? (L - 1) * plane : zo - plane;
+  const uint32_t r0 = y0 * Lh + xh;                               // in-plane index of row y0
+  const uint32_t r_m = y0 == 0 ? (L - 1) * Lh + xh : r0 - Lh;     // row y0 - 1
+  const uint32_t r_p = y0 + R == L ? xh : r0 + (uint32_t)R * Lh;  // row y0 + R
+  const uint32_t dxp = xh + 1 == Lh ? 1u - Lh : 1u, dxm = xh == 0 ? Lh - 1u : 0xFFFFFFFFu;  // modulo 2^32
+  float4 o_m = a.template other<Off>(zo + r_m), o_0 = a.template other<Off>(zo + r0);
+#pragma unroll
+  for (int k = 0; k < R; ++k) {
+    const uint32_t r = r0 + (uint32_t)k * Lh, q = zo + r;
+    const uint32_t p = (p0 ^ (uint32_t)k) & 1u;  // x = 2 xh + p
+    const float4 o_p = a.template other<Off>(zo + (k + 1 < R ? r + Lh : r_p));
+    const float4 side = a.template other<Off>(q + (p ? dxp : dxm));
+    SiteInputs in;
+    in.sxp = p ? side : o_0;
+    in.sxm = p ? o_0 : side;
+    in.syp = o_p;
+    in.sym = o_m;
+    in.szp = a.template other<Off>(zpo + r);
+    in.szm = a.template other<Off>(zmo + r);
+    in.jxp = __ldg(elem<Off>(a.jx_own, q));
+    in.jxm = __ldg(elem<Off>(a.jx_oth, p ? q : q + dxm));
+    in.jyp = __ldg(elem<Off>(a.jy_own, q));
+    in.jym = __ldg(elem<Off>(a.jy_oth, zo + (k > 0 ? r - Lh : r_m)));
+    in.jzp = __ldg(elem<Off>(a.jz_own, q));
+    in.jzm = __ldg(elem<Off>(a.jz_oth, zmo + r));
+    in.s = make_float3(0.0f, 0.0f, 0.0f);
+    if constexpr (U != U_HB) in.s = a.template old<Off>(q);
+    in.q = q;
+    in.site = (2 * xh + p) + (y0 + (uint32_t)k) * L + z * L * L;
+    a.template put<Off>(q, site_result<U>(in, a.colour, d.sweep_lo, d.sweep_hi, d.k0, d.k1, d.beta, d.step, d.hits,
+                                          d.hit0));
+    o_m = o_0;
+    o_0 = o_p;
+  }
 }
 
 // Unsigned division by an invariant d (Granlund & Montgomery, "Division by

@@ -4,10 +4,10 @@
 // ordered).
 //
 // Two variants over the colour-split layout of hsg_device.cuh:
-//   global : one thread per updated site; the six neighbours come through
-//            L1/L2 (the lattice is streamed once per half-sweep from HBM).
-//            Its heat-bath launches march a thread up a short column of
-//            planes instead (k_half_sweep_column).
+//   global : one thread per one, two or four sites of a column of rows; the
+//            neighbours come through L1/L2 (the lattice is streamed once per
+//            half-sweep from HBM).  Its heat-bath launches on large lattices
+//            march a thread up a short column of planes (k_half_sweep_column).
 //   slab   : a CTA owns a (32 xh) x (4 y) column tile and marches up a chunk
 //            of z planes.  The other colour's plane z (with a one-site halo)
 //            is staged in shared memory for the x and y neighbours; planes
@@ -26,40 +26,67 @@ __device__ __forceinline__ uint32_t site_number(int xh, int p, int y, int z, int
 }
 
 // ---------------------------------------------------------------------------
-// Global variant.  Block shape (chosen at launch): 64 x 2 threads when a row
-// holds at least 64 sites of a colour, else 32 x 4 (measured at L = 256:
-// 64 x 2 and 128 x 2 beat 32 x 8 by ~4 %).
+// Global variant.  A thread updates R consecutive rows of one column of a
+// plane (update_rows, hsg_device.cuh); the (xh, row group) pairs of a plane
+// are numbered through, so that a row of any length fills its warps, and one
+// multiply-shift division per thread recovers them.  Byte offsets are 32-bit
+// up to L = 812 (16 N/2 < 2^32) and added to the arrays' bases by the load
+// instructions.  Measured on GB300 per half-sweep in replayed graphs,
+// against one site per thread on 64 x 2 or 32 x 4 blocks (half of their
+// threads idle at L/2 = 33 or 65) with 64-bit addresses:
+//   L = 66   OR 3.57 -> 2.30, 4-hit Metropolis 7.10 -> 4.10, heat-bath (column
+//            kernel below) 6.48 -> 3.08 us
+//   L = 100  5.37 -> 4.10, 13.3 -> 11.2, 10.2 -> 7.2 us
+//   L = 128  7.94 -> 6.66, 20.7 -> 20.5, 15.1 -> 12.3 us
+//   L = 130  11.0 -> 7.9, 32.8 -> 22.6, 17.5 -> 13.3 us
+//   L = 256  85.0 -> 83.5, 160.6 -> 154.4 us; heat-bath stays with the column
+//            kernel (93.2 us; 95.8 with two rows per thread)
+//   packed, L = 130: 12.1 -> 7.7, 35.7 -> 23.6, 21.4 -> 13.9 us; L = 256: 89.6 ->
+//            84.3, 170.6 -> 165, 102.9 -> 94.1 us
+// Rows per thread (row_shape below): the own-column neighbour of one row is
+// the y neighbour of the next, so R rows load 2 + 2/R + 1 neighbours each
+// instead of five; but R rows per thread leave 1/R of the threads, and below
+// about 10^6 sites those are too few (L = 64, 4-hit Metropolis: 4.1, 5.1,
+// 7.2 us with one, two, four rows).
+// A grid of exactly the resident CTAs looping over the sites (grid-stride,
+// or an equal contiguous range per CTA) made the 4-hit Metropolis half-sweep at
+// L = 128 slower: 28.1-30.1 us against 25.9 us.
 // ---------------------------------------------------------------------------
 constexpr int G_THREADS = 128;
+constexpr int kMaxOff32L = 812;  // L^3/2 * 16 bytes < 2^32
 
-// Indices are 32-bit: q < N/2 <= 1624^3/2 < 2^31.  The over-relaxation
-// kernel is held to 32 registers so that 16 blocks (full occupancy) fit on
-// an SM (measured at L = 256: OR 92 us at 32 registers vs 99 us at 36-40);
-// Metropolis, which would spill, keeps its registers.  A grid of exactly
-// the resident CTAs looping over the sites (grid-stride, or an equal
-// contiguous range per CTA; 10 or 12 CTAs per SM) made the 4-hit Metropolis
-// half-sweep at L = 128 slower: 28.1-30.1 us against 25.9 us.
-template <int U>
-__global__ void __launch_bounds__(G_THREADS, U == U_OR ? 16 : 1) k_half_sweep_global(const SweepArgs a) {
-  const uint32_t xh = blockIdx.x * blockDim.x + threadIdx.x;
-  const uint32_t y = blockIdx.y * blockDim.y + threadIdx.y;
-  const uint32_t z = blockIdx.z;
-  const uint32_t L = a.L, Lh = a.Lh;
-  if (xh >= Lh || y >= L) return;
-  uint32_t sweep_lo = a.sweep_lo, sweep_hi = a.sweep_hi;
+template <int U, int R, int MIN_BLOCKS, class Off, bool PACKED>
+__global__ void __launch_bounds__(G_THREADS, MIN_BLOCKS)
+    k_half_sweep_rows(const SweepArgs a, FastDiv by_lh, uint32_t columns) {
+  const uint32_t t = blockIdx.x * G_THREADS + threadIdx.x;
+  if (t >= columns) return;
+  const uint32_t g = fast_div(t, by_lh), xh = t - g * (uint32_t)a.Lh, y0 = g * R, z = blockIdx.y;
+  const RowLattice<PACKED> lat{a.own,    a.oth,    a.jx_own, a.jy_own,      a.jz_own,       a.jx_oth,
+                               a.jy_oth, a.jz_oth, a.stride, (uint32_t)a.L, (uint32_t)a.Lh, (uint32_t)a.colour};
+  DrawArgs d{a.sweep_lo, a.sweep_hi, a.k0, a.k1, a.beta, a.step, a.hits, 0};
   if constexpr (U != U_OR) {
     if (a.sweep_ptr) {
       const unsigned long long sw = *a.sweep_ptr;
-      sweep_lo = (uint32_t)sw;
-      sweep_hi = (uint32_t)(sw >> 32);
+      d.sweep_lo = (uint32_t)sw;
+      d.sweep_hi = (uint32_t)(sw >> 32);
     }
   }
-  half_sweep_site<U>(a.own, a.oth, a.jx_own, a.jy_own, a.jz_own, a.jx_oth, a.jy_oth, a.jz_oth, xh, y, z, L, Lh,
-                     (uint32_t)a.colour, sweep_lo, sweep_hi, a.k0, a.k1, a.beta, a.step, a.hits);
+  // x = 2 xh + p.  With R even, y0 is even and p the same for the block:
+  // one branch, and no selects inside.
+  const uint32_t p = ((uint32_t)a.colour + (R == 1 ? y0 : 0u) + z) & 1u;
+  if constexpr (R == 1) {
+    update_rows<U, R, Off>(lat, xh, y0, z, p, d);
+  } else {
+    if (p)
+      update_rows<U, R, Off>(lat, xh, y0, z, 1u, d);
+    else
+      update_rows<U, R, Off>(lat, xh, y0, z, 0u, d);
+  }
 }
 
-// Heat-bath half-sweeps of the global variant: one thread per (xh, y)
-// column of the updated colour over ZM_PLANES consecutive planes.  The
+// Heat-bath half-sweeps of the global variant from L = ZM_MIN_L, where they
+// stream from HBM: one thread per (xh, y) column of the updated colour over
+// ZM_PLANES consecutive planes.  The
 // other colour's spins in the thread's own column on planes z-1 and z (the
 // site's -z neighbour and one of its x neighbours) are carried from the
 // plane before, so a site loads four neighbour spins instead of six; the
@@ -77,9 +104,12 @@ __global__ void __launch_bounds__(G_THREADS, U == U_OR ? 16 : 1) k_half_sweep_gl
 // flushed); 32 x 4, 128 x 1, 8 x 16 and 256-thread blocks 89.9-91.1 us;
 // streaming (evict-first) stores of the new spins gained 0.2 us more.
 constexpr int ZM_PLANES = 6;
+// From here on the column march wins: 93.2 against 95.8 us at L = 256; below,
+// the rows kernel does (L = 192 43.6 against 43.2 us, L = 128 15.1 against 12.3,
+// L = 64 5.4 against 3.1 us: six planes per thread are too few threads).
+constexpr int ZM_MIN_L = 224;
 constexpr int ZM_BX = 16, ZM_BY = 8;
 
-template <int U>
 __global__ void __launch_bounds__(G_THREADS, 12) k_half_sweep_column(const SweepArgs a) {
   const uint32_t xh = blockIdx.x * blockDim.x + threadIdx.x;
   const uint32_t y = blockIdx.y * blockDim.y + threadIdx.y;
@@ -119,44 +149,15 @@ __global__ void __launch_bounds__(G_THREADS, 12) k_half_sweep_column(const Sweep
     in.jym = __ldg(a.jy_oth + zo + row_m + xh);
     in.jzp = __ldg(a.jz_own + q);
     in.jzm = __ldg(a.jz_oth + zmo + row + xh);
-    in.s = make_float3(0.0f, 0.0f, 0.0f);
-    if constexpr (U != U_HB) {
-      const float4 o = a.own[q];
-      in.s = make_float3(o.x, o.y, o.z);
-    }
+    in.s = make_float3(0.0f, 0.0f, 0.0f);  // the heat-bath does not read the old spin
     in.q = q;
     in.site = (2 * xh + p) + y * L + z * L * L;
-    a.own[q] = site_result<U>(in, (uint32_t)a.colour, sweep_lo, sweep_hi, a.k0, a.k1, a.beta, a.step, a.hits);
+    a.own[q] = site_result<U_HB>(in, (uint32_t)a.colour, sweep_lo, sweep_hi, a.k0, a.k1, a.beta, a.step, a.hits);
     s_m = s_0;
     s_0 = s_p;
     zmo = zo;
     zo = zpo;
   }
-}
-
-// The global variant over the packed layout (three fp32 arrays per colour,
-// 12 bytes a spin: 60 bytes per over-relaxation update instead of 72).  Same
-// site code on the same values, so bit-identical to the float4 kernel.
-template <int U>
-__global__ void __launch_bounds__(G_THREADS, (U == U_OR || U == U_HB) ? 16 : 1)
-    k_half_sweep_global_packed(const SweepArgs a) {
-  const uint32_t xh = blockIdx.x * blockDim.x + threadIdx.x;
-  const uint32_t y = blockIdx.y * blockDim.y + threadIdx.y;
-  const uint32_t z = blockIdx.z;
-  const uint32_t L = a.L, Lh = a.Lh;
-  if (xh >= Lh || y >= L) return;
-  uint32_t sweep_lo = a.sweep_lo, sweep_hi = a.sweep_hi;
-  if constexpr (U != U_OR) {
-    if (a.sweep_ptr) {
-      const unsigned long long sw = *a.sweep_ptr;
-      sweep_lo = (uint32_t)sw;
-      sweep_hi = (uint32_t)(sw >> 32);
-    }
-  }
-  const SpinsSoA own{reinterpret_cast<float*>(a.own), a.stride};
-  const SpinsSoA oth{const_cast<float*>(reinterpret_cast<const float*>(a.oth)), a.stride};
-  half_sweep_site_packed<U>(own, oth, a.jx_own, a.jy_own, a.jz_own, a.jx_oth, a.jy_oth, a.jz_oth, xh, y, z, L, Lh,
-                            (uint32_t)a.colour, sweep_lo, sweep_hi, a.k0, a.k1, a.beta, a.step, a.hits);
 }
 
 // ---------------------------------------------------------------------------
@@ -256,28 +257,64 @@ int slab_zc(int L, unsigned tiles, int sm_count) {
   return zc < 1 ? 1 : (zc > SLAB_ZC_MAX ? SLAB_ZC_MAX : zc);
 }
 
+template <int U, int R, int MIN_BLOCKS, class Off, bool PACKED>
+void launch_rows(const SweepArgs& a, cudaStream_t s) {
+  const uint32_t columns = (uint32_t)a.Lh * (uint32_t)(a.L / R);
+  k_half_sweep_rows<U, R, MIN_BLOCKS, Off, PACKED>
+      <<<dim3(cdiv(columns, G_THREADS), (unsigned)a.L), G_THREADS, 0, s>>>(a, make_fastdiv((uint32_t)a.Lh), columns);
+}
+
+// Rows per thread and the register bound, by the measurements above and (MB:
+// 4-hit Metropolis; R rows at B resident CTAs of 128):
+//   heat-bath      L = 96 6.2 (R 1) 6.1 (R 2), 128 13.2 / 12.3, 256 97.4 / 95.8 us
+//   MB             L = 128 21.4 / 20.5 / 22.4 (R 4), 192 74.5 / 71.9 / 69.1, 256 171 / 161 / 154 us
+//   OR             L = 128 6.66 / 7.11, 256 83.5 / 89.4 us
+//   packed OR      L = 130 7.7 / 11.2, 192 38.9 / 37.5, 256 89.3 / 84.3 us; heat-bath 130 15.3 / 13.9, 256 105 / 94.1;
+//   packed MB      L = 128 22.2 / 22.8, 192 73.0 / 72.0, 256 170 / 165 us
+template <int U, bool PACKED>
+cudaError_t launch_global(const SweepArgs& a, cudaStream_t s) {
+  constexpr bool MET = U != U_OR && U != U_HB;
+  if (a.L > kMaxOff32L) {
+    launch_rows<U, 1, MET ? 1 : 12, unsigned long long, PACKED>(a, s);
+  } else if constexpr (U == U_OR) {
+    if (PACKED && a.L >= 160)
+      launch_rows<U, 2, 10, uint32_t, PACKED>(a, s);
+    else
+      launch_rows<U, 1, 12, uint32_t, PACKED>(a, s);
+  } else if constexpr (U == U_HB) {
+    if (a.L < 96)
+      launch_rows<U, 1, 12, uint32_t, PACKED>(a, s);
+    else
+      launch_rows<U, 2, PACKED ? 10 : 16, uint32_t, PACKED>(a, s);
+  } else {
+    if (!PACKED && a.L >= 160 && a.L % 4 == 0)
+      launch_rows<U, 4, 1, uint32_t, PACKED>(a, s);
+    else if (a.L >= (PACKED ? 160 : 96))
+      launch_rows<U, 2, 1, uint32_t, PACKED>(a, s);
+    else
+      launch_rows<U, 1, 1, uint32_t, PACKED>(a, s);
+  }
+  return cudaGetLastError();
+}
+
 template <int U>
 cudaError_t launch_kind(int variant, const SweepArgs& a, int sm_count, cudaStream_t s) {
-  if (a.packed) {
-    const dim3 block = a.Lh >= 64 ? dim3(64, 2) : dim3(32, 4);
-    const dim3 grid(cdiv(a.Lh, block.x), cdiv(a.L, block.y), (unsigned)a.L);
-    k_half_sweep_global_packed<U><<<grid, block, 0, s>>>(a);
-  } else if (variant == V_SLAB) {
+  if (a.packed) return launch_global<U, true>(a, s);
+  if (variant == V_SLAB) {
     const unsigned tx = cdiv(a.Lh, TX), ty = cdiv(a.L, SLAB_TY);
     const int zc = slab_zc(a.L, tx * ty, sm_count);
     const dim3 grid(tx, ty, cdiv(a.L, zc));
     k_half_sweep_slab<U><<<grid, dim3(TX, SLAB_TY), 0, s>>>(a, zc);
-  } else {
-    const dim3 block = a.Lh >= 64 ? dim3(64, 2) : dim3(32, 4);
-    const dim3 grid(cdiv(a.Lh, block.x), cdiv(a.L, block.y), (unsigned)a.L);
-    if constexpr (U == U_HB) {
-      const dim3 gcol(cdiv(a.Lh, ZM_BX), cdiv(a.L, ZM_BY), cdiv(a.L, ZM_PLANES));
-      k_half_sweep_column<U><<<gcol, dim3(ZM_BX, ZM_BY), 0, s>>>(a);
-    } else {
-      k_half_sweep_global<U><<<grid, block, 0, s>>>(a);
+    return cudaGetLastError();
+  }
+  if constexpr (U == U_HB) {
+    if (a.L >= ZM_MIN_L) {
+      const dim3 grid(cdiv(a.Lh, ZM_BX), cdiv(a.L, ZM_BY), cdiv(a.L, ZM_PLANES));
+      k_half_sweep_column<<<grid, dim3(ZM_BX, ZM_BY), 0, s>>>(a);
+      return cudaGetLastError();
     }
   }
-  return cudaGetLastError();
+  return launch_global<U, false>(a, s);
 }
 
 }  // namespace

@@ -1,0 +1,65 @@
+"""The global half-sweep kernels at the sizes where their launch rule changes
+(needs a CUDA GPU): one, two or four rows per thread, the heat-bath's column
+march, 32- and 64-bit byte offsets, both spin layouts.  The slab kernel, which
+shares none of their index arithmetic, has to give the same bits."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def hsg():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1006_2566_gb300 import build
+
+    build.build()
+    from paper_1006_2566_gb300 import hsg as h
+
+    return h
+
+
+def updates(hsg):
+    return [(hsg.HSG_OVERRELAX, 0, 1), (hsg.HSG_HEATBATH, 0, 1), (hsg.HSG_METROPOLIS, 0, 2), (hsg.HSG_METROPOLIS, 1, 3),
+            (hsg.HSG_METROPOLIS_OR, 0, 2), (hsg.HSG_METROPOLIS_OR, 1, 2)]
+
+
+def sweep_halves(hsg, lat, kernel):
+    for upd, prop, hits in updates(hsg):
+        for colour in (0, 1):
+            lat.half_sweep(hsg.schedule(T=0.7, hits=hits, proposal=prop, kernel=kernel), upd, colour)
+
+
+# 4, 6: the smallest; 94 | 96: one | two rows; 158 | 160, 162: four rows where
+# 4 divides L, packed two rows; 222 | 224, 226: the column march
+@pytest.mark.parametrize("L", [4, 6, 94, 96, 158, 160, 162, 222, 224, 226])
+def test_global_kernels_equal_the_slab_kernel(hsg, L):
+    outs = []
+    for layout, kernel in ((hsg.HSG_LAYOUT_FLOAT4, hsg.HSG_KERNEL_SLAB), (hsg.HSG_LAYOUT_FLOAT4, hsg.HSG_KERNEL_GLOBAL),
+                           (hsg.HSG_LAYOUT_PACKED, hsg.HSG_KERNEL_GLOBAL)):
+        with hsg.Lattice(L, 17, 2, 1, layout=layout) as lat:
+            lat.generate_couplings()
+            sweep_halves(hsg, lat, kernel)
+            outs.append(lat.spins())
+    assert np.array_equal(outs[0], outs[1])
+    assert np.array_equal(outs[0], outs[2])
+
+
+@pytest.mark.parametrize("L", [812, 814])
+def test_either_side_of_the_32_bit_offsets(hsg, L):
+    """16 L^3/2 passes 2^32 between L = 812 and 814: random sites, the
+    corners and the last plane."""
+    rng = np.random.default_rng(L)
+    sites = np.concatenate([rng.integers(0, L ** 3, 4000), L ** 3 - 1 - rng.integers(0, L * L, 2000),
+                            rng.integers(0, L * L, 2000), [0, L - 1, L * L - 1, L ** 3 - 1]]).astype(np.uint32)
+    outs = []
+    for layout, kernel in ((hsg.HSG_LAYOUT_FLOAT4, hsg.HSG_KERNEL_SLAB), (hsg.HSG_LAYOUT_FLOAT4, hsg.HSG_KERNEL_GLOBAL),
+                           (hsg.HSG_LAYOUT_PACKED, hsg.HSG_KERNEL_GLOBAL)):
+        with hsg.Lattice(L, 3, layout=layout) as lat:
+            lat.generate_couplings()
+            sweep_halves(hsg, lat, kernel)
+            outs.append(hsg.hsg_get_sites(lat.ctx, sites, want_bonds=False)[0])
+    assert np.array_equal(outs[0], outs[1])
+    assert np.array_equal(outs[0], outs[2])
