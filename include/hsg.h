@@ -80,7 +80,9 @@ enum {
   HSG_KERNEL_AUTO = 0,   /* library's choice: HSG_KERNEL_WAVE when the lattice's
                           * spins and bonds (28 N bytes) exceed three quarters of
                           * the device's L2, so that the sweep streams much of it
-                          * from HBM; else GLOBAL */
+                          * from HBM; else GLOBAL.  hsg_sweep runs all sweeps up to
+                          * an energy in one launch where the lattice is small (L <=
+                          * 32, few hits): the same results */
   HSG_KERNEL_GLOBAL = 1, /* one thread per one to four sites of a column, neighbours through L1/L2 (heat-bath from
                           * L = 224: one thread per six-plane column, carrying its column's
                           * neighbours; the same results) */

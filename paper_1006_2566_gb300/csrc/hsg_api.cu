@@ -4,6 +4,7 @@
 // schedule (which kernels run in which order), the energy log and the
 // event-based profiler.  Every step of the Monte Carlo itself runs in the
 // kernels of hsg_sweep.cu and hsg_aux.cu.
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdio>
@@ -469,6 +470,63 @@ hsg_status capture_period(hsg_ctx* c, const hsg_schedule* s, int variant, int pe
   return HSG_OK;
 }
 
+// The main update's kind in a whole-schedule kernel (U_OR: none).
+int main_update(const hsg_schedule* s) {
+  const bool ball = s->proposal == HSG_PROP_BALL;
+  switch (s->kind) {
+    case HSG_METROPOLIS: return ball ? hsg::U_MET_BALL : hsg::U_MET_SPHERE;
+    case HSG_METROPOLIS_OR: return ball ? hsg::U_MET_OR_BALL : hsg::U_MET_OR_SPHERE;
+    case HSG_HEATBATH: return hsg::U_HB;
+    default: return hsg::U_OR;
+  }
+}
+
+// Whether hsg_sweep runs schedule s in the resident kernel
+// (hsg_resident.cu): AUTO only, and neither under the profiler, whose classes
+// are single half-sweeps, nor while the caller captures the stream (what a
+// capture takes, and what it refuses, stays with the half-sweep launches).
+bool use_resident(const hsg_ctx* c, const hsg_schedule* s) {
+  if (s->kernel != HSG_KERNEL_AUTO || c->prof || !hsg::resident_takes(main_update(s), c->L, s->hits)) return false;
+  if (s->kind == HSG_NONE && s->n_or == 0) return false;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(c->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+}
+
+// n_sweeps sweeps in the resident kernel, one launch up to each energy due.
+hsg_status run_resident(hsg_ctx* c, const hsg_schedule* s, int n_sweeps) {
+  const int upd = main_update(s);
+  hsg_status st;
+  for (int k = 0; k < n_sweeps;) {
+    uint64_t m = (uint64_t)(n_sweeps - k);
+    if (s->energy_every > 0) m = std::min(m, (uint64_t)s->energy_every - c->sweep % (uint64_t)s->energy_every);
+    hsg::ResidentArgs a{};
+    a.spins = c->spins;
+    a.J = c->J;
+    a.nh = (size_t)c->Nh;
+    a.packed = c->packed;
+    a.L = (uint32_t)c->L;
+    a.Lh = (uint32_t)c->Lh;
+    a.sweeps = (uint32_t)m;
+    a.per_sweep = (s->kind != HSG_NONE ? 2u : 0u) + 2u * (uint32_t)s->n_or;
+    a.renorm_every = (uint32_t)s->renorm_every;
+    a.k0 = c->k0;
+    a.k1 = c->k1;
+    a.beta = beta_of(s->T);
+    a.step = s->step;
+    a.hits = s->hits;
+    a.sweep_ptr = c->d_ctr;
+    st = launch(c, HSG_PROF_LAYOUT, 1, "resident sweeps kernel", [&] { return hsg::launch_resident(upd, a, c->stream); });
+    if (st != HSG_OK) return st;
+    c->sweep += m;
+    k += (int)m;
+    if (s->energy_every > 0 && c->sweep % (uint64_t)s->energy_every == 0) {
+      if ((st = run_energy(c, c->elog, true)) != HSG_OK) return st;
+      c->elog_n += 1;
+    }
+  }
+  return HSG_OK;
+}
+
 hsg_status grow_elog(hsg_ctx* c, int need) {
   if (need <= c->elog_cap) return HSG_OK;
   int cap = c->elog_cap > 0 ? c->elog_cap : kElogInit;
@@ -669,6 +727,7 @@ hsg_status hsg_sweep(hsg_ctx* c, const hsg_schedule* s, int n_sweeps) {
     st = grow_elog(c, c->elog_n + (int)logged);
     if (st != HSG_OK) return st;
   }
+  if (use_resident(c, s)) return run_resident(c, s, n_sweeps);
   const int variant = pick_variant(c, s->kernel);
   const int swaps = variant == hsg::V_WAVE ? wave_sweeps_per_sweep(s) : 0;
   if (swaps > 0 && !c->spins_alt) {

@@ -17,6 +17,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "hsg_internal.h"
+
 namespace hsg {
 
 // Update kinds of the half-sweep kernels.  U_MET_OR_* is the fused colour
@@ -479,10 +481,6 @@ __device__ __forceinline__ void update_rows(const RowLattice<PACKED>& a, uint32_
 // invariant integers using multiplication", PLDI 1994): with l = ceil(log2 d)
 // and m = floor(2^32 (2^l - d) / d) + 1, n / d = (t + ((n - t) >> s1)) >> s2
 // for every 32-bit n, where t = mulhi(m, n), s1 = min(l, 1), s2 = max(l - 1, 0).
-struct FastDiv {
-  uint32_t m, s1, s2;
-};
-
 // The constants for divisor d >= 1 (host).
 inline FastDiv make_fastdiv(uint32_t d) {
   uint32_t l = 0;

@@ -123,6 +123,34 @@ struct WaveArgs {
 // with `renorm` set to those half-sweeps followed by launch_renorm.
 cudaError_t launch_or_sweep_wave(const WaveArgs& a, int sm_count, cudaStream_t s);
 
+// Unsigned division by an invariant (make_fastdiv, hsg_device.cuh).
+struct FastDiv {
+  uint32_t m, s1, s2;
+};
+
+// Sweeps of one small lattice in one launch (hsg_resident.cu).
+struct ResidentArgs {
+  float4* spins;  // S[2][N/2] (packed: [2][3][N/2] floats), read and written back
+  const float* J;  // J[3][2][N/2]
+  size_t nh;       // N/2
+  bool packed;
+  uint32_t L, Lh;
+  uint32_t sweeps;        // sweeps to run
+  uint32_t per_sweep;     // half-sweeps of a sweep, the main update's two first
+  uint32_t renorm_every;  // 0 = never
+  uint32_t k0, k1;
+  float beta, step;
+  int hits;
+  unsigned long long* sweep_ptr;  // device sweep counter, advanced by `sweeps`
+  // set by launch_resident
+  uint32_t cluster, max_planes, plane;
+  FastDiv by_plane, by_Lh;
+};
+constexpr int kResidentMaxL = 32;
+// `upd`: the main update's kind, or U_OR for over-relaxation only.
+bool resident_takes(int upd, int L, int hits);
+cudaError_t launch_resident(int upd, const ResidentArgs& a, cudaStream_t s);
+
 // Halo-padded copy of the colour-split bonds, read by the sweep's tensor
 // boxes: Jp[a][z][yp][xp] with a = 2d + c, yp = y + 2 in [0, L + 4) and
 // xp = xh + 2 in [0, W), W = roundup(L/2 + 4, 4), holding the bond of

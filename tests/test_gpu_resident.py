@@ -1,0 +1,85 @@
+"""The resident kernel (whole sweeps of a lone small lattice in one launch)
+against the half-sweep launches, bit for bit (needs a CUDA GPU)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def hsg():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1006_2566_gb300 import build
+
+    build.build()
+    from paper_1006_2566_gb300 import hsg as h
+
+    return h
+
+
+def chain(hsg, L, kernel, layout, stream, **kw):
+    """Calls that start and end between cadences, a counter that crosses 2^32
+    and one set by hand, spins set from outside: spins, log, counter, E/N."""
+    sched = hsg.schedule(kernel=kernel, T=0.6, renorm_every=3, energy_every=2, **kw)
+    with hsg.Lattice(L, 29, 1, 1, stream=stream, layout=layout) as lat:
+        lat.generate_couplings()
+        lat.sweep(sched, 1)
+        lat.sweep_count = 2 ** 32 - 4
+        lat.sweep(sched, 7)
+        mid = lat.spins()
+        lat.set_spins(mid[::-1].reshape(-1, 3)[:, ::-1].reshape(-1).copy())
+        lat.sweep(sched, 4)
+        return lat.spins(), lat.energy_log(), lat.sweep_count, lat.energy(), mid
+
+
+# 4, 6, 8: one CTA; 10, 12, 14: eight CTAs, one or two planes each; 16, 18,
+# 22, 30: sixteen, ragged; 32: 1024 threads each; 34: past the rule
+@pytest.mark.parametrize("L", [4, 6, 8, 10, 12, 14, 16, 18, 22, 30, 32, 34])
+def test_resident_sweeps_equal_half_sweep_launches(hsg, L):
+    kinds = [dict(kind=hsg.HSG_METROPOLIS, hits=1, proposal=hsg.HSG_PROP_SPHERE, n_or=0),
+             dict(kind=hsg.HSG_METROPOLIS, hits=3, proposal=hsg.HSG_PROP_BALL, n_or=2),
+             dict(kind=hsg.HSG_HEATBATH, n_or=1),
+             dict(kind=hsg.HSG_METROPOLIS_OR, hits=2, proposal=hsg.HSG_PROP_SPHERE, n_or=0),
+             dict(kind=hsg.HSG_METROPOLIS_OR, hits=2, proposal=hsg.HSG_PROP_BALL, n_or=1),
+             dict(kind=hsg.HSG_NONE, n_or=2),
+             # the most hits that the rule lets in, and one more
+             dict(kind=hsg.HSG_METROPOLIS, hits=16 if L <= 16 else 5 if L <= 24 else 2, proposal=1, n_or=1),
+             dict(kind=hsg.HSG_METROPOLIS, hits=17 if L <= 16 else 6 if L <= 24 else 3, proposal=0, n_or=1)]
+    for i, kw in enumerate(kinds):
+        layout = (hsg.HSG_LAYOUT_FLOAT4, hsg.HSG_LAYOUT_PACKED)[i % 2]
+        stream = torch.cuda.Stream() if i % 3 else None
+        want = chain(hsg, L, hsg.HSG_KERNEL_GLOBAL, layout, stream, **kw)
+        got = chain(hsg, L, hsg.HSG_KERNEL_AUTO, layout, stream, **kw)
+        for a, b in zip(got, want):
+            assert np.array_equal(a, b), (L, kw)
+
+
+def test_nothing_to_do_only_counts(hsg):
+    with hsg.Lattice(16, 3) as lat:
+        lat.generate_couplings()
+        s0 = lat.spins()
+        lat.sweep(hsg.schedule(kind=hsg.HSG_NONE, n_or=0, energy_every=2), 5)
+        assert lat.sweep_count == 5 and len(lat.energy_log()) == 2
+        assert np.array_equal(lat.spins(), s0)
+
+
+def test_a_captured_sweep_replays_as_new_sweeps(hsg):
+    """A caller's own stream capture takes the half-sweep launches, which
+    read the sweep counter from the device: each replay is the next sweep."""
+    L, kw = 16, dict(kind=hsg.HSG_METROPOLIS, hits=2, proposal=1, T=0.7, n_or=1, renorm_every=9)
+    stream = torch.cuda.Stream()
+    with hsg.Lattice(L, 5, stream=stream) as lat, hsg.Lattice(L, 5) as ref:
+        for x in (lat, ref):
+            x.generate_couplings()
+        ref.sweep(hsg.schedule(**kw), 3)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=stream):
+            lat.sweep(hsg.schedule(**kw), 1)
+        for _ in range(3):
+            with torch.cuda.stream(stream):
+                g.replay()
+        torch.cuda.synchronize()
+        assert np.array_equal(lat.spins(), ref.spins())
