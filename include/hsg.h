@@ -121,7 +121,7 @@ enum {
   HSG_PROF_OVERRELAX = 2,
   HSG_PROF_METROPOLIS = 3,
   HSG_PROF_HEATBATH = 4,
-  HSG_PROF_ENERGY = 5,   /* both energy kernels */
+  HSG_PROF_ENERGY = 5,   /* the energy kernel (a logged energy: both of its kernels) */
   HSG_PROF_RENORM = 6,
   HSG_PROF_OVERRELAX_RENORM = 7, /* an over-relaxation wave sweep that also renormalises what it stores
                                   * (a renormalisation due right after it, fused into it) */

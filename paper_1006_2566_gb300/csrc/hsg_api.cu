@@ -24,6 +24,7 @@ namespace {
 constexpr int kVersion = 100;  // 0.1.0
 constexpr int kMaxL = 1624;    // L^3 < 2^32: site indices are 32-bit Philox counters
 constexpr int kElogInit = 64;
+constexpr int kCounters = 4;   // words at hsg_ctx::d_ctr
 constexpr long long kMaxGraphPeriod = 64;  // longest sweep period captured as one graph
 
 thread_local std::string g_thread_error;
@@ -64,7 +65,6 @@ struct hsg_ctx {
   void* stage = nullptr;  // site-major staging for host copies
   size_t stage_bytes = 0;
   double* partials = nullptr;  // energy first-pass sums
-  double* e_out = nullptr;     // hsg_energy result
   double* elog = nullptr;      // energy log
   int elog_cap = 0, elog_n = 0;
   double* host_e = nullptr;  // pinned, 2 doubles: E/N and the bond-box wait flag
@@ -76,7 +76,8 @@ struct hsg_ctx {
   uint64_t launches = 0;
   // Device counters: [0] the sweep counter the kernels read, [1] the energy
   // log position; the host mirrors both (sweep, elog_n).  [2] is set by a
-  // temporally blocked sweep whose bounded wait for a bond box gave up.
+  // temporally blocked sweep whose bounded wait for a bond box gave up.  [3]
+  // counts the energy kernel's blocks, zero between launches.
   unsigned long long* d_ctr = nullptr;
   // One captured period of sweeps (see hsg_sweep), replayed while the
   // schedule, the kernel variant and the energy log buffer stay the same.
@@ -192,7 +193,6 @@ void release(hsg_ctx* c) {
   dev_free(c->Jpad, s);
   dev_free(c->stage, s);
   dev_free(c->partials, s);
-  dev_free(c->e_out, s);
   dev_free(c->elog, s);
   dev_free(c->d_ctr, s);
   cudaStreamSynchronize(s);
@@ -353,13 +353,9 @@ hsg_status prepare_bond_boxes(hsg_ctx* c) {
   return HSG_OK;
 }
 
-// The bond-box wait flag of the temporally blocked sweeps: queue its copy
-// into the second pinned word (after the work queued so far), and, once the
-// stream has been synchronised, HSG_ETIMEOUT if one of them gave up.
-cudaError_t queue_box_flag(hsg_ctx* c) {
-  if (!c->use_tma) return cudaSuccess;
-  return cudaMemcpyAsync(c->host_e + 1, c->d_ctr + 2, sizeof(double), cudaMemcpyDeviceToHost, c->stream);
-}
+// The bond-box wait flag of the temporally blocked sweeps, which the energy
+// kernel has copied to the second pinned word: once the stream has been
+// synchronised, HSG_ETIMEOUT if one of them gave up.
 hsg_status check_box_waits(hsg_ctx* c) {
   if (!c->use_tma) return HSG_OK;
   unsigned long long flag = 0;
@@ -375,11 +371,23 @@ hsg_status check_box_waits(hsg_ctx* c) {
               "valid");
 }
 
-// E/N into *out_dev, or (logged) into the energy log at the device position.
-hsg_status run_energy(hsg_ctx* c, double* out_dev, bool logged) {
-  unsigned long long* idx = logged ? c->d_ctr + 1 : nullptr;
-  return launch(c, HSG_PROF_ENERGY, 2, "energy kernels",
-                [&] { return hsg::launch_energy(c->spins, c->packed, c->J, c->L, c->partials, out_dev, idx, c->stream); });
+// E/N into the energy log at the device position, or into the pinned result
+// word (with the wait flag into the one beside it).
+hsg_status run_energy(hsg_ctx* c, bool logged) {
+  hsg::EnergyArgs a{};
+  a.S = c->spins;
+  a.packed = c->packed;
+  a.J = c->J;
+  a.L = c->L;
+  a.partials = c->partials;
+  a.ticket = reinterpret_cast<uint32_t*>(c->d_ctr + 3);
+  a.out = logged ? c->elog : c->host_e;
+  a.log_idx = logged ? c->d_ctr + 1 : nullptr;
+  if (!logged && c->use_tma) {
+    a.flag = c->d_ctr + 2;
+    a.flag_out = reinterpret_cast<unsigned long long*>(c->host_e + 1);
+  }
+  return launch(c, HSG_PROF_ENERGY, logged ? 2 : 1, "energy kernel", [&] { return hsg::launch_energy(a, c->stream); });
 }
 
 hsg_status run_advance(hsg_ctx* c) {
@@ -417,7 +425,7 @@ hsg_status enqueue_one_sweep(hsg_ctx* c, const hsg_schedule* s) {
   if (renorm_due && !fuse_renorm)
     if ((st = run_renorm(c)) != HSG_OK) return st;
   if (s->energy_every > 0 && c->sweep % (uint64_t)s->energy_every == 0) {
-    if ((st = run_energy(c, c->elog, true)) != HSG_OK) return st;
+    if ((st = run_energy(c, true)) != HSG_OK) return st;
     c->elog_n += 1;
   }
   return HSG_OK;
@@ -520,7 +528,7 @@ hsg_status run_resident(hsg_ctx* c, const hsg_schedule* s, int n_sweeps) {
     c->sweep += m;
     k += (int)m;
     if (s->energy_every > 0 && c->sweep % (uint64_t)s->energy_every == 0) {
-      if ((st = run_energy(c, c->elog, true)) != HSG_OK) return st;
+      if ((st = run_energy(c, true)) != HSG_OK) return st;
       c->elog_n += 1;
     }
   }
@@ -599,8 +607,7 @@ hsg_status hsg_create_layout(hsg_ctx** out, int L, uint64_t seed, uint32_t sampl
       {reinterpret_cast<void**>(&c->spins), (c->packed ? 3 * sizeof(float) : sizeof(float4)) * (size_t)c->N, "spins"},
       {reinterpret_cast<void**>(&c->J), sizeof(float) * 3 * (size_t)c->N, "couplings"},
       {reinterpret_cast<void**>(&c->partials), sizeof(double) * hsg::energy_partials(L), "energy partials"},
-      {reinterpret_cast<void**>(&c->e_out), sizeof(double), "energy result"},
-      {reinterpret_cast<void**>(&c->d_ctr), 3 * sizeof(unsigned long long), "device counters"},
+      {reinterpret_cast<void**>(&c->d_ctr), kCounters * sizeof(unsigned long long), "device counters"},
   };
   for (auto& a : allocs) {
     e = dev_alloc(a.p, a.bytes, c->stream);
@@ -617,7 +624,7 @@ hsg_status hsg_create_layout(hsg_ctx** out, int L, uint64_t seed, uint32_t sampl
     return st;
   }
   e = cudaMallocHost(&c->host_e, 2 * sizeof(double));
-  if (e == cudaSuccess) e = cudaMemsetAsync(c->d_ctr, 0, 3 * sizeof(unsigned long long), c->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->d_ctr, 0, kCounters * sizeof(unsigned long long), c->stream);
   if (e != cudaSuccess) {
     if (!c->host_e) c->host_e = nullptr;
     st = cuda_fail(nullptr, e, "pinned host slot / counters");
@@ -774,11 +781,9 @@ hsg_status hsg_energy(hsg_ctx* c, double* e_per_spin) {
   if (device_guard.status() != cudaSuccess) return cuda_fail(c, device_guard.status(), "cudaSetDevice");
   if (!e_per_spin) return fail(c, HSG_EINVAL, "e_per_spin is NULL");
   if (!c->have_J) return fail(c, HSG_EINVAL, "couplings not set");
-  hsg_status st = run_energy(c, c->e_out, false);
+  hsg_status st = run_energy(c, false);
   if (st != HSG_OK) return st;
-  cudaError_t e = cudaMemcpyAsync(c->host_e, c->e_out, sizeof(double), cudaMemcpyDeviceToHost, c->stream);
-  if (e == cudaSuccess) e = queue_box_flag(c);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+  const cudaError_t e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "energy readback");
   *e_per_spin = *c->host_e;
   return check_box_waits(c);

@@ -40,7 +40,8 @@ constexpr int ENERGY_THREADS = 256;
 // build on 1064 CTAs, whose registers, allocated per warp, leave room for
 // only six CTAs per SM.
 constexpr int ENERGY_BLOCKS = 760;
-constexpr int FINAL_THREADS = 1024;
+constexpr int FINAL_LANES = 1024;  // of the last sum: its order
+static_assert(ENERGY_BLOCKS <= FINAL_LANES, "one partial per lane");
 
 // Spin initialisation: site i gets the sphere point of Philox counter
 // (i, 0, INIT<<24, 0).  Grid (Lh/32, L/8, 2L): blockIdx.z = 2 z + colour.
@@ -189,76 +190,97 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// Energy, last sum: one block adds the n partials in a fixed order -- as
+// FINAL_LANES lanes that take them in turn, a warp of lanes at a time -- and
+// writes E/N = -(sum)/N to *out, or, with log_idx set, to out[*log_idx] and
+// then advances *log_idx.
+__device__ __forceinline__ void energy_finish(const double* partials, uint32_t n, double inv_n_sites, double* out,
+                                              unsigned long long* log_idx) {
+  __shared__ double part[FINAL_LANES / 32];
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  for (uint32_t w = warp; w < FINAL_LANES / 32; w += ENERGY_THREADS / 32) {
+    double v = 0.0;
+    for (uint32_t k = w * 32u + lane; k < n; k += FINAL_LANES) v += __ldcg(partials + k);
+    v = warp_sum(v);
+    if (lane == 0) part[w] = v;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    const double w = warp_sum(part[lane]);
+    if (lane == 0) {
+      const unsigned long long k = log_idx ? *log_idx : 0ull;
+      out[k] = -w * inv_n_sites;
+      if (log_idx) *log_idx = k + 1;
+    }
+  }
+}
+
 // Energy, first pass.  Every bond joins a colour-0 and a colour-1 site, so
 // sum_bonds J s_i.s_j = sum over colour-0 sites of s_i . h_i with h_i the
 // local field of Eq. 2.  The site term s_i . h_i is formed in FP32 (as in
 // the updates, relative error a few ulp); every sum over sites is FP64.
-// Block b writes partials[b].
-template <bool PACKED>
-__global__ void __launch_bounds__(ENERGY_THREADS) k_energy_partial(const void* __restrict__ S,
-                                                                   const float* __restrict__ J, int L,
-                                                                   double* __restrict__ partials) {
-  const uint32_t Lh = (uint32_t)L / 2;
-  const uint32_t nh = (uint32_t)L * (uint32_t)L * Lh;
+// Block b writes partials[b].  FINISH: the block that finds itself the last to
+// have done so (ticket, zero before and after) also does the last sum into
+// *out, which may be pinned host memory, and copies *flag to *flag_out -- one
+// launch and no copy for a caller that waits for the value.  hsg_energy as
+// its caller sees it, against two launches and a copy, and 64-bit indices with
+// hardware divisions: L = 16 27 -> 16 us, L = 100 26 -> 21, L = 256 99.7 -> 90.5
+// (packed 137 -> 97.5): at L = 256 the pass over 470 MB itself, 5.4 TB/s of it.
+template <bool PACKED, class Off, bool FINISH>
+__global__ void __launch_bounds__(ENERGY_THREADS, 5)
+    k_energy_partial(const void* __restrict__ S, const float* __restrict__ J, uint32_t L, FastDiv by_lh, FastDiv by_L,
+                     double* __restrict__ partials, uint32_t* ticket, double inv_n_sites, double* out,
+                     const unsigned long long* flag, unsigned long long* flag_out) {
+  const uint32_t Lh = L / 2, nh = L * L * Lh;
   const float *jx0 = J, *jx1 = J + nh, *jy0 = J + 2ull * nh, *jy1 = J + 3ull * nh, *jz0 = J + 4ull * nh,
               *jz1 = J + 5ull * nh;
+  const RowLattice<PACKED> lat{static_cast<float4*>(const_cast<void*>(S)),
+                               PACKED ? reinterpret_cast<const float4*>(static_cast<const float*>(S) + 3ull * nh)
+                                      : static_cast<const float4*>(S) + nh,
+                               jx0, jy0, jz0, jx1, jy1, jz1, nh, L, Lh, 0u};
   double acc = 0.0;
-  for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < nh; t += gridDim.x * blockDim.x) {
-    const int xh = (int)(t % Lh);
-    const uint32_t r = t / Lh;
-    const int y = (int)(r % (uint32_t)L), z = (int)(r / (uint32_t)L);
-    const int p = (y + z) & 1;  // colour 0
-    const long long row = (long long)r * Lh;
-    const long long q_xp = row + (p ? wrap_inc(xh, (int)Lh) : xh);
-    const long long q_xm = row + (p ? xh : wrap_dec(xh, (int)Lh));
-    const long long q_yp = ((long long)z * L + wrap_inc(y, L)) * Lh + xh;
-    const long long q_ym = ((long long)z * L + wrap_dec(y, L)) * Lh + xh;
-    const long long q_zp = ((long long)wrap_inc(z, L) * L + y) * Lh + xh;
-    const long long q_zm = ((long long)wrap_dec(z, L) * L + y) * Lh + xh;
-    const float3 h = local_field(spin_get<PACKED>(S, nh, 1, q_xp), spin_get<PACKED>(S, nh, 1, q_xm),
-                                 spin_get<PACKED>(S, nh, 1, q_yp), spin_get<PACKED>(S, nh, 1, q_ym),
-                                 spin_get<PACKED>(S, nh, 1, q_zp), spin_get<PACKED>(S, nh, 1, q_zm), __ldg(jx0 + t),
-                                 __ldg(jx1 + q_xm), __ldg(jy0 + t), __ldg(jy1 + q_ym), __ldg(jz0 + t),
-                                 __ldg(jz1 + q_zm));
-    const float4 s = spin_get<PACKED>(S, nh, 0, t);
-    acc += (double)dot3(make_float3(s.x, s.y, s.z), h);
+  for (uint32_t t = blockIdx.x * ENERGY_THREADS + threadIdx.x; t < nh; t += gridDim.x * ENERGY_THREADS) {
+    const uint32_t r = fast_div(t, by_lh), xh = t - r * Lh, z = fast_div(r, by_L), y = r - z * L;
+    const SiteIndex i = site_index(xh, y, z, L, Lh, 0u);
+    const float3 h = local_field(lat.template other<Off>(i.q_xp), lat.template other<Off>(i.q_xm),
+                                 lat.template other<Off>(i.q_yp), lat.template other<Off>(i.q_ym),
+                                 lat.template other<Off>(i.q_zp), lat.template other<Off>(i.q_zm),
+                                 __ldg(elem<Off>(jx0, t)), __ldg(elem<Off>(jx1, i.q_xm)), __ldg(elem<Off>(jy0, t)),
+                                 __ldg(elem<Off>(jy1, i.q_ym)), __ldg(elem<Off>(jz0, t)), __ldg(elem<Off>(jz1, i.q_zm)));
+    acc += (double)dot3(lat.template old<Off>(t), h);
   }
   __shared__ double warp_part[ENERGY_THREADS / 32];
   acc = warp_sum(acc);
   if ((threadIdx.x & 31) == 0) warp_part[threadIdx.x >> 5] = acc;
   __syncthreads();
+  [[maybe_unused]] __shared__ bool last;
   if (threadIdx.x < 32) {
     double v = threadIdx.x < ENERGY_THREADS / 32 ? warp_part[threadIdx.x] : 0.0;
     v = warp_sum(v);
-    if (threadIdx.x == 0) partials[blockIdx.x] = v;
-  }
-}
-
-// Energy, second pass: one block adds the partials in a fixed order and
-// writes E/N = -(sum)/N to *out, or, with log_idx set, to out[*log_idx]
-// and then advances *log_idx.
-__global__ void __launch_bounds__(FINAL_THREADS) k_energy_final(const double* __restrict__ partials, int n,
-                                                                double inv_n_sites, double* __restrict__ out,
-                                                                unsigned long long* __restrict__ log_idx) {
-  double v = 0.0;
-  for (int k = threadIdx.x; k < n; k += FINAL_THREADS) v += partials[k];
-  __shared__ double warp_part[FINAL_THREADS / 32];
-  v = warp_sum(v);
-  if ((threadIdx.x & 31) == 0) warp_part[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double w = warp_part[threadIdx.x];
-    w = warp_sum(w);
     if (threadIdx.x == 0) {
-      if (log_idx) {
-        const unsigned long long k = *log_idx;
-        out[k] = -w * inv_n_sites;
-        *log_idx = k + 1;
-      } else {
-        *out = -w * inv_n_sites;
+      partials[blockIdx.x] = v;
+      if constexpr (FINISH) {
+        __threadfence();  // the partial before the ticket
+        last = atomicAdd(ticket, 1u) + 1u == gridDim.x;
+        __threadfence();  // the ticket before the others' partials
       }
     }
   }
+  if constexpr (FINISH) {
+    __syncthreads();
+    if (!last) return;
+    energy_finish(partials, gridDim.x, inv_n_sites, out, nullptr);
+    if (threadIdx.x == 0) {
+      *ticket = 0u;
+      if (flag_out) *flag_out = *flag;
+    }
+  }
+}
+
+// Energy, second pass of a logged energy (a launch of its own).
+__global__ void __launch_bounds__(ENERGY_THREADS) k_energy_final(const double* partials, uint32_t n, double inv_n_sites,
+                                                                 double* out, unsigned long long* log_idx) {
+  energy_finish(partials, n, inv_n_sites, out, log_idx);
 }
 
 __global__ void k_set_u64(unsigned long long* p, unsigned long long v) { *p = v; }
@@ -352,16 +374,26 @@ size_t energy_partials(int L) {
   return (size_t)(b < ENERGY_BLOCKS ? b : ENERGY_BLOCKS);
 }
 
-cudaError_t launch_energy(const void* S, bool packed, const float* J, int L, double* partials, double* out,
-                          unsigned long long* log_idx, cudaStream_t s) {
-  const int nb = (int)energy_partials(L);
-  if (packed)
-    k_energy_partial<true><<<nb, ENERGY_THREADS, 0, s>>>(S, J, L, partials);
+template <bool PACKED, class Off>
+void launch_energy_layout(const EnergyArgs& a, cudaStream_t s) {
+  const int nb = (int)energy_partials(a.L);
+  const FastDiv by_lh = make_fastdiv((uint32_t)a.L / 2), by_L = make_fastdiv((uint32_t)a.L);
+  const double inv_n = 1.0 / ((double)a.L * a.L * a.L);
+  if (a.log_idx) {
+    k_energy_partial<PACKED, Off, false><<<nb, ENERGY_THREADS, 0, s>>>(a.S, a.J, (uint32_t)a.L, by_lh, by_L, a.partials,
+                                                                       nullptr, inv_n, nullptr, nullptr, nullptr);
+    k_energy_final<<<1, ENERGY_THREADS, 0, s>>>(a.partials, (uint32_t)nb, inv_n, a.out, a.log_idx);
+  } else {
+    k_energy_partial<PACKED, Off, true><<<nb, ENERGY_THREADS, 0, s>>>(a.S, a.J, (uint32_t)a.L, by_lh, by_L, a.partials,
+                                                                      a.ticket, inv_n, a.out, a.flag, a.flag_out);
+  }
+}
+
+cudaError_t launch_energy(const EnergyArgs& a, cudaStream_t s) {
+  if (a.L > kMaxOff32L)
+    a.packed ? launch_energy_layout<true, unsigned long long>(a, s) : launch_energy_layout<false, unsigned long long>(a, s);
   else
-    k_energy_partial<false><<<nb, ENERGY_THREADS, 0, s>>>(S, J, L, partials);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_energy_final<<<1, FINAL_THREADS, 0, s>>>(partials, nb, 1.0 / ((double)L * L * L), out, log_idx);
+    a.packed ? launch_energy_layout<true, uint32_t>(a, s) : launch_energy_layout<false, uint32_t>(a, s);
   return cudaGetLastError();
 }
 

@@ -123,6 +123,9 @@ struct WaveArgs {
 // with `renorm` set to those half-sweeps followed by launch_renorm.
 cudaError_t launch_or_sweep_wave(const WaveArgs& a, int sm_count, cudaStream_t s);
 
+// The largest L whose arrays' byte offsets fit 32 bits: L^3/2 * 16 < 2^32.
+constexpr int kMaxOff32L = 812;
+
 // Unsigned division by an invariant (make_fastdiv, hsg_device.cuh).
 struct FastDiv {
   uint32_t m, s1, s2;
@@ -190,13 +193,25 @@ cudaError_t launch_gather_spins(const void* S, bool packed, float* dst, int L, c
 cudaError_t launch_gather_sites(const void* S, bool packed, const float* J, int L, const uint32_t* sites, int n,
                                 float* spins, float* bonds, cudaStream_t s);
 
-// Energy: number of FP64 partial sums the first pass writes, and the
-// two-pass E/N into *out (device).  Two launches.
-// With log_idx set, E/N goes to out[*log_idx] and *log_idx is incremented
-// (an energy log whose position lives in device memory).
+// Energy: number of FP64 partial sums the first pass writes, and E/N.  With
+// log_idx set, E/N goes to out[*log_idx] and *log_idx advances (a log whose
+// position lives in device memory): two launches.  Without, E/N goes to *out
+// (device or pinned host memory), and, with flag_out set, *flag to *flag_out:
+// one launch.
 size_t energy_partials(int L);
-cudaError_t launch_energy(const void* S, bool packed, const float* J, int L, double* partials, double* out,
-                          unsigned long long* log_idx, cudaStream_t s);
+struct EnergyArgs {
+  const void* S;
+  bool packed;
+  const float* J;
+  int L;
+  double* partials;  // energy_partials(L) doubles
+  uint32_t* ticket;  // device word, zero before and after
+  double* out;
+  unsigned long long* log_idx;
+  const unsigned long long* flag;
+  unsigned long long* flag_out;
+};
+cudaError_t launch_energy(const EnergyArgs& a, cudaStream_t s);
 
 // Device counters: *p = v, *p += d.  One single-thread launch each.
 cudaError_t launch_set_u64(unsigned long long* p, unsigned long long v, cudaStream_t s);

@@ -52,15 +52,14 @@ __device__ __forceinline__ double warp_sum(double v) {
 // is fp64.  Block b writes partials[b].
 __global__ void __launch_bounds__(kThreads) k_energy_sitemajor_partial(const float* __restrict__ s,
                                                                       const float* __restrict__ J, int L,
-                                                                      double* __restrict__ partials) {
+                                                                      hsg::FastDiv by_L, double* __restrict__ partials) {
   const long long n = (long long)L * L * L;
   const long long plane = (long long)L * L;
   double acc = 0.0;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const int x = (int)(i % L);
-    const long long r = i / L;
-    const int y = (int)(r % L);
-    const int z = (int)(r / L);
+    // i < 1624^3 < 2^32: 32-bit multiply-shift divisions
+    const uint32_t r = hsg::fast_div((uint32_t)i, by_L), zu = hsg::fast_div(r, by_L);
+    const int x = (int)((uint32_t)i - r * (uint32_t)L), y = (int)(r - zu * (uint32_t)L), z = (int)zu;
     const long long ix = x + 1 == L ? i - (L - 1) : i + 1;
     const long long iy = y + 1 == L ? i - (long long)(L - 1) * L : i + L;
     const long long iz = z + 1 == L ? i - (long long)(L - 1) * plane : i + plane;
@@ -166,7 +165,7 @@ extern "C" hsg_status hsg_energy_noalloc(int L, const float* spins, const float*
   const int blocks = (int)(want < kScratchDoubles ? want : kScratchDoubles);
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   double* partials = static_cast<double*>(scratch);
-  k_energy_sitemajor_partial<<<blocks, kThreads, 0, s>>>(spins, J, L, partials);
+  k_energy_sitemajor_partial<<<blocks, kThreads, 0, s>>>(spins, J, L, hsg::make_fastdiv((uint32_t)L), partials);
   e = cudaGetLastError();
   if (e == cudaSuccess) {
     k_energy_sitemajor_final<<<1, kFinalThreads, 0, s>>>(partials, blocks, 1.0 / (double)n, e_out);

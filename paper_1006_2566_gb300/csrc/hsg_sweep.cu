@@ -53,7 +53,6 @@ __device__ __forceinline__ uint32_t site_number(int xh, int p, int y, int z, int
 // L = 128 slower: 28.1-30.1 us against 25.9 us.
 // ---------------------------------------------------------------------------
 constexpr int G_THREADS = 128;
-constexpr int kMaxOff32L = 812;  // L^3/2 * 16 bytes < 2^32
 
 template <int U, int R, int MIN_BLOCKS, class Off, bool PACKED>
 __global__ void __launch_bounds__(G_THREADS, MIN_BLOCKS)
