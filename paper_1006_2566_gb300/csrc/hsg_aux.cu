@@ -283,8 +283,15 @@ __global__ void __launch_bounds__(ENERGY_THREADS) k_energy_final(const double* p
   energy_finish(partials, n, inv_n_sites, out, log_idx);
 }
 
-__global__ void k_set_u64(unsigned long long* p, unsigned long long v) { *p = v; }
-__global__ void k_add_u64(unsigned long long* p, unsigned long long d) { *p += d; }
+// (Launched ahead of the end of the half-sweep before, which reads the counter.)
+__global__ void k_set_u64(unsigned long long* p, unsigned long long v) {
+  wait_for_previous();
+  *p = v;
+}
+__global__ void k_add_u64(unsigned long long* p, unsigned long long d) {
+  wait_for_previous();
+  *p += d;
+}
 
 // Renormalisation of every spin (renorm_spin, hsg_device.cuh); n = N sites,
 // t = c * N/2 + q.
@@ -398,13 +405,11 @@ cudaError_t launch_energy(const EnergyArgs& a, cudaStream_t s) {
 }
 
 cudaError_t launch_set_u64(unsigned long long* p, unsigned long long v, cudaStream_t s) {
-  k_set_u64<<<1, 1, 0, s>>>(p, v);
-  return cudaGetLastError();
+  return launch_overlapped(k_set_u64, dim3(1), dim3(1), s, p, v);
 }
 
 cudaError_t launch_add_u64(unsigned long long* p, unsigned long long d, cudaStream_t s) {
-  k_add_u64<<<1, 1, 0, s>>>(p, d);
-  return cudaGetLastError();
+  return launch_overlapped(k_add_u64, dim3(1), dim3(1), s, p, d);
 }
 
 // Grid-stride over the spins on the CTAs that are resident at once (one

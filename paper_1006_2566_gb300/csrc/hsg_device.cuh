@@ -382,10 +382,18 @@ __device__ __forceinline__ const T* elem(const T* b, uint32_t q) {
   return reinterpret_cast<const T*>(reinterpret_cast<const char*>(b) + (Off)q * (Off)sizeof(T));
 }
 
+// Programmatic dependent launch (launch_overlapped): the CTAs of a launch may
+// start once every CTA of the launch before has called let_next_start or
+// ended, and see its memory after wait_for_previous.
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+
 // One colour of a lattice as update_rows sees it, in either spin layout
 // (float4 per spin, or three component arrays `stride` floats apart: both
-// hand the site code the same values, so the results are the same).
-template <bool PACKED>
+// hand the site code the same values, so the results are the same).  LIVE:
+// the other colour may have been written since this launch began (the launch
+// overlaps the one before), so it is not read through the read-only path.
+template <bool PACKED, bool LIVE = false>
 struct RowLattice {
   float4* own;        // packed: component 0, as are the other colour's
   const float4* oth;
@@ -396,11 +404,17 @@ struct RowLattice {
   __device__ __forceinline__ float4 other(uint32_t q) const {
     if constexpr (PACKED) {
       const float* b = reinterpret_cast<const float*>(oth);
-      return make_float4(__ldg(elem<Off>(b, q)), __ldg(elem<Off>(b + stride, q)), __ldg(elem<Off>(b + 2 * stride, q)),
-                         0.0f);
+      return make_float4(get(elem<Off>(b, q)), get(elem<Off>(b + stride, q)), get(elem<Off>(b + 2 * stride, q)), 0.0f);
     } else {
-      return __ldg(elem<Off>(oth, q));
+      return get(elem<Off>(oth, q));
     }
+  }
+  template <class T>
+  static __device__ __forceinline__ T get(const T* p) {
+    if constexpr (LIVE)
+      return *p;
+    else
+      return __ldg(p);
   }
   template <class Off>
   __device__ __forceinline__ float3 old(uint32_t q) const {
@@ -437,8 +451,8 @@ struct DrawArgs {
 // mod 2, a constant at the call where R is even.  The indices are those of
 // site_index: the column's other-colour spin of row y is the y neighbour of
 // rows y - 1 and y + 1 and one of row y's x neighbours, and is loaded once.
-template <int U, int R, class Off, bool PACKED>
-__device__ __forceinline__ void update_rows(const RowLattice<PACKED>& a, uint32_t xh, uint32_t y0, uint32_t z,
+template <int U, int R, class Off, class Lattice>
+__device__ __forceinline__ void update_rows(const Lattice& a, uint32_t xh, uint32_t y0, uint32_t z,
                                             uint32_t p0, const DrawArgs& d) {
   const uint32_t L = a.L, Lh = a.Lh, plane = L * Lh;
   const uint32_t zo = z * plane, zpo = z + 1 == L ? 0u : zo + plane, zmo = z == 0 ? (L - 1) * plane : zo - plane;

@@ -66,6 +66,23 @@ inline bool key_stream_ok(uint32_t sample, uint32_t replica) { return replica <=
 constexpr const char* kKeyStreamMsg = "replica must be 0 or 1 and sample < 2^31 (the Philox key's stream number "
                                       "2*sample + replica must name each pair once)";
 
+// Launch `kernel` so that its CTAs may start before the launch queued before
+// it on the stream has ended (programmatic dependent launch).  The kernel
+// waits (griddepcontrol.wait) before it touches memory.
+template <class... P, class... A>
+cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // Arguments of one half-sweep (see hsg_device.cuh for the layout).
 struct SweepArgs {
   float4* own;          // spins of the colour being updated

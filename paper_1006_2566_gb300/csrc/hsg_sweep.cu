@@ -54,13 +54,17 @@ __device__ __forceinline__ uint32_t site_number(int xh, int p, int y, int z, int
 // ---------------------------------------------------------------------------
 constexpr int G_THREADS = 128;
 
-template <int U, int R, int MIN_BLOCKS, class Off, bool PACKED>
+template <int U, int R, int MIN_BLOCKS, class Off, bool PACKED, bool OVERLAP>
 __global__ void __launch_bounds__(G_THREADS, MIN_BLOCKS)
-    k_half_sweep_rows(const SweepArgs a, FastDiv by_lh, uint32_t columns) {
+    k_half_sweep_rows(const SweepArgs a, FastDiv by_lh, uint32_t columns, bool early) {
   const uint32_t t = blockIdx.x * G_THREADS + threadIdx.x;
+  if constexpr (OVERLAP) {
+    if (early) let_next_start();
+    wait_for_previous();
+  }
   if (t >= columns) return;
   const uint32_t g = fast_div(t, by_lh), xh = t - g * (uint32_t)a.Lh, y0 = g * R, z = blockIdx.y;
-  const RowLattice<PACKED> lat{a.own,    a.oth,    a.jx_own, a.jy_own,      a.jz_own,       a.jx_oth,
+  const RowLattice<PACKED, OVERLAP> lat{a.own,    a.oth,    a.jx_own, a.jy_own,      a.jz_own,       a.jx_oth,
                                a.jy_oth, a.jz_oth, a.stride, (uint32_t)a.L, (uint32_t)a.Lh, (uint32_t)a.colour};
   DrawArgs d{a.sweep_lo, a.sweep_hi, a.k0, a.k1, a.beta, a.step, a.hits, 0};
   if constexpr (U != U_OR) {
@@ -80,6 +84,9 @@ __global__ void __launch_bounds__(G_THREADS, MIN_BLOCKS)
       update_rows<U, R, Off>(lat, xh, y0, z, 1u, d);
     else
       update_rows<U, R, Off>(lat, xh, y0, z, 0u, d);
+  }
+  if constexpr (OVERLAP) {
+    if (!early) let_next_start();
   }
 }
 
@@ -256,11 +263,39 @@ int slab_zc(int L, unsigned tiles, int sm_count) {
   return zc < 1 ? 1 : (zc > SLAB_ZC_MAX ? SLAB_ZC_MAX : zc);
 }
 
+// How a launch of the rows kernel overlaps the next one on the stream: not
+// at all, letting its CTAs start when this launch's last CTAs have started
+// (EARLY), or as each CTA is done (LATE).  Small launches are mostly start-up:
+// up to one wave of CTAs LATE takes 0.3-1 us off each (a waiting CTA of the
+// next launch would take the place of a working one; with EARLY L = 66 was
+// slower, 2.55 against 2.05 us).  Beyond, the over-relaxation is better left
+// alone (its reads then also go through the read-only path), and the longer
+// updates gain a little from EARLY while they fill a few waves.  In graphs, us,
+// none / LATE / EARLY:
+//   OR         L = 40 1.54 / 1.23 / 1.29, 66 2.31 / 2.05 / 2.55, 76 2.58 / 2.76 / 2.82, 128 6.66 / 9.23 / 8.65
+//   heat-bath  L = 40 2.04 / 1.03 / 2.05, 66 3.07 / 3.07 / 3.99, 80 5.10 / 4.30 / 5.06, 104 8.09 / 8.11 / 7.20,
+//              120 11.1 / 11.3 / 10.3, 128 12.3 / 12.3 / 12.1
+//   4 hits     L = 40 3.06 / 2.04 / 2.06, 80 7.12 / 6.19 / 6.18, 110 15.3 / 14.8 / 14.4, 128 20.6 / 20.5 / 20.4
+enum Overlap { NONE, EARLY, LATE };
+template <int U>
+Overlap overlap(int L) {
+  if (U == U_OR) return L <= 72 ? LATE : NONE;
+  return L <= 90 ? LATE : L <= 126 ? EARLY : NONE;
+}
+
 template <int U, int R, int MIN_BLOCKS, class Off, bool PACKED>
-void launch_rows(const SweepArgs& a, cudaStream_t s) {
+cudaError_t launch_rows(const SweepArgs& a, cudaStream_t s) {
   const uint32_t columns = (uint32_t)a.Lh * (uint32_t)(a.L / R);
-  k_half_sweep_rows<U, R, MIN_BLOCKS, Off, PACKED>
-      <<<dim3(cdiv(columns, G_THREADS), (unsigned)a.L), G_THREADS, 0, s>>>(a, make_fastdiv((uint32_t)a.Lh), columns);
+  const FastDiv by_lh = make_fastdiv((uint32_t)a.Lh);
+  const dim3 grid(cdiv(columns, G_THREADS), (unsigned)a.L);
+  if constexpr (sizeof(Off) == 4 && R < 4) {
+    const Overlap o = overlap<U>(a.L);
+    if (o != NONE)
+      return launch_overlapped(k_half_sweep_rows<U, R, MIN_BLOCKS, Off, PACKED, true>, grid, dim3(G_THREADS), s, a, by_lh,
+                               columns, o == EARLY);
+  }
+  k_half_sweep_rows<U, R, MIN_BLOCKS, Off, PACKED, false><<<grid, G_THREADS, 0, s>>>(a, by_lh, columns, false);
+  return cudaGetLastError();
 }
 
 // Rows per thread and the register bound, by the measurements above and (MB:
@@ -274,26 +309,25 @@ template <int U, bool PACKED>
 cudaError_t launch_global(const SweepArgs& a, cudaStream_t s) {
   constexpr bool MET = U != U_OR && U != U_HB;
   if (a.L > kMaxOff32L) {
-    launch_rows<U, 1, MET ? 1 : 12, unsigned long long, PACKED>(a, s);
+    return launch_rows<U, 1, MET ? 1 : 12, unsigned long long, PACKED>(a, s);
   } else if constexpr (U == U_OR) {
     if (PACKED && a.L >= 160)
-      launch_rows<U, 2, 10, uint32_t, PACKED>(a, s);
+      return launch_rows<U, 2, 10, uint32_t, PACKED>(a, s);
     else
-      launch_rows<U, 1, 12, uint32_t, PACKED>(a, s);
+      return launch_rows<U, 1, 12, uint32_t, PACKED>(a, s);
   } else if constexpr (U == U_HB) {
     if (a.L < 96)
-      launch_rows<U, 1, 12, uint32_t, PACKED>(a, s);
+      return launch_rows<U, 1, 12, uint32_t, PACKED>(a, s);
     else
-      launch_rows<U, 2, PACKED ? 10 : 16, uint32_t, PACKED>(a, s);
+      return launch_rows<U, 2, PACKED ? 10 : 16, uint32_t, PACKED>(a, s);
   } else {
     if (!PACKED && a.L >= 160 && a.L % 4 == 0)
-      launch_rows<U, 4, 1, uint32_t, PACKED>(a, s);
+      return launch_rows<U, 4, 1, uint32_t, PACKED>(a, s);
     else if (a.L >= (PACKED ? 160 : 96))
-      launch_rows<U, 2, 1, uint32_t, PACKED>(a, s);
+      return launch_rows<U, 2, 1, uint32_t, PACKED>(a, s);
     else
-      launch_rows<U, 1, 1, uint32_t, PACKED>(a, s);
+      return launch_rows<U, 1, 1, uint32_t, PACKED>(a, s);
   }
-  return cudaGetLastError();
 }
 
 template <int U>

@@ -63,3 +63,25 @@ def test_either_side_of_the_32_bit_offsets(hsg, L):
             outs.append(hsg.hsg_get_sites(lat.ctx, sites, want_bonds=False)[0])
     assert np.array_equal(outs[0], outs[1])
     assert np.array_equal(outs[0], outs[2])
+
+
+# either side of where launches overlap the next one, and how: over-relaxation
+# up to 72, the other updates up to 90 and up to 126
+@pytest.mark.parametrize("L", [34, 72, 74, 90, 92, 126, 128])
+@pytest.mark.parametrize("use_stream", [True, False])
+def test_overlapping_launches_equal_the_slab_kernel(hsg, L, use_stream):
+    for kw in (dict(kind=hsg.HSG_HEATBATH, n_or=2), dict(kind=hsg.HSG_METROPOLIS, hits=2, proposal=1, n_or=1),
+               dict(kind=hsg.HSG_METROPOLIS_OR, hits=1, n_or=0)):
+        outs = []
+        for layout, kernel in ((0, hsg.HSG_KERNEL_SLAB), (0, hsg.HSG_KERNEL_GLOBAL), (1, hsg.HSG_KERNEL_GLOBAL)):
+            stream = torch.cuda.Stream() if use_stream else None
+            with hsg.Lattice(L, 31, stream=stream, layout=layout) as lat:
+                lat.generate_couplings()
+                sched = hsg.schedule(T=0.7, kernel=kernel, renorm_every=3, energy_every=2, **kw)
+                lat.sweep(sched, 1)
+                lat.sweep_count = 6
+                lat.sweep(sched, 13)
+                lat.half_sweep(sched, hsg.HSG_HEATBATH, 1)
+                outs.append((lat.spins(), lat.energy_log(), lat.energy()))
+        for o in outs[1:]:
+            assert all(np.array_equal(a, b) for a, b in zip(o, outs[0]))
