@@ -28,7 +28,9 @@
  *     then restores the caller's, so objects of several devices can be used
  *     from one thread in any order.
  *   - Device memory is owned by the context (stream-ordered allocations),
- *     released by hsg_destroy.  Caller arrays are copied, never retained.
+ *     released by hsg_destroy.  The library keeps up to 512 MB of released
+ *     memory per device for its next contexts.  Caller arrays are copied,
+ *     never retained.
  *   - hsg_last_error() gives a message for the last failure.
  *   - A context is not thread-safe; distinct contexts are independent.
  */

@@ -108,7 +108,7 @@ hsg_status cuda_fail(hsg_ctx* c, cudaError_t e, const char* what) {
 cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t s) {
   *p = nullptr;
   if (g_fail_alloc_countdown > 0 && --g_fail_alloc_countdown == 0) return cudaErrorMemoryAllocation;
-  return cudaMallocAsync(p, bytes, s);
+  return hsg::device_alloc(p, bytes, s);
 }
 
 void dev_free(void* p, cudaStream_t s) {
@@ -197,7 +197,7 @@ void release(hsg_ctx* c) {
   dev_free(c->d_ctr, s);
   cudaStreamSynchronize(s);
   if (c->gexec) cudaGraphExecDestroy(c->gexec);
-  if (c->host_e) cudaFreeHost(c->host_e);
+  hsg::give_result_words(c->host_e);
   for (auto& r : c->recs) {
     cudaEventDestroy(r.start);
     if (r.stop) cudaEventDestroy(r.stop);
@@ -623,10 +623,9 @@ hsg_status hsg_create_layout(hsg_ctx** out, int L, uint64_t seed, uint32_t sampl
     release(c);
     return st;
   }
-  e = cudaMallocHost(&c->host_e, 2 * sizeof(double));
+  e = hsg::take_result_words(&c->host_e);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_ctr, 0, kCounters * sizeof(unsigned long long), c->stream);
   if (e != cudaSuccess) {
-    if (!c->host_e) c->host_e = nullptr;
     st = cuda_fail(nullptr, e, "pinned host slot / counters");
     release(c);
     return st;

@@ -237,6 +237,12 @@ cudaError_t launch_add_u64(unsigned long long* p, unsigned long long d, cudaStre
 // FP64 renormalisation of the n = N spins.  One launch.
 cudaError_t launch_renorm(void* S, bool packed, long long n, int sm_count, cudaStream_t s);
 
+// Stream-ordered device memory from the library's pool on the current device
+// (hsg_memory.cu; freed with cudaFreeAsync), and four pinned words for results.
+cudaError_t device_alloc(void** p, size_t bytes, cudaStream_t s);
+cudaError_t take_result_words(double** p);
+void give_result_words(double* p);
+
 // Record the calling thread's last error message (read by hsg_last_error(NULL)).
 void set_thread_error(const std::string& msg);
 

@@ -1,0 +1,150 @@
+// hsg_memory.cu -- where contexts take their device memory and pinned result
+// words from (host code).
+//
+// A program that solves one sample after another creates and destroys a
+// context per sample.  From the default memory pool, which gives everything
+// back to the operating system at the next synchronisation, and with
+// cudaMallocHost for two result words, that cost more than the sweeps of a
+// small lattice: creation 255 us and destruction 277 us at L = 48, 421 and 890 us
+// at L = 192.  So each device has one memory pool of the library's own, which keeps
+// up to kKeepBytes of freed memory for the next context (more is given back at the
+// next synchronisation, all of it before an allocation may fail), and the
+// result words are cut from pinned pages, given back once none of a page is
+// in use (the first page stays).  Both are kept per CUDA context (by its id, so that
+// nothing outlives a device reset) under one lock; stream order is CUDA's.
+#include <cstdint>
+#include <mutex>
+
+#include "hsg_internal.h"
+
+namespace hsg {
+namespace {
+
+constexpr unsigned long long kKeepBytes = 512ull << 20;  // an L = 192 context and its uploads: 490 MB
+constexpr int kWordBytes = 32, kPageBytes = 4096, kSlots = kPageBytes / kWordBytes;
+constexpr int kPages = 64;
+
+struct Page {
+  char* base;
+  uint64_t used[kSlots / 64];
+};
+struct Device {
+  unsigned long long ctx_id;
+  cudaMemPool_t pool;
+  Page pages[kPages];
+};
+
+std::mutex g_mu;
+Device g_devices[kMaxDevices];
+int g_n = 0;
+
+using CtxGetCurrentFn = CUresult (*)(CUcontext*);
+using CtxGetIdFn = CUresult (*)(CUcontext, unsigned long long*);
+
+template <class F>
+F driver_function(const char* name) {
+  void* p = nullptr;
+  cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+  if (cudaGetDriverEntryPointByVersion(name, &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+      q != cudaDriverEntryPointSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  return reinterpret_cast<F>(p);
+}
+
+// The current CUDA context's record (g_mu held), or nullptr: no such entry
+// points, or more contexts over the process's life than there are records.
+Device* current_device() {
+  static const CtxGetCurrentFn get_current = driver_function<CtxGetCurrentFn>("cuCtxGetCurrent");
+  static const CtxGetIdFn get_id = driver_function<CtxGetIdFn>("cuCtxGetId");
+  if (!get_current || !get_id || cudaFree(nullptr) != cudaSuccess) return nullptr;
+  CUcontext ctx = nullptr;
+  unsigned long long id = 0;
+  if (get_current(&ctx) != CUDA_SUCCESS || !ctx || get_id(ctx, &id) != CUDA_SUCCESS) return nullptr;
+  for (int i = 0; i < g_n; ++i)
+    if (g_devices[i].ctx_id == id) return &g_devices[i];
+  int dev = 0;
+  if (g_n == kMaxDevices || cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+  cudaMemPoolProps props = {};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = dev;
+  Device d = {};
+  d.ctx_id = id;
+  unsigned long long keep = kKeepBytes;
+  if (cudaMemPoolCreate(&d.pool, &props) != cudaSuccess ||
+      cudaMemPoolSetAttribute(d.pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+    cudaGetLastError();
+    if (d.pool) cudaMemPoolDestroy(d.pool);
+    return nullptr;
+  }
+  g_devices[g_n] = d;
+  return &g_devices[g_n++];
+}
+
+}  // namespace
+
+cudaError_t device_alloc(void** p, size_t bytes, cudaStream_t s) {
+  cudaMemPool_t pool = nullptr;
+  {
+    std::lock_guard<std::mutex> lock(g_mu);
+    if (Device* d = current_device()) pool = d->pool;
+  }
+  if (!pool) return cudaMallocAsync(p, bytes, s);
+  cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    cudaMemPoolTrimTo(pool, 0);
+    e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+  }
+  return e;
+}
+
+cudaError_t take_result_words(double** p) {
+  *p = nullptr;
+  std::lock_guard<std::mutex> lock(g_mu);
+  if (Device* d = current_device()) {
+    for (Page& page : d->pages) {
+      if (!page.base) {
+        const cudaError_t e = cudaMallocHost(reinterpret_cast<void**>(&page.base), kPageBytes);
+        if (e != cudaSuccess) {
+          page.base = nullptr;
+          return e;
+        }
+      }
+      for (int k = 0; k < kSlots; ++k) {
+        uint64_t& word = page.used[k / 64];
+        const uint64_t bit = 1ull << (k % 64);
+        if (word & bit) continue;
+        word |= bit;
+        *p = reinterpret_cast<double*>(page.base + k * kWordBytes);
+        return cudaSuccess;
+      }
+    }
+  }
+  return cudaMallocHost(reinterpret_cast<void**>(p), kWordBytes);
+}
+
+void give_result_words(double* p) {
+  if (!p) return;
+  const char* c = reinterpret_cast<const char*>(p);
+  std::lock_guard<std::mutex> lock(g_mu);
+  for (int i = 0; i < g_n; ++i)
+    for (int j = 0; j < kPages; ++j) {
+      Page& page = g_devices[i].pages[j];
+      if (!page.base || c < page.base || c >= page.base + kPageBytes) continue;
+      const int k = (int)((c - page.base) / kWordBytes);
+      page.used[k / 64] &= ~(1ull << (k % 64));
+      bool any = false;
+      for (uint64_t w : page.used) any |= w != 0;
+      if (!any && j > 0) {
+        cudaFreeHost(page.base);
+        page.base = nullptr;
+      }
+      return;
+    }
+  cudaFreeHost(p);
+}
+
+}  // namespace hsg

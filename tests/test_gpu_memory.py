@@ -1,0 +1,85 @@
+"""Contexts come and go: memory and result words taken again by the next ones
+(needs a CUDA GPU)."""
+import threading
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def hsg():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1006_2566_gb300 import build
+
+    build.build()
+    from paper_1006_2566_gb300 import hsg as h
+
+    return h
+
+
+def solve(hsg, L, seed, stream):
+    with hsg.Lattice(L, seed, stream=stream) as lat:
+        lat.generate_couplings()
+        lat.sweep(hsg.schedule(kind=hsg.HSG_METROPOLIS, hits=2, proposal=1, T=0.5, n_or=1, energy_every=2), 4)
+        return lat.energy(), lat.energy_log(), lat.spins()
+
+
+def same(a, b):
+    return a[0] == b[0] and np.array_equal(a[1], b[1]) and np.array_equal(a[2], b[2])
+
+
+def test_solves_in_many_threads_and_streams(hsg):
+    """Reused memory holds nothing of the context before: each solve gives
+    what it gave alone, whatever runs beside it."""
+    jobs = [(L, seed) for seed in range(4) for L in (8, 34, 66)]
+    want = {j: solve(hsg, *j, None) for j in jobs}
+    bad = []
+
+    def work(k):
+        stream = torch.cuda.Stream()
+        for j in jobs[k:] + jobs[:k]:
+            if not same(solve(hsg, *j, stream), want[j]):
+                bad.append(j)
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(6)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad
+
+
+def test_more_contexts_than_a_page_of_result_words(hsg):
+    lats = [hsg.Lattice(4, seed) for seed in range(300)]
+    for lat in lats:
+        lat.generate_couplings()
+    e = [lat.energy() for lat in lats]
+    for lat in lats[::2]:
+        lat.close()
+    again = [hsg.Lattice(4, seed) for seed in range(0, 300, 2)]
+    for lat in again:
+        lat.generate_couplings()
+    assert [lat.energy() for lat in again] == e[::2]
+    assert [lat.energy() for lat in lats[1::2]] == e[1::2]
+    for lat in lats + again:
+        lat.close()
+
+
+def test_released_memory_is_kept_within_its_bound(hsg):
+    def used():
+        torch.cuda.synchronize()
+        free, total = torch.cuda.mem_get_info()
+        return total - free
+
+    with hsg.Lattice(16, 1) as lat:
+        lat.generate_couplings()
+    before = used()
+    for _ in range(3):
+        lats = [hsg.Lattice(256, k) for k in range(4)]  # 470 MB each
+        for lat in lats:
+            lat.close()
+    assert used() - before <= (512 + 64) << 20
