@@ -298,35 +298,50 @@ cudaError_t launch_rows(const SweepArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// Rows per thread and the register bound, by the measurements above and (MB:
-// 4-hit Metropolis; R rows at B resident CTAs of 128):
-//   heat-bath      L = 96 6.2 (R 1) 6.1 (R 2), 128 13.2 / 12.3, 256 97.4 / 95.8 us
-//   MB             L = 128 21.4 / 20.5 / 22.4 (R 4), 192 74.5 / 71.9 / 69.1, 256 171 / 161 / 154 us
-//   OR             L = 128 6.66 / 7.11, 256 83.5 / 89.4 us
-//   packed OR      L = 130 7.7 / 11.2, 192 38.9 / 37.5, 256 89.3 / 84.3 us; heat-bath 130 15.3 / 13.9, 256 105 / 94.1;
-//   packed MB      L = 128 22.2 / 22.8, 192 73.0 / 72.0, 256 170 / 165 us
+// Rows per thread (R) and the register bound (B resident CTAs of 128), by
+// kind, size and hits.  Registers, spills and the neighbour rows that a
+// thread keeps weigh differently for each kind's code; from about L = 150 the
+// half-sweeps of few hits stream from HBM and want loads in flight (B 10 to
+// 14), the ones of many hits registers.  us per half-sweep at L = 128 / 160 or
+// 156 / 192 / 256 (one site per thread, 64-bit addresses, in brackets):
+//   OR         R 1, B 12   6.7 / - / 36.4 / 83.5          [7.9 / - / 37.9 / 85.0]
+//   heat-bath  R 2, B 16   12.3 / - / 43.2 / 95.8 (R 1, B 12 13.2 / - / 43.0 / 97.4)
+//   sphere     R 2, B 10   1 hit 9.6 / 24.7 / 40.9 / 92 [10.2 / 30.7 / 46.9 / 101], 4 hits 18.4 / 35.1 / 58.9 / 133
+//                          [18.4 / 47 / 69 / 153]; R 1, B 12 1 hit 10.3 / 27.8 / 46.7 / 106
+//   ball       R 1, B 12   1 hit 10.3 / 25.5 / 42.2 / 96 [10.3 / 29.7 / 44.6 / 97] (R 4 10.9 / 25.7 / 47.1 / 102);
+//              R 4         4 hits 22.5 / 42.3 / 68.9 / 155 [20.5 / 50.2 / 71.5 / 161] (R 1, B 12 21.5 / 42.5 / 71.0 / 164)
+//   sphere+OR  R 1, B 14   1 hit 10.4 / 25.0 / 41.5 / 94 [10.3 / 27.0 / 41.8 / 91];
+//              R 2, B 8    4 hits 18.5 / 36.9 / 60.7 / 139 [18.5 / 45.1 / 65.1 / 143]
+//   ball+OR    R 2         1 hit 10.3 / 24.0 / 40.3 / 92 [10.3 / 33.1 / 50.0 / 107], 4 hits 21.5 / 40.3 / 67.7 / 155
+//                          [20.6 / 52.3 / 76.6 / 169]
+//   packed OR  L = 130 7.7 (R 1) 11.2 (R 2), 192 38.9 / 37.5, 256 89.3 / 84.3; packed heat-bath 130 15.3 / 13.9, 256 105 / 94;
+//   packed ball, 4 hits: 128 22.2 / 22.8, 192 73.0 / 72.0, 256 170 / 165
 template <int U, bool PACKED>
 cudaError_t launch_global(const SweepArgs& a, cudaStream_t s) {
   constexpr bool MET = U != U_OR && U != U_HB;
-  if (a.L > kMaxOff32L) {
-    return launch_rows<U, 1, MET ? 1 : 12, unsigned long long, PACKED>(a, s);
-  } else if constexpr (U == U_OR) {
-    if (PACKED && a.L >= 160)
-      return launch_rows<U, 2, 10, uint32_t, PACKED>(a, s);
-    else
-      return launch_rows<U, 1, 12, uint32_t, PACKED>(a, s);
+  if (a.L > kMaxOff32L) return launch_rows<U, 1, MET ? 1 : 12, unsigned long long, PACKED>(a, s);
+  if constexpr (U == U_OR) {
+    if (PACKED && a.L >= 160) return launch_rows<U, 2, 10, uint32_t, PACKED>(a, s);
+    return launch_rows<U, 1, 12, uint32_t, PACKED>(a, s);
   } else if constexpr (U == U_HB) {
-    if (a.L < 96)
-      return launch_rows<U, 1, 12, uint32_t, PACKED>(a, s);
-    else
-      return launch_rows<U, 2, PACKED ? 10 : 16, uint32_t, PACKED>(a, s);
+    if (a.L < 96) return launch_rows<U, 1, 12, uint32_t, PACKED>(a, s);
+    return launch_rows<U, 2, PACKED ? 10 : 16, uint32_t, PACKED>(a, s);
+  } else if constexpr (PACKED) {
+    if (a.L >= 160) return launch_rows<U, 2, 1, uint32_t, PACKED>(a, s);
+    return launch_rows<U, 1, 1, uint32_t, PACKED>(a, s);
   } else {
-    if (!PACKED && a.L >= 160 && a.L % 4 == 0)
-      return launch_rows<U, 4, 1, uint32_t, PACKED>(a, s);
-    else if (a.L >= (PACKED ? 160 : 96))
+    if (a.L < 96) return launch_rows<U, 1, 1, uint32_t, PACKED>(a, s);
+    if constexpr (U == U_MET_SPHERE) {
+      return launch_rows<U, 2, 10, uint32_t, PACKED>(a, s);
+    } else if constexpr (U == U_MET_BALL) {
+      if (a.hits > 1 && a.L >= 152 && a.L % 4 == 0) return launch_rows<U, 4, 1, uint32_t, PACKED>(a, s);
+      return launch_rows<U, 1, 12, uint32_t, PACKED>(a, s);
+    } else if constexpr (U == U_MET_OR_SPHERE) {
+      if (a.hits == 1) return launch_rows<U, 1, 14, uint32_t, PACKED>(a, s);
+      return launch_rows<U, 2, 8, uint32_t, PACKED>(a, s);
+    } else {
       return launch_rows<U, 2, 1, uint32_t, PACKED>(a, s);
-    else
-      return launch_rows<U, 1, 1, uint32_t, PACKED>(a, s);
+    }
   }
 }
 
