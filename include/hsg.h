@@ -331,11 +331,13 @@ hsg_status hsg_philox(uint64_t seed, uint32_t sample, uint32_t replica, uint32_t
 
 /*
  * Pools: many independent lattices (disorder samples, replicas, requests) of
- * uneven L in one device arena, swept together.  Every half-sweep of a pool
- * is ONE persistent kernel over a work list of (lattice, site-range) tiles
- * covering all admitted lattices, and a sweep's launches are captured once
- * in a CUDA graph and replayed (on a non-default stream) while lattices come
- * and go.  Each lattice keeps its own side, Philox key, temperature and
+ * uneven L in one device arena, swept together.  Every half-sweep of the
+ * small lattices is ONE persistent kernel over a work list of (lattice,
+ * site-range) tiles, and a sweep's launches are captured once in a CUDA graph
+ * and replayed (on a non-default stream) while lattices come and go; lattices of
+ * L >= 32 are swept in batches that fit in L2, one launch per half-sweep of a
+ * batch, partly on streams of the pool's own between the work queued before and
+ * after on the pool's stream.  Each lattice keeps its own side, Philox key, temperature and
  * sweep counter, and is updated by the same device code with the same
  * random numbers as a single-lattice context: its spins are bit-identical
  * to those of the same lattice swept alone with hsg_sweep.
@@ -398,7 +400,7 @@ hsg_status hsg_pool_get_sweep(hsg_pool* pool, int slot, uint64_t* sweep);
 /* Arena bytes in use, the budget, and the number of admitted lattices. */
 hsg_status hsg_pool_usage(hsg_pool* pool, uint64_t* bytes_used, uint64_t* bytes_budget, int* active);
 
-/* Launch configuration of the pool kernels: threads per CTA (64, 128 or
+/* Launch configuration of the pool's persistent kernels: threads per CTA (64, 128 or
  * 256), sites per tile (a multiple of threads, <= 8192), CTAs per SM of the
  * persistent grid (1..32), and Metropolis hits per pass (0: all of a
  * colour's hits in one pass; h > 0: the hits in passes of at most h, each a

@@ -19,7 +19,7 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 OBJDIR = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libhsg.so")
-SOURCES = ["hsg_sweep.cu", "hsg_aux.cu", "hsg_api.cu", "hsg_noalloc.cu", "hsg_pool.cu", "hsg_wave.cu", "hsg_resident.cu", "hsg_memory.cu"]
+SOURCES = ["hsg_sweep.cu", "hsg_aux.cu", "hsg_api.cu", "hsg_noalloc.cu", "hsg_pool.cu", "hsg_wave.cu", "hsg_resident.cu", "hsg_memory.cu", "hsg_batch.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # -fmad=false: every fused multiply-add is an explicit fmaf, so kernels that
 # share the site code agree bit for bit.  -ftz=true: fp32 subnormals flush to

@@ -171,6 +171,30 @@ constexpr int kResidentMaxL = 32;
 bool resident_takes(int upd, int L, int hits);
 cudaError_t launch_resident(int upd, const ResidentArgs& a, cudaStream_t s);
 
+// A batch of pool lattices swept by one launch per half-sweep (hsg_batch.cu),
+// handed over as kernel parameters.
+struct BatchLattice {
+  float4* spins;   // S[2][nh]
+  const float* J;  // J[3][2][nh]
+  unsigned long long sweep;
+  uint32_t nh, L, Lh;
+  uint32_t k0, k1;
+  float beta;
+  uint32_t cta0;             // first CTA (set by the launcher)
+  FastDiv by_lh, by_groups;  // by_groups: set by the launcher
+};
+constexpr int kBatchMax = 24;   // 2 KB of parameters: 3 us of host time per launch (40: 4 us)
+constexpr int kBatchMinL = 32;  // smaller lattices stay with the pool's persistent kernels
+struct BatchArgs {
+  int n;
+  BatchLattice lat[kBatchMax];
+};
+// Half-sweep `upd` of colour `colour` of every lattice of the batch, hits
+// hit0 .. hit0 + hits - 1, at its sweep counter plus sweep_add.
+cudaError_t launch_batch_half(int upd, BatchArgs& a, uint32_t colour, int hits, int hit0, float step, uint32_t sweep_add,
+                              cudaStream_t s);
+cudaError_t launch_batch_renorm(const BatchArgs& a, cudaStream_t s);
+
 // Halo-padded copy of the colour-split bonds, read by the sweep's tensor
 // boxes: Jp[a][z][yp][xp] with a = 2d + c, yp = y + 2 in [0, L + 4) and
 // xp = xh + 2 in [0, W), W = roundup(L/2 + 4, 4), holding the bond of

@@ -11,9 +11,12 @@
 // and replayed while lattices are admitted and retired: only the work list
 // and the slot table change, in device memory, between replays.
 //
-// Every site is updated by half_sweep_site, the same device function as the
-// single-lattice kernel, with the same key and counters: a lattice swept in
-// a pool is bit-identical to the same lattice swept alone.
+// From 2^17 sites of lattices of L >= 32 on, those lattices are swept in
+// batches instead (hsg_batch.cu), beside the persistent kernels of the others.
+//
+// Every site is updated by half_sweep_site or update_rows, the same device code as
+// the single-lattice kernels, with the same key and counters: a lattice swept
+// in a pool is bit-identical to the same lattice swept alone.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -54,6 +57,11 @@ __device__ __forceinline__ void decode_site(const PoolDesc* d, uint32_t q, uint3
 
 constexpr size_t kAlign = 256;
 
+// Batches (hsg_batch.cu): the bytes of lattices in one, and the sites of
+// lattices of L >= kBatchMinL from which they are worth their launches beside
+// the persistent kernels' (one L = 40 lattice among small ones is not).
+constexpr uint64_t kBatchBytes = 32ull << 20, kBatchMinSites = 1ull << 17;
+
 inline unsigned cdiv_u(unsigned long long a, unsigned long long b) { return (unsigned)((a + b - 1) / b); }
 
 // At most 64 registers (four CTAs of 256 threads per SM): the over-relaxation
@@ -91,13 +99,14 @@ __global__ void __launch_bounds__(256, 4) k_pool_half_sweep(const PoolDesc* __re
   }
 }
 
-// Counter advance of every active slot, after the last half-sweep of a sweep.
-__global__ void k_pool_advance(PoolDesc* __restrict__ desc, int n) {
+// Counter advance of every active slot by `sweeps`, after the last half-sweep
+// of a sweep (or of all of them).
+__global__ void k_pool_advance(PoolDesc* __restrict__ desc, int n, uint32_t sweeps) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     if (!desc[i].active) continue;
-    const uint32_t lo = desc[i].sweep_lo + 1u;
+    const uint32_t lo = desc[i].sweep_lo + sweeps;
     desc[i].sweep_lo = lo;
-    if (lo == 0u) desc[i].sweep_hi += 1u;
+    if (lo < sweeps) desc[i].sweep_hi += 1u;
   }
 }
 
@@ -233,8 +242,17 @@ struct hsg_pool {
   uint2* d_tiles = nullptr;
   uint2* h_tiles = nullptr;  // pinned, 2 x tiles_cap
   size_t tiles_cap = 0;
+  // Tiles that the persistent sweep kernels take (word 0) and all of them
+  // (word 1): the list holds the lattices of the batches last.
   uint32_t* d_ntiles = nullptr;
-  uint32_t* h_ntiles = nullptr;  // pinned, 2
+  uint32_t* h_ntiles = nullptr;  // pinned, 2 x 2
+  // Sweeping of the large lattices in batches (hsg_batch.cu): whether the
+  // admitted lattices ask for it (set with the tables), whether others are left
+  // to the persistent kernels, and the streams beside the pool's own, made on first use.
+  bool batched = false, unbatched_left = true;
+  static constexpr int kSide = 2;
+  cudaStream_t side[kSide] = {nullptr, nullptr};
+  cudaEvent_t fork_ev = nullptr, join_ev[kSide] = {nullptr, nullptr};
   cudaEvent_t up_ev[2] = {nullptr, nullptr};
   bool up_rec[2] = {false, false};
   int up_buf = 0;
@@ -364,38 +382,47 @@ hsg_status sync_tables(hsg_pool* p) {
   }
   PoolDesc* h_desc = p->h_desc + (size_t)b * p->max_slots;
   uint2* h_tiles = p->h_tiles + (size_t)b * p->tiles_cap;
-  uint32_t* h_ntiles = p->h_ntiles + b;
+  uint32_t* h_ntiles = p->h_ntiles + 2 * b;
+  uint64_t large_sites = 0;
+  for (const Slot& s : p->slots)
+    if (s.active && s.L >= hsg::kBatchMinL) large_sites += (uint64_t)s.L * s.L * s.L;
+  p->batched = large_sites >= kBatchMinSites;
   uint32_t nt = 0;
-  for (int i = 0; i < p->max_slots; ++i) {
-    const Slot& s = p->slots[i];
-    PoolDesc& d = h_desc[i];
-    memset(&d, 0, sizeof(d));
-    if (!s.active) continue;
-    const uint64_t n = (uint64_t)s.L * s.L * s.L;
-    d.L = (uint32_t)s.L;
-    d.Lh = (uint32_t)s.L / 2;
-    d.nh = (uint32_t)(n / 2);
-    d.plane = d.L * d.Lh;
-    d.k0 = (uint32_t)(s.seed & 0xFFFFFFFFu);
-    d.k1 = (uint32_t)(s.seed >> 32) ^ ((2u * s.sample + s.replica) * 0x9E3779B9u);
-    d.sweep_lo = (uint32_t)(s.sweep & 0xFFFFFFFFu);
-    d.sweep_hi = (uint32_t)(s.sweep >> 32);
-    d.beta = std::isinf(s.T) ? 0.0f : (float)(1.0 / s.T);
-    d.active = 1;
-    d.spin_off = s.off / sizeof(float4);
-    d.j_off = (s.off + sizeof(float4) * n) / sizeof(float);
-    d.by_plane = hsg::make_fastdiv(d.plane);
-    d.by_lh = hsg::make_fastdiv(d.Lh);
-    d.tile_begin = nt;
-    for (uint32_t q0 = 0; q0 < d.nh; q0 += (uint32_t)p->tile_sites) h_tiles[nt++] = make_uint2((uint32_t)i, q0);
-    d.tile_count = nt - d.tile_begin;
+  // The slots of the persistent kernels first, those of the batches after them.
+  for (int pass = 0; pass < 2; ++pass) {
+    for (int i = 0; i < p->max_slots; ++i) {
+      const Slot& s = p->slots[i];
+      PoolDesc& d = h_desc[i];
+      if (s.active && (p->batched && s.L >= hsg::kBatchMinL) != (pass == 1)) continue;
+      memset(&d, 0, sizeof(d));
+      if (!s.active) continue;
+      const uint64_t n = (uint64_t)s.L * s.L * s.L;
+      d.L = (uint32_t)s.L;
+      d.Lh = (uint32_t)s.L / 2;
+      d.nh = (uint32_t)(n / 2);
+      d.plane = d.L * d.Lh;
+      d.k0 = (uint32_t)(s.seed & 0xFFFFFFFFu);
+      d.k1 = (uint32_t)(s.seed >> 32) ^ ((2u * s.sample + s.replica) * 0x9E3779B9u);
+      d.sweep_lo = (uint32_t)(s.sweep & 0xFFFFFFFFu);
+      d.sweep_hi = (uint32_t)(s.sweep >> 32);
+      d.beta = std::isinf(s.T) ? 0.0f : (float)(1.0 / s.T);
+      d.active = 1;
+      d.spin_off = s.off / sizeof(float4);
+      d.j_off = (s.off + sizeof(float4) * n) / sizeof(float);
+      d.by_plane = hsg::make_fastdiv(d.plane);
+      d.by_lh = hsg::make_fastdiv(d.Lh);
+      d.tile_begin = nt;
+      for (uint32_t q0 = 0; q0 < d.nh; q0 += (uint32_t)p->tile_sites) h_tiles[nt++] = make_uint2((uint32_t)i, q0);
+      d.tile_count = nt - d.tile_begin;
+    }
+    h_ntiles[pass] = nt;
   }
-  *h_ntiles = nt;
+  p->unbatched_left = h_ntiles[0] > 0;
   if ((e = cudaMemcpyAsync(p->d_desc, h_desc, sizeof(PoolDesc) * p->max_slots, cudaMemcpyHostToDevice,
                            p->stream)) != cudaSuccess ||
       (nt && (e = cudaMemcpyAsync(p->d_tiles, h_tiles, sizeof(uint2) * nt, cudaMemcpyHostToDevice, p->stream)) !=
                  cudaSuccess) ||
-      (e = cudaMemcpyAsync(p->d_ntiles, h_ntiles, sizeof(uint32_t), cudaMemcpyHostToDevice, p->stream)) !=
+      (e = cudaMemcpyAsync(p->d_ntiles, h_ntiles, 2 * sizeof(uint32_t), cudaMemcpyHostToDevice, p->stream)) !=
           cudaSuccess ||
       (e = cudaEventRecord(p->up_ev[b], p->stream)) != cudaSuccess)
     return pcuda(p, e, "pool table upload");
@@ -407,7 +434,7 @@ hsg_status sync_tables(hsg_pool* p) {
 
 unsigned pool_grid(const hsg_pool* p) { return (unsigned)(p->sm_count * p->blocks_per_sm); }
 
-cudaError_t launch_pool_half(hsg_pool* p, int upd, uint32_t colour, float step, int hits, int hit0) {
+cudaError_t launch_pool_half(hsg_pool* p, const uint32_t* NT, int upd, uint32_t colour, float step, int hits, int hit0) {
   const dim3 g(pool_grid(p)), b(p->threads);
   const float4* S4 = reinterpret_cast<const float4*>(p->arena);
   float4* S = const_cast<float4*>(S4);
@@ -415,7 +442,6 @@ cudaError_t launch_pool_half(hsg_pool* p, int upd, uint32_t colour, float step, 
   const uint32_t ts = (uint32_t)p->tile_sites;
   const PoolDesc* D = p->d_desc;
   const uint2* T = p->d_tiles;
-  const uint32_t* NT = p->d_ntiles;
   cudaStream_t st = p->stream;
   switch (upd) {
     case hsg::U_OR: k_pool_half_sweep<hsg::U_OR><<<g, b, 0, st>>>(D, T, NT, S, J, colour, step, hits, hit0, ts); break;
@@ -448,8 +474,10 @@ int main_passes(const hsg_pool* p, const hsg_schedule* s) {
 }
 
 // The launches of one sweep, in the single-lattice order: main update on
-// colour 0 then 1, n_or OR sweeps, counter advance, renormalisation.
-cudaError_t enqueue_sweep(hsg_pool* p, const hsg_schedule* s) {
+// colour 0 then 1, n_or OR sweeps, counter advance, renormalisation.  `all`:
+// every lattice, else those that are not batched.
+cudaError_t enqueue_sweep(hsg_pool* p, const hsg_schedule* s, bool all) {
+  const uint32_t* NT = p->d_ntiles + (all ? 1 : 0);
   cudaError_t e = cudaSuccess;
   if (s->kind != HSG_NONE) {
     const bool ball = s->proposal == HSG_PROP_BALL;
@@ -462,21 +490,147 @@ cudaError_t enqueue_sweep(hsg_pool* p, const hsg_schedule* s) {
       for (int k = 0, j0 = 0; k < passes && e == cudaSuccess; ++k, j0 += per) {
         const int n = std::min(per, s->hits - j0);
         // the fused reflection follows the colour's last hit only
-        e = launch_pool_half(p, (fused && k + 1 < passes) ? met : upd, c, s->step, n, j0);
+        e = launch_pool_half(p, NT, (fused && k + 1 < passes) ? met : upd, c, s->step, n, j0);
       }
   }
   for (int o = 0; o < s->n_or && e == cudaSuccess; ++o)
-    for (uint32_t c = 0; c < 2 && e == cudaSuccess; ++c) e = launch_pool_half(p, hsg::U_OR, c, s->step, s->hits, 0);
+    for (uint32_t c = 0; c < 2 && e == cudaSuccess; ++c) e = launch_pool_half(p, NT, hsg::U_OR, c, s->step, s->hits, 0);
   if (e != cudaSuccess) return e;
-  k_pool_advance<<<cdiv_u((unsigned)p->max_slots, 256), 256, 0, p->stream>>>(p->d_desc, p->max_slots);
+  k_pool_advance<<<cdiv_u((unsigned)p->max_slots, 256), 256, 0, p->stream>>>(p->d_desc, p->max_slots, 1u);
   p->launches += 1;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (s->renorm_every > 0) {
-    k_pool_renorm<<<pool_grid(p), p->threads, 0, p->stream>>>(p->d_desc, p->d_tiles, p->d_ntiles,
+    k_pool_renorm<<<pool_grid(p), p->threads, 0, p->stream>>>(p->d_desc, p->d_tiles, NT,
                                                               reinterpret_cast<float4*>(p->arena),
                                                               (uint32_t)s->renorm_every, (uint32_t)p->tile_sites);
     p->launches += 1;
     e = cudaGetLastError();
+  }
+  return e;
+}
+
+// A batch and the stream that sweeps it: 0 the pool's own, k the side stream k - 1.
+struct PoolBatch {
+  hsg::BatchArgs a;
+  int lane;
+};
+constexpr int kLanes = 1 + hsg_pool::kSide;
+
+// The slots' lattices of L >= kBatchMinL in batches of about kBatchBytes, each
+// given to the lane with the fewest bytes so far (the pool's own stream
+// first sweeps the other lattices: counted twice, their kernels being slower).
+std::vector<PoolBatch> make_batches(const hsg_pool* p) {
+  std::vector<PoolBatch> out;
+  uint64_t load[kLanes] = {};
+  for (const Slot& sl : p->slots)
+    if (sl.active && sl.L < hsg::kBatchMinL) load[0] += 2 * sl.bytes;
+  uint64_t bytes = 0;
+  for (const Slot& sl : p->slots) {
+    if (!sl.active || sl.L < hsg::kBatchMinL) continue;
+    if (out.empty() || out.back().a.n == hsg::kBatchMax || bytes + sl.bytes > kBatchBytes) {
+      out.emplace_back();
+      out.back().a.n = 0;
+      out.back().lane = (int)(std::min_element(load, load + kLanes) - load);
+      bytes = 0;
+    }
+    bytes += sl.bytes;
+    load[out.back().lane] += sl.bytes;
+    hsg::BatchLattice& l = out.back().a.lat[out.back().a.n++];
+    const uint64_t n = (uint64_t)sl.L * sl.L * sl.L;
+    l.spins = reinterpret_cast<float4*>(p->arena + sl.off);
+    l.J = reinterpret_cast<const float*>(p->arena + sl.off + sizeof(float4) * n);
+    l.sweep = sl.sweep;
+    l.nh = (uint32_t)(n / 2);
+    l.L = (uint32_t)sl.L;
+    l.Lh = (uint32_t)sl.L / 2;
+    l.k0 = (uint32_t)(sl.seed & 0xFFFFFFFFu);
+    l.k1 = (uint32_t)(sl.seed >> 32) ^ ((2u * sl.sample + sl.replica) * 0x9E3779B9u);
+    l.beta = std::isinf(sl.T) ? 0.0f : (float)(1.0 / sl.T);
+    l.by_lh = hsg::make_fastdiv(l.Lh);
+  }
+  return out;
+}
+
+// The launches of one sweep of a batch, in the single-lattice order.
+struct BatchSweep {
+  hsg_pool* p;
+  const hsg_schedule* s;
+  int upd, met, passes, per;
+  BatchSweep(hsg_pool* pool, const hsg_schedule* sched) : p(pool), s(sched) {
+    const bool ball = s->proposal == HSG_PROP_BALL;
+    met = ball ? hsg::U_MET_BALL : hsg::U_MET_SPHERE;
+    upd = s->kind == HSG_HEATBATH         ? hsg::U_HB
+          : s->kind == HSG_METROPOLIS_OR ? (ball ? hsg::U_MET_OR_BALL : hsg::U_MET_OR_SPHERE)
+                                          : met;
+    passes = main_passes(p, s);
+    per = passes ? (s->hits + passes - 1) / passes : 0;
+  }
+  int steps() const { return 2 * passes + 2 * s->n_or + (s->renorm_every > 0); }
+  cudaError_t launch(hsg::BatchArgs& a, int step, int sweep_add, cudaStream_t st) const {
+    if (step < 2 * passes) {
+      const int q = step % passes, j0 = q * per;
+      // the fused reflection follows the colour's last hit only
+      const int u = s->kind == HSG_METROPOLIS_OR && q + 1 < passes ? met : upd;
+      p->launches += 1;
+      return hsg::launch_batch_half(u, a, (uint32_t)(step / passes), std::min(per, s->hits - j0), j0, s->step,
+                                    (uint32_t)sweep_add, st);
+    }
+    step -= 2 * passes;
+    if (step < 2 * s->n_or) {
+      p->launches += 1;
+      return hsg::launch_batch_half(hsg::U_OR, a, (uint32_t)step & 1u, 1, 0, s->step, (uint32_t)sweep_add, st);
+    }
+    hsg::BatchArgs due;
+    due.n = 0;
+    for (int k = 0; k < a.n; ++k)
+      if ((a.lat[k].sweep + (uint64_t)sweep_add + 1) % (uint64_t)s->renorm_every == 0) due.lat[due.n++] = a.lat[k];
+    if (due.n) p->launches += 1;
+    return hsg::launch_batch_renorm(due, st);
+  }
+};
+
+// The side streams and events, made once.
+cudaError_t make_side_streams(hsg_pool* p) {
+  cudaError_t e = cudaSuccess;
+  if (!p->fork_ev) e = cudaEventCreateWithFlags(&p->fork_ev, cudaEventDisableTiming);
+  for (int i = 0; i < hsg_pool::kSide && e == cudaSuccess; ++i) {
+    if (!p->side[i]) e = cudaStreamCreateWithFlags(&p->side[i], cudaStreamNonBlocking);
+    if (e == cudaSuccess && !p->join_ev[i]) e = cudaEventCreateWithFlags(&p->join_ev[i], cudaEventDisableTiming);
+  }
+  return e;
+}
+
+// n_sweeps sweeps of the batches, each batch all of its sweeps on its lane,
+// the lanes' launches interleaved.  The side streams start after what the
+// pool's stream held at fork_ev, and the pool's stream then waits for them.
+cudaError_t sweep_batches(hsg_pool* p, const hsg_schedule* s, int n_sweeps, std::vector<PoolBatch>& batches) {
+  const cudaStream_t st[kLanes] = {p->stream, p->side[0], p->side[1]};
+  const BatchSweep sweep(p, s);
+  cudaError_t e = cudaSuccess;
+  bool used[kLanes] = {};
+  for (const PoolBatch& b : batches) used[b.lane] = true;
+  for (int l = 1; l < kLanes && e == cudaSuccess; ++l)
+    if (used[l]) e = cudaStreamWaitEvent(st[l], p->fork_ev, 0);
+  size_t at[kLanes] = {};  // each lane's batch at hand
+  for (;;) {
+    bool any = false;
+    for (int l = 0; l < kLanes; ++l) {
+      while (at[l] < batches.size() && batches[at[l]].lane != l) ++at[l];
+      any |= at[l] < batches.size();
+    }
+    if (!any || e != cudaSuccess) break;
+    for (int k = 0; k < n_sweeps && e == cudaSuccess; ++k)
+      for (int i = 0; i < sweep.steps() && e == cudaSuccess; ++i)
+        for (int l = 0; l < kLanes && e == cudaSuccess; ++l)
+          if (at[l] < batches.size()) e = sweep.launch(batches[at[l]].a, i, k, st[l]);
+    for (size_t& i : at) ++i;
+  }
+  // whatever was queued on the side streams, the pool's stream waits for
+  for (int l = 1; l < kLanes; ++l) {
+    if (!used[l]) continue;
+    cudaError_t j = cudaEventRecord(p->join_ev[l - 1], st[l]);
+    if (j == cudaSuccess) j = cudaStreamWaitEvent(p->stream, p->join_ev[l - 1], 0);
+    if (e == cudaSuccess) e = j;
   }
   return e;
 }
@@ -518,8 +672,8 @@ hsg_status hsg_pool_create(hsg_pool** out, uint64_t budget_bytes, int max_slots,
   if (e == cudaSuccess) e = cudaMalloc(&p->arena, p->budget);
   if (e == cudaSuccess) e = cudaMalloc(&p->d_desc, sizeof(PoolDesc) * max_slots);
   if (e == cudaSuccess) e = cudaMallocHost(&p->h_desc, 2 * sizeof(PoolDesc) * max_slots);
-  if (e == cudaSuccess) e = cudaMalloc(&p->d_ntiles, sizeof(uint32_t));
-  if (e == cudaSuccess) e = cudaMallocHost(&p->h_ntiles, 2 * sizeof(uint32_t));
+  if (e == cudaSuccess) e = cudaMalloc(&p->d_ntiles, 2 * sizeof(uint32_t));
+  if (e == cudaSuccess) e = cudaMallocHost(&p->h_ntiles, 4 * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc(&p->d_energy, sizeof(double) * max_slots);
   if (e == cudaSuccess) e = cudaMallocHost(&p->h_energy, hsg_pool::kEnergyBufs * sizeof(double) * max_slots);
   if (e == cudaSuccess) e = cudaMallocHost(&p->h_sel, (size_t)hsg_pool::kEnergyBufs * max_slots);
@@ -533,7 +687,6 @@ hsg_status hsg_pool_create(hsg_pool** out, uint64_t budget_bytes, int max_slots,
     return st;
   }
   p->free_blocks[0] = p->budget;
-  p->h_ntiles[0] = p->h_ntiles[1] = 0;
   *out = p;
   return HSG_OK;
 }
@@ -557,6 +710,11 @@ hsg_status hsg_pool_destroy(hsg_pool* p) {
   cudaFreeHost(p->h_energy);
   cudaFreeHost(p->h_sel);
   cudaFree(p->d_sel);
+  if (p->fork_ev) cudaEventDestroy(p->fork_ev);
+  for (int i = 0; i < hsg_pool::kSide; ++i) {
+    if (p->side[i]) cudaStreamDestroy(p->side[i]);
+    if (p->join_ev[i]) cudaEventDestroy(p->join_ev[i]);
+  }
   for (cudaEvent_t ev : p->up_ev)
     if (ev) cudaEventDestroy(ev);
   for (cudaEvent_t ev : p->en_ev)
@@ -665,17 +823,41 @@ hsg_status hsg_pool_sweep(hsg_pool* p, const hsg_schedule* sched, int n_sweeps) 
                                sched->renorm_every, p->threads,   p->tile_sites,        p->blocks_per_sm,
                                p->hits_per_pass, sched->step};
   cudaError_t e = cudaSuccess;
+  // While the caller captures the stream, the persistent kernels take every
+  // lattice: they read the sweep counters from the device, so that each
+  // replay of the caller's graph is the next sweep.
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if ((e = cudaStreamIsCapturing(p->stream, &cap)) != cudaSuccess) return pcuda(p, e, "pool sweep");
+  const bool batch = p->batched && cap == cudaStreamCaptureStatusNone;
+  std::vector<PoolBatch> batches;
+  if (batch) {
+    try {
+      batches = make_batches(p);
+    } catch (const std::bad_alloc&) {
+      return pfail(p, HSG_ENOMEM, "host allocation failed");
+    }
+    if ((e = make_side_streams(p)) == cudaSuccess) e = cudaEventRecord(p->fork_ev, p->stream);
+    if (e != cudaSuccess) return pcuda(p, e, "pool streams");
+  }
   // One sweep is captured once per (schedule, launch configuration) and
   // replayed; the legacy default stream cannot be captured, so there the
   // launches are issued directly.
-  if (p->stream != nullptr) {
+  if (p->batched && !batch) {
+    for (int k = 0; k < n_sweeps && e == cudaSuccess; ++k) e = enqueue_sweep(p, sched, true);
+  } else if (batch && !p->unbatched_left) {
+    // the device's counters follow the host's
+    k_pool_advance<<<cdiv_u((unsigned)p->max_slots, 256), 256, 0, p->stream>>>(p->d_desc, p->max_slots,
+                                                                              (uint32_t)n_sweeps);
+    p->launches += 1;
+    e = cudaGetLastError();
+  } else if (p->stream != nullptr) {
     if (!p->have_graph || !(p->gkey == key)) {
       drop_graph(p);
       cudaGraph_t g = nullptr;
       e = cudaStreamBeginCapture(p->stream, cudaStreamCaptureModeThreadLocal);
       if (e == cudaSuccess) {
         const uint64_t before = p->launches;
-        cudaError_t e2 = enqueue_sweep(p, sched);
+        cudaError_t e2 = enqueue_sweep(p, sched, false);
         p->launches = before;
         e = cudaStreamEndCapture(p->stream, &g);
         if (e == cudaSuccess) e = e2;
@@ -692,8 +874,9 @@ hsg_status hsg_pool_sweep(hsg_pool* p, const hsg_schedule* sched, int n_sweeps) 
       p->launches += (uint64_t)per_sweep;
     }
   } else {
-    for (int k = 0; k < n_sweeps && e == cudaSuccess; ++k) e = enqueue_sweep(p, sched);
+    for (int k = 0; k < n_sweeps && e == cudaSuccess; ++k) e = enqueue_sweep(p, sched, false);
   }
+  if (batch && e == cudaSuccess) e = sweep_batches(p, sched, n_sweeps, batches);
   if (e != cudaSuccess) return pcuda(p, e, "pool sweep");
   for (Slot& s : p->slots)
     if (s.active) s.sweep += (uint64_t)n_sweeps;
@@ -724,7 +907,7 @@ hsg_status enqueue_energies(hsg_pool* p, int b, const int* slots = nullptr, int 
     sel = p->d_sel;
   }
   if (p->n_active > 0 && (!slots || n > 0)) {
-    k_pool_energy_partial<<<pool_grid(p), 256, 0, p->stream>>>(p->d_desc, p->d_tiles, p->d_ntiles,
+    k_pool_energy_partial<<<pool_grid(p), 256, 0, p->stream>>>(p->d_desc, p->d_tiles, p->d_ntiles + 1,
                                                                 reinterpret_cast<const float4*>(p->arena),
                                                                 reinterpret_cast<const float*>(p->arena),
                                                                 (uint32_t)p->tile_sites, sel, p->d_partials);
