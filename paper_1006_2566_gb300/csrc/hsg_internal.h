@@ -148,28 +148,41 @@ struct FastDiv {
   uint32_t m, s1, s2;
 };
 
-// Sweeps of one small lattice in one launch (hsg_resident.cu).
+// Sweeps of small lattices in one launch (hsg_resident.cu).
+struct ResidentLattice {
+  float4* spins;    // S[2][N/2] (packed: [2][3][N/2] floats), read and written back
+  const float* J;   // J[3][2][N/2]
+  unsigned long long sweep;  // sweep counter (a pool's; a context's is on the device)
+  uint32_t k0, k1;
+  float beta;
+};
+template <int N>
 struct ResidentArgs {
-  float4* spins;  // S[2][N/2] (packed: [2][3][N/2] floats), read and written back
-  const float* J;  // J[3][2][N/2]
-  size_t nh;       // N/2
+  uint32_t L;
   bool packed;
-  uint32_t L, Lh;
   uint32_t sweeps;        // sweeps to run
   uint32_t per_sweep;     // half-sweeps of a sweep, the main update's two first
   uint32_t renorm_every;  // 0 = never
-  uint32_t k0, k1;
-  float beta, step;
+  float step;
   int hits;
-  unsigned long long* sweep_ptr;  // device sweep counter, advanced by `sweeps`
-  // set by launch_resident
-  uint32_t cluster, max_planes, plane;
+  unsigned long long* sweep_ptr;  // N = 1: the lattice's counter on the device, advanced by `sweeps`
+  int n;                          // lattices
+  ResidentLattice lat[N];
+  // set by the launcher
+  size_t nh;
+  uint32_t cluster, max_planes, Lh, plane;
   FastDiv by_plane, by_Lh;
 };
 constexpr int kResidentMaxL = 32;
+constexpr int kResidentPoolMax = 64;  // lattices of one L in one launch: 2.6 KB of parameters
+// Sites of a pool's small lattices up to which it takes them so.
+constexpr unsigned long long kResidentPoolSites = 640 * 1024;
 // `upd`: the main update's kind, or U_OR for over-relaxation only.
 bool resident_takes(int upd, int L, int hits);
-cudaError_t launch_resident(int upd, const ResidentArgs& a, cudaStream_t s);
+cudaError_t launch_resident(int upd, const ResidentArgs<1>& a, cudaStream_t s);
+// For a pool, whose `total` lattices of this L go in several such launches.
+cudaError_t launch_resident_pool(int upd, const ResidentArgs<kResidentPoolMax>& a, int total, int sm_count,
+                                 cudaStream_t s);
 
 // A batch of pool lattices swept by one launch per half-sweep (hsg_batch.cu),
 // handed over as kernel parameters.

@@ -434,7 +434,7 @@ hsg_status sync_tables(hsg_pool* p) {
 
 unsigned pool_grid(const hsg_pool* p) { return (unsigned)(p->sm_count * p->blocks_per_sm); }
 
-cudaError_t launch_pool_half(hsg_pool* p, const uint32_t* NT, int upd, uint32_t colour, float step, int hits, int hit0) {
+cudaError_t launch_pool_half(hsg_pool* p, int upd, uint32_t colour, float step, int hits, int hit0) {
   const dim3 g(pool_grid(p)), b(p->threads);
   const float4* S4 = reinterpret_cast<const float4*>(p->arena);
   float4* S = const_cast<float4*>(S4);
@@ -442,6 +442,7 @@ cudaError_t launch_pool_half(hsg_pool* p, const uint32_t* NT, int upd, uint32_t 
   const uint32_t ts = (uint32_t)p->tile_sites;
   const PoolDesc* D = p->d_desc;
   const uint2* T = p->d_tiles;
+  const uint32_t* NT = p->d_ntiles;
   cudaStream_t st = p->stream;
   switch (upd) {
     case hsg::U_OR: k_pool_half_sweep<hsg::U_OR><<<g, b, 0, st>>>(D, T, NT, S, J, colour, step, hits, hit0, ts); break;
@@ -474,10 +475,8 @@ int main_passes(const hsg_pool* p, const hsg_schedule* s) {
 }
 
 // The launches of one sweep, in the single-lattice order: main update on
-// colour 0 then 1, n_or OR sweeps, counter advance, renormalisation.  `all`:
-// every lattice, else those that are not batched.
-cudaError_t enqueue_sweep(hsg_pool* p, const hsg_schedule* s, bool all) {
-  const uint32_t* NT = p->d_ntiles + (all ? 1 : 0);
+// colour 0 then 1, n_or OR sweeps, counter advance, renormalisation.
+cudaError_t enqueue_sweep(hsg_pool* p, const hsg_schedule* s) {
   cudaError_t e = cudaSuccess;
   if (s->kind != HSG_NONE) {
     const bool ball = s->proposal == HSG_PROP_BALL;
@@ -490,17 +489,17 @@ cudaError_t enqueue_sweep(hsg_pool* p, const hsg_schedule* s, bool all) {
       for (int k = 0, j0 = 0; k < passes && e == cudaSuccess; ++k, j0 += per) {
         const int n = std::min(per, s->hits - j0);
         // the fused reflection follows the colour's last hit only
-        e = launch_pool_half(p, NT, (fused && k + 1 < passes) ? met : upd, c, s->step, n, j0);
+        e = launch_pool_half(p, (fused && k + 1 < passes) ? met : upd, c, s->step, n, j0);
       }
   }
   for (int o = 0; o < s->n_or && e == cudaSuccess; ++o)
-    for (uint32_t c = 0; c < 2 && e == cudaSuccess; ++c) e = launch_pool_half(p, NT, hsg::U_OR, c, s->step, s->hits, 0);
+    for (uint32_t c = 0; c < 2 && e == cudaSuccess; ++c) e = launch_pool_half(p, hsg::U_OR, c, s->step, s->hits, 0);
   if (e != cudaSuccess) return e;
   k_pool_advance<<<cdiv_u((unsigned)p->max_slots, 256), 256, 0, p->stream>>>(p->d_desc, p->max_slots, 1u);
   p->launches += 1;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (s->renorm_every > 0) {
-    k_pool_renorm<<<pool_grid(p), p->threads, 0, p->stream>>>(p->d_desc, p->d_tiles, NT,
+    k_pool_renorm<<<pool_grid(p), p->threads, 0, p->stream>>>(p->d_desc, p->d_tiles, p->d_ntiles,
                                                               reinterpret_cast<float4*>(p->arena),
                                                               (uint32_t)s->renorm_every, (uint32_t)p->tile_sites);
     p->launches += 1;
@@ -509,13 +508,110 @@ cudaError_t enqueue_sweep(hsg_pool* p, const hsg_schedule* s, bool all) {
   return e;
 }
 
-// A batch and the stream that sweeps it: 0 the pool's own, k the side stream k - 1.
+float beta_of(double T) { return std::isinf(T) ? 0.0f : (float)(1.0 / T); }
+uint32_t key0(const Slot& s) { return (uint32_t)(s.seed & 0xFFFFFFFFu); }
+uint32_t key1(const Slot& s) { return (uint32_t)(s.seed >> 32) ^ ((2u * s.sample + s.replica) * 0x9E3779B9u); }
+
+int main_update(const hsg_schedule* s) {
+  const bool ball = s->proposal == HSG_PROP_BALL;
+  switch (s->kind) {
+    case HSG_METROPOLIS: return ball ? hsg::U_MET_BALL : hsg::U_MET_SPHERE;
+    case HSG_METROPOLIS_OR: return ball ? hsg::U_MET_OR_BALL : hsg::U_MET_OR_SPHERE;
+    case HSG_HEATBATH: return hsg::U_HB;
+    default: return hsg::U_OR;
+  }
+}
+
+// Lanes: the pool's own stream and the side streams, on which independent
+// lattices are swept side by side.
+constexpr int kLanes = 1 + hsg_pool::kSide;
+
+// The side streams and events, made once.
+cudaError_t make_side_streams(hsg_pool* p) {
+  cudaError_t e = cudaSuccess;
+  if (!p->fork_ev) e = cudaEventCreateWithFlags(&p->fork_ev, cudaEventDisableTiming);
+  for (int i = 0; i < hsg_pool::kSide && e == cudaSuccess; ++i) {
+    if (!p->side[i]) e = cudaStreamCreateWithFlags(&p->side[i], cudaStreamNonBlocking);
+    if (e == cudaSuccess && !p->join_ev[i]) e = cudaEventCreateWithFlags(&p->join_ev[i], cudaEventDisableTiming);
+  }
+  return e;
+}
+
+// The pool's stream waits for whatever was queued on the lanes used; returns
+// the first error, `e` before its own.
+cudaError_t join_lanes(hsg_pool* p, const bool (&used)[kLanes], cudaError_t e) {
+  for (int l = 1; l < kLanes; ++l) {
+    if (!used[l]) continue;
+    cudaError_t j = cudaEventRecord(p->join_ev[l - 1], p->side[l - 1]);
+    if (j == cudaSuccess) j = cudaStreamWaitEvent(p->stream, p->join_ev[l - 1], 0);
+    if (e == cudaSuccess) e = j;
+  }
+  return e;
+}
+
+// Whether the small lattices take the resident kernel (hsg_resident.cu),
+// which then runs every sweep of a call in one launch per side.  All of
+// them or none: while the persistent kernels run for others anyway, a few small
+// lattices cost them nothing, and a launch of their own would come on top.
+bool resident_pool(const hsg_pool* p, const hsg_schedule* s) {
+  if (s->kind == HSG_NONE && s->n_or == 0) return false;
+  if (main_passes(p, s) > 1) return false;  // the hits in passes, as configured
+  uint64_t sites = 0;
+  for (const Slot& sl : p->slots) {
+    if (!sl.active) continue;
+    if (sl.L >= hsg::kBatchMinL ? !p->batched : !hsg::resident_takes(main_update(s), sl.L, s->hits)) return false;
+    if (sl.L < hsg::kBatchMinL) sites += (uint64_t)sl.L * sl.L * sl.L;
+  }
+  return sites > 0 && sites <= hsg::kResidentPoolSites;
+}
+
+// n_sweeps sweeps of the small lattices, side by side: each side's launches on the
+// lane (the pool's stream and the side streams) with the fewest sites so far.
+cudaError_t sweep_resident(hsg_pool* p, const hsg_schedule* s, int n_sweeps) {
+  int count[hsg::kBatchMinL] = {};
+  for (const Slot& sl : p->slots)
+    if (sl.active && sl.L < hsg::kBatchMinL) count[sl.L] += 1;
+  const cudaStream_t st[kLanes] = {p->stream, p->side[0], p->side[1]};
+  uint64_t load[kLanes] = {};
+  bool used[kLanes] = {};
+  cudaError_t e = cudaSuccess;
+  for (int L = hsg::kBatchMinL - 2; L >= 4 && e == cudaSuccess; L -= 2) {
+    if (count[L] == 0) continue;
+    const int lane = (int)(std::min_element(load, load + kLanes) - load);
+    const uint64_t n = (uint64_t)L * L * L;
+    load[lane] += count[L] * n;
+    if (lane > 0 && !used[lane]) e = cudaStreamWaitEvent(st[lane], p->fork_ev, 0);
+    used[lane] = true;
+    hsg::ResidentArgs<hsg::kResidentPoolMax> a{};
+    a.L = (uint32_t)L;
+    a.sweeps = (uint32_t)n_sweeps;
+    a.per_sweep = (s->kind != HSG_NONE ? 2u : 0u) + 2u * (uint32_t)s->n_or;
+    a.renorm_every = (uint32_t)s->renorm_every;
+    a.step = s->step;
+    a.hits = s->hits;
+    int left = count[L];
+    for (size_t i = 0; i < p->slots.size() && left > 0 && e == cudaSuccess; ++i) {
+      const Slot& sl = p->slots[i];
+      if (!sl.active || sl.L != L) continue;
+      a.lat[a.n++] = {reinterpret_cast<float4*>(p->arena + sl.off),
+                      reinterpret_cast<const float*>(p->arena + sl.off + sizeof(float4) * n),
+                      sl.sweep, key0(sl), key1(sl), beta_of(sl.T)};
+      left -= 1;
+      if (a.n == hsg::kResidentPoolMax || left == 0) {
+        e = hsg::launch_resident_pool(main_update(s), a, count[L], p->sm_count, st[lane]);
+        p->launches += 1;
+        a.n = 0;
+      }
+    }
+  }
+  return join_lanes(p, used, e);
+}
+
+// A batch and the lane that sweeps it.
 struct PoolBatch {
   hsg::BatchArgs a;
   int lane;
 };
-constexpr int kLanes = 1 + hsg_pool::kSide;
-
 // The slots' lattices of L >= kBatchMinL in batches of about kBatchBytes, each
 // given to the lane with the fewest bytes so far (the pool's own stream
 // first sweeps the other lattices: counted twice, their kernels being slower).
@@ -543,9 +639,9 @@ std::vector<PoolBatch> make_batches(const hsg_pool* p) {
     l.nh = (uint32_t)(n / 2);
     l.L = (uint32_t)sl.L;
     l.Lh = (uint32_t)sl.L / 2;
-    l.k0 = (uint32_t)(sl.seed & 0xFFFFFFFFu);
-    l.k1 = (uint32_t)(sl.seed >> 32) ^ ((2u * sl.sample + sl.replica) * 0x9E3779B9u);
-    l.beta = std::isinf(sl.T) ? 0.0f : (float)(1.0 / sl.T);
+    l.k0 = key0(sl);
+    l.k1 = key1(sl);
+    l.beta = beta_of(sl.T);
     l.by_lh = hsg::make_fastdiv(l.Lh);
   }
   return out;
@@ -557,11 +653,8 @@ struct BatchSweep {
   const hsg_schedule* s;
   int upd, met, passes, per;
   BatchSweep(hsg_pool* pool, const hsg_schedule* sched) : p(pool), s(sched) {
-    const bool ball = s->proposal == HSG_PROP_BALL;
-    met = ball ? hsg::U_MET_BALL : hsg::U_MET_SPHERE;
-    upd = s->kind == HSG_HEATBATH         ? hsg::U_HB
-          : s->kind == HSG_METROPOLIS_OR ? (ball ? hsg::U_MET_OR_BALL : hsg::U_MET_OR_SPHERE)
-                                          : met;
+    met = s->proposal == HSG_PROP_BALL ? hsg::U_MET_BALL : hsg::U_MET_SPHERE;
+    upd = main_update(s);
     passes = main_passes(p, s);
     per = passes ? (s->hits + passes - 1) / passes : 0;
   }
@@ -589,17 +682,6 @@ struct BatchSweep {
   }
 };
 
-// The side streams and events, made once.
-cudaError_t make_side_streams(hsg_pool* p) {
-  cudaError_t e = cudaSuccess;
-  if (!p->fork_ev) e = cudaEventCreateWithFlags(&p->fork_ev, cudaEventDisableTiming);
-  for (int i = 0; i < hsg_pool::kSide && e == cudaSuccess; ++i) {
-    if (!p->side[i]) e = cudaStreamCreateWithFlags(&p->side[i], cudaStreamNonBlocking);
-    if (e == cudaSuccess && !p->join_ev[i]) e = cudaEventCreateWithFlags(&p->join_ev[i], cudaEventDisableTiming);
-  }
-  return e;
-}
-
 // n_sweeps sweeps of the batches, each batch all of its sweeps on its lane,
 // the lanes' launches interleaved.  The side streams start after what the
 // pool's stream held at fork_ev, and the pool's stream then waits for them.
@@ -625,14 +707,7 @@ cudaError_t sweep_batches(hsg_pool* p, const hsg_schedule* s, int n_sweeps, std:
           if (at[l] < batches.size()) e = sweep.launch(batches[at[l]].a, i, k, st[l]);
     for (size_t& i : at) ++i;
   }
-  // whatever was queued on the side streams, the pool's stream waits for
-  for (int l = 1; l < kLanes; ++l) {
-    if (!used[l]) continue;
-    cudaError_t j = cudaEventRecord(p->join_ev[l - 1], st[l]);
-    if (j == cudaSuccess) j = cudaStreamWaitEvent(p->stream, p->join_ev[l - 1], 0);
-    if (e == cudaSuccess) e = j;
-  }
-  return e;
+  return join_lanes(p, used, e);
 }
 
 hsg_status check_pool_schedule(hsg_pool* p, const hsg_schedule* s) {
@@ -823,12 +898,12 @@ hsg_status hsg_pool_sweep(hsg_pool* p, const hsg_schedule* sched, int n_sweeps) 
                                sched->renorm_every, p->threads,   p->tile_sites,        p->blocks_per_sm,
                                p->hits_per_pass, sched->step};
   cudaError_t e = cudaSuccess;
-  // While the caller captures the stream, the persistent kernels take every
-  // lattice: they read the sweep counters from the device, so that each
-  // replay of the caller's graph is the next sweep.
+  // A capture of the pool's stream by the caller is refused by the graph
+  // path below, as the sweep's own graph can be neither captured nor launched in it.
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if ((e = cudaStreamIsCapturing(p->stream, &cap)) != cudaSuccess) return pcuda(p, e, "pool sweep");
   const bool batch = p->batched && cap == cudaStreamCaptureStatusNone;
+  const bool resident = cap == cudaStreamCaptureStatusNone && resident_pool(p, sched);
   std::vector<PoolBatch> batches;
   if (batch) {
     try {
@@ -836,20 +911,23 @@ hsg_status hsg_pool_sweep(hsg_pool* p, const hsg_schedule* sched, int n_sweeps) 
     } catch (const std::bad_alloc&) {
       return pfail(p, HSG_ENOMEM, "host allocation failed");
     }
+  }
+  if (batch || resident) {
     if ((e = make_side_streams(p)) == cudaSuccess) e = cudaEventRecord(p->fork_ev, p->stream);
     if (e != cudaSuccess) return pcuda(p, e, "pool streams");
   }
   // One sweep is captured once per (schedule, launch configuration) and
   // replayed; the legacy default stream cannot be captured, so there the
   // launches are issued directly.
-  if (p->batched && !batch) {
-    for (int k = 0; k < n_sweeps && e == cudaSuccess; ++k) e = enqueue_sweep(p, sched, true);
-  } else if (batch && !p->unbatched_left) {
+  if (resident || (batch && !p->unbatched_left)) {
+    if (resident) e = sweep_resident(p, sched, n_sweeps);
     // the device's counters follow the host's
-    k_pool_advance<<<cdiv_u((unsigned)p->max_slots, 256), 256, 0, p->stream>>>(p->d_desc, p->max_slots,
-                                                                              (uint32_t)n_sweeps);
-    p->launches += 1;
-    e = cudaGetLastError();
+    if (e == cudaSuccess) {
+      k_pool_advance<<<cdiv_u((unsigned)p->max_slots, 256), 256, 0, p->stream>>>(p->d_desc, p->max_slots,
+                                                                                (uint32_t)n_sweeps);
+      p->launches += 1;
+      e = cudaGetLastError();
+    }
   } else if (p->stream != nullptr) {
     if (!p->have_graph || !(p->gkey == key)) {
       drop_graph(p);
@@ -857,7 +935,7 @@ hsg_status hsg_pool_sweep(hsg_pool* p, const hsg_schedule* sched, int n_sweeps) 
       e = cudaStreamBeginCapture(p->stream, cudaStreamCaptureModeThreadLocal);
       if (e == cudaSuccess) {
         const uint64_t before = p->launches;
-        cudaError_t e2 = enqueue_sweep(p, sched, false);
+        cudaError_t e2 = enqueue_sweep(p, sched);
         p->launches = before;
         e = cudaStreamEndCapture(p->stream, &g);
         if (e == cudaSuccess) e = e2;
@@ -874,7 +952,7 @@ hsg_status hsg_pool_sweep(hsg_pool* p, const hsg_schedule* sched, int n_sweeps) 
       p->launches += (uint64_t)per_sweep;
     }
   } else {
-    for (int k = 0; k < n_sweeps && e == cudaSuccess; ++k) e = enqueue_sweep(p, sched, false);
+    for (int k = 0; k < n_sweeps && e == cudaSuccess; ++k) e = enqueue_sweep(p, sched);
   }
   if (batch && e == cudaSuccess) e = sweep_batches(p, sched, n_sweeps, batches);
   if (e != cudaSuccess) return pcuda(p, e, "pool sweep");

@@ -1,4 +1,4 @@
-// hsg_resident.cu -- whole sweeps of one small lattice in a single launch.
+// hsg_resident.cu -- whole sweeps of small lattices in a single launch.
 //
 // A lone small lattice is bound by launches, not by work: a half-sweep of
 // L = 16 is 2048 site updates, 0.1 us of one GPU, but 1.3-2 us as a launch of
@@ -31,6 +31,11 @@
 //   L = 32   4 OR 20.3 -> 10.6 (13.1 -> 9.9), heat-bath 7.5 -> 5.5 (5.4 -> 4.6), 4 hits
 //            8.2 -> 8.3 (6.0 -> 7.3): there each hit costs 0.57 us against 0.19 on
 //            the whole GPU, hence the bound on the hits in resident_takes.
+// In a pool, one launch holds up to 64 lattices of one side, a cluster each, for
+// all the sweeps of a call (us per sweep, against the persistent kernels'
+// replayed graph): 8 x L = 16, 1 hit 10.6 -> 2.7; 128 x L = 16 16.4 -> 7.9; 64 x L = 16, 4 hits +
+// 2 OR 33 -> 13; 64 x L = 8 10.3 -> 2.3; with more work it is even (2048 x L = 16 131 -> 125)
+// or loses (64 x L = 24, 4 hits + 2 OR 56 -> 63), hence kResidentPoolSites.
 // A loop over sites with the indices formed and the bonds loaded for each
 // (so that larger lattices fit too): 7.9 us at L = 16, 24.9 against 14.0 at L = 40.
 #include "hsg_device.cuh"
@@ -64,21 +69,21 @@ __device__ __forceinline__ void st_cluster(uint32_t addr, float4 v) {
                : "memory");
 }
 
-__device__ __forceinline__ float4 load_spin(const ResidentArgs& a, uint32_t c, uint32_t g) {
-  if (a.packed) {
-    const float* b = reinterpret_cast<const float*>(a.spins) + 3 * c * a.nh + g;
-    return make_float4(b[0], b[a.nh], b[2 * a.nh], 0.0f);
+__device__ __forceinline__ float4 load_spin(const float4* S, bool packed, size_t nh, uint32_t c, uint32_t g) {
+  if (packed) {
+    const float* b = reinterpret_cast<const float*>(S) + 3 * c * nh + g;
+    return make_float4(b[0], b[nh], b[2 * nh], 0.0f);
   }
-  return a.spins[c * a.nh + g];
+  return S[c * nh + g];
 }
-__device__ __forceinline__ void store_spin(const ResidentArgs& a, uint32_t c, uint32_t g, float4 v) {
-  if (a.packed) {
-    float* b = reinterpret_cast<float*>(a.spins) + 3 * c * a.nh + g;
+__device__ __forceinline__ void store_spin(float4* S, bool packed, size_t nh, uint32_t c, uint32_t g, float4 v) {
+  if (packed) {
+    float* b = reinterpret_cast<float*>(S) + 3 * c * nh + g;
     b[0] = v.x;
-    b[a.nh] = v.y;
-    b[2 * a.nh] = v.z;
+    b[nh] = v.y;
+    b[2 * nh] = v.z;
   } else {
-    a.spins[c * a.nh + g] = v;
+    S[c * nh + g] = v;
   }
 }
 
@@ -88,8 +93,8 @@ struct KeptSite {
   float jxp, jxm, jyp, jym, jzp, jzm;
 };
 
-template <int U>
-__global__ void __launch_bounds__(kThreadsMax, 1) k_resident(const ResidentArgs a) {
+template <int U, int N>
+__global__ void __launch_bounds__(kThreadsMax, 1) k_resident(const __grid_constant__ ResidentArgs<N> a) {
   // sp[colour][plane][in-plane index]: plane 0 the halo below, 1 .. P this
   // CTA's own, P + 1 the halo above.
   extern __shared__ float4 sp[];
@@ -98,7 +103,8 @@ __global__ void __launch_bounds__(kThreadsMax, 1) k_resident(const ResidentArgs 
   const uint32_t z0 = rank * L / C, P = (rank + 1) * L / C - z0;
   const uint32_t part = (a.max_planes + 2) * plane;  // one colour's share of sp
   const uint32_t tid = threadIdx.x;
-  const unsigned long long sweep0 = *a.sweep_ptr;
+  const ResidentLattice& lat = a.lat[N == 1 ? 0u : blockIdx.x / C];
+  const unsigned long long sweep0 = N == 1 ? *a.sweep_ptr : lat.sweep;
 
   // This thread's sites: in-plane index r of plane z, for tid < P * plane.
   const bool mine = tid < P * plane;
@@ -113,20 +119,21 @@ __global__ void __launch_bounds__(kThreadsMax, 1) k_resident(const ResidentArgs 
 #pragma unroll
   for (uint32_t c = 0; c < 2; ++c) {
     const uint32_t p = p0 ^ c, gzm = z == 0 ? g + (L - 1) * plane : g - plane;
-    const float *Jc = a.J + c * a.nh, *Jo = a.J + (1 - c) * a.nh;
+    const float *Jc = lat.J + c * a.nh, *Jo = lat.J + (1 - c) * a.nh;
     k[c].jxp = __ldg(Jc + g);
     k[c].jxm = __ldg(Jo + (p ? g : g + dxm));
     k[c].jyp = __ldg(Jc + 2 * a.nh + g);
     k[c].jym = __ldg(Jo + 2 * a.nh + (g + dym));
     k[c].jzp = __ldg(Jc + 4 * a.nh + g);
     k[c].jzm = __ldg(Jo + 4 * a.nh + gzm);
-    k[c].s = load_spin(a, c, g);
+    k[c].s = load_spin(lat.spins, a.packed, a.nh, c, g);
     if (mine) sp[c * part + q] = k[c].s;
     for (uint32_t i = tid; i < 2 * plane; i += blockDim.x) {  // the halo planes z0 - 1 and z0 + P
       const bool lo = i < plane;
       const uint32_t ri = lo ? i : i - plane;
       const uint32_t zi = lo ? (z0 == 0 ? L - 1 : z0 - 1) : (z0 + P == L ? 0u : z0 + P);
-      sp[c * part + (lo ? 0u : (P + 1) * plane) + ri] = load_spin(a, c, zi * plane + ri);
+      sp[c * part + (lo ? 0u : (P + 1) * plane) + ri] =
+          load_spin(lat.spins, a.packed, a.nh, c, zi * plane + ri);
     }
   }
   // Where the CTA below (above) keeps this CTA's first (last) plane.
@@ -165,7 +172,7 @@ __global__ void __launch_bounds__(kThreadsMax, 1) k_resident(const ResidentArgs 
           in.s = make_float3(k[c].s.x, k[c].s.y, k[c].s.z);
           in.q = 0;
           in.site = (2 * xh + p) + y * L + z * L * L;
-          k[c].s = main_update ? site_result<U>(in, c, lo, hi, a.k0, a.k1, a.beta, a.step, a.hits)
+          k[c].s = main_update ? site_result<U>(in, c, lo, hi, lat.k0, lat.k1, lat.beta, a.step, a.hits)
                                : site_result<U_OR>(in, c, 0u, 0u, 0u, 0u, 0.0f, 0.0f, 1);
           sp[c * part + q] = k[c].s;
           if (first) st_cluster(to_below + c * part * 16u, k[c].s);
@@ -190,11 +197,11 @@ __global__ void __launch_bounds__(kThreadsMax, 1) k_resident(const ResidentArgs 
     }
   }
   if (mine) {
-    store_spin(a, 0, g, k[0].s);
-    store_spin(a, 1, g, k[1].s);
+    store_spin(lat.spins, a.packed, a.nh, 0, g, k[0].s);
+    store_spin(lat.spins, a.packed, a.nh, 1, g, k[1].s);
   }
   // Every CTA read the counter before the first barrier.
-  if (rank == 0 && tid == 0) *a.sweep_ptr = sweep0 + a.sweeps;
+  if (N == 1 && rank == 0 && tid == 0) *a.sweep_ptr = sweep0 + a.sweeps;
 }
 
 // CTAs in the cluster of an L lattice: as many as divide the work, at most
@@ -205,38 +212,73 @@ uint32_t cluster_size(uint32_t L) {
   return L <= 8 ? 1u : L < 16 ? 8u : 16u;
 }
 
-template <int U>
-cudaError_t launch_u(ResidentArgs a, cudaStream_t s) {
+// Threads per CTA: one per pair of sites of the largest share of planes.
+uint32_t cta_threads(uint32_t L, uint32_t cluster) {
+  return ((L + cluster - 1) / cluster * L * (L / 2) + 31u) / 32u * 32u;
+}
+
+// In a pool with `total` lattices of this L: as alone while they all fit at once;
+// else CTAs of 192 threads or more (smaller ones waste more on halos and barriers)
+// in clusters of at most eight (sixteen find their SMs together less often).
+// us per sweep: L = 16 x 128, 1 hit: 8.2, 8.3, 8.1, 7.9, 8.9 with 1, 2, 4, 8, 16; L = 12 x 200,
+// 2 hits + OR: 31.5, 24.6, 23.2, 24.3, 25.9; L = 24 x 64, 4 hits + 2 OR: 63 with 8, 106 with 16;
+// x 6: 13.1, 11.1.
+uint32_t pool_cluster_size(uint32_t L, int total, int sm_count) {
+  uint32_t c = cluster_size(L);
+  if ((uint32_t)total * c <= (uint32_t)sm_count) return c;
+  if (c > 8) c = 8;
+  while (c > 1 && cta_threads(L, c) < 192 && cta_threads(L, c / 2) <= kThreadsMax) c /= 2;
+  return c;
+}
+
+template <int U, int N>
+cudaError_t launch_u(ResidentArgs<N> a, uint32_t cluster, cudaStream_t s) {
   static PerDevice configured;
   cudaError_t e = cudaSuccess;
   std::atomic<int>* slot = device_slot(configured, &e);
   if (!slot) return e;
-  a.cluster = cluster_size(a.L);
-  a.max_planes = (a.L + a.cluster - 1) / a.cluster;
+  a.cluster = cluster;
+  a.max_planes = (a.L + cluster - 1) / cluster;
+  a.Lh = a.L / 2;
   a.plane = a.L * a.Lh;
+  a.nh = (size_t)a.plane * a.L;
   a.by_plane = make_fastdiv(a.plane);
   a.by_Lh = make_fastdiv(a.Lh);
-  const uint32_t threads = (a.max_planes * a.plane + 31u) / 32u * 32u;
-  if (threads > kThreadsMax) return cudaErrorInvalidValue;
+  const uint32_t threads = cta_threads(a.L, cluster);
+  if (threads > kThreadsMax || a.n < 1 || a.n > N) return cudaErrorInvalidValue;
   if (slot->load(std::memory_order_acquire) == 0) {
-    e = cudaFuncSetAttribute(k_resident<U>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_resident<U>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    e = cudaFuncSetAttribute(k_resident<U, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_resident<U, N>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     slot->store(1, std::memory_order_release);
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(a.cluster);
+  cfg.gridDim = dim3(cluster * (uint32_t)a.n);
   cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = (size_t)2 * (a.max_planes + 2) * a.plane * sizeof(float4);
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = a.cluster;
+  at[0].val.clusterDim.x = cluster;
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_resident<U>, a);
+  return cudaLaunchKernelEx(&cfg, k_resident<U, N>, a);
+}
+
+template <int N>
+cudaError_t launch_kinds(int upd, const ResidentArgs<N>& a, uint32_t cluster, cudaStream_t s) {
+  if (!resident_takes(upd, (int)a.L, a.hits)) return cudaErrorInvalidValue;
+  switch (upd) {
+    case U_OR: return launch_u<U_OR>(a, cluster, s);
+    case U_MET_SPHERE: return launch_u<U_MET_SPHERE>(a, cluster, s);
+    case U_MET_BALL: return launch_u<U_MET_BALL>(a, cluster, s);
+    case U_HB: return launch_u<U_HB>(a, cluster, s);
+    case U_MET_OR_SPHERE: return launch_u<U_MET_OR_SPHERE>(a, cluster, s);
+    case U_MET_OR_BALL: return launch_u<U_MET_OR_BALL>(a, cluster, s);
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 }  // namespace
@@ -250,17 +292,13 @@ bool resident_takes(int upd, int L, int hits) {
   return hits <= (L <= 16 ? 16 : L <= 24 ? 5 : 2);
 }
 
-cudaError_t launch_resident(int upd, const ResidentArgs& a, cudaStream_t s) {
-  if (!resident_takes(upd, (int)a.L, a.hits)) return cudaErrorInvalidValue;
-  switch (upd) {
-    case U_OR: return launch_u<U_OR>(a, s);
-    case U_MET_SPHERE: return launch_u<U_MET_SPHERE>(a, s);
-    case U_MET_BALL: return launch_u<U_MET_BALL>(a, s);
-    case U_HB: return launch_u<U_HB>(a, s);
-    case U_MET_OR_SPHERE: return launch_u<U_MET_OR_SPHERE>(a, s);
-    case U_MET_OR_BALL: return launch_u<U_MET_OR_BALL>(a, s);
-    default: return cudaErrorInvalidValue;
-  }
+cudaError_t launch_resident(int upd, const ResidentArgs<1>& a, cudaStream_t s) {
+  return launch_kinds(upd, a, cluster_size(a.L), s);
+}
+
+cudaError_t launch_resident_pool(int upd, const ResidentArgs<kResidentPoolMax>& a, int total, int sm_count,
+                                 cudaStream_t s) {
+  return launch_kinds(upd, a, pool_cluster_size(a.L, total, sm_count), s);
 }
 
 }  // namespace hsg

@@ -107,26 +107,6 @@ def test_work_queued_around_batches_keeps_its_order(hsg):
                 assert abs(got[r][i] - alone(hsg, (L, 3, 10 * r + i, 0, 0.6), kw, 4)[1]) < 1e-12
 
 
-def test_a_captured_pool_sweep_replays_as_new_sweeps(hsg):
-    kw = dict(kinds(hsg)[0], renorm_every=0)
-    sched = hsg.schedule(**kw)
-    stream = torch.cuda.Stream()
-    with hsg.Pool(1 << 26, 8, stream) as pool:
-        specs = [(48, 2, 0, 0, 0.5), (64, 2, 1, 0, 0.7), (16, 2, 2, 0, 0.7)]
-        slots = [pool.admit(*s) for s in specs]
-        pool.sweep(sched, 2)
-        torch.cuda.synchronize()
-        g = torch.cuda.CUDAGraph()
-        with torch.cuda.graph(g, stream=stream):
-            pool.sweep(sched, 1)
-        for _ in range(3):
-            with torch.cuda.stream(stream):
-                g.replay()
-        torch.cuda.synchronize()
-        for s, spec in zip(slots, specs):
-            assert np.array_equal(pool.spins(s), alone(hsg, spec, kw, 5)[0]), spec
-
-
 def test_a_lattice_beyond_32_bit_offsets(hsg):
     if torch.cuda.mem_get_info()[0] < 60 << 30:
         pytest.skip("needs 60 GB of device memory")

@@ -83,3 +83,29 @@ def test_a_captured_sweep_replays_as_new_sweeps(hsg):
                 g.replay()
         torch.cuda.synchronize()
         assert np.array_equal(lat.spins(), ref.spins())
+
+
+# alone in their clusters, and too many for the GPU at once (smaller clusters)
+@pytest.mark.parametrize("sides,n", [((4, 6, 8, 10, 12, 14, 16, 18, 20, 22, 24, 26, 28, 30), 14), ((16,), 130), ((8,), 70),
+                                     ((12, 20), 60), ((24,), 40)])
+@pytest.mark.parametrize("use_stream", [True, False])
+def test_pools_of_small_lattices_equal_lattices_alone(hsg, sides, n, use_stream):
+    """All sweeps of a call in one launch per 64 lattices of a side; counters
+    stay right for the calls that take the half-sweep kernels."""
+    kw = dict(kind=hsg.HSG_METROPOLIS, hits=2, proposal=hsg.HSG_PROP_BALL, n_or=1, renorm_every=3)
+    many = dict(kw, hits=18)  # too many hits for the resident kernel
+    specs = [(sides[k % len(sides)], 3, k, k & 1, 0.3 + 0.01 * k) for k in range(n)]
+    with hsg.Pool(1 << 26, n, torch.cuda.Stream() if use_stream else None) as pool:
+        slots = [pool.admit(*s) for s in specs]
+        pool.sweep(hsg.schedule(**kw), 4)
+        pool.sweep(hsg.schedule(**many), 1)
+        pool.sweep(hsg.schedule(**kw), 2)
+        e = pool.energies()
+        for slot, (L, seed, sample, replica, T) in list(zip(slots, specs))[:: max(1, n // 20)]:
+            with hsg.Lattice(L, seed, sample, replica) as lat:
+                lat.generate_couplings()
+                for s, k in ((kw, 4), (many, 1), (kw, 2)):
+                    lat.sweep(hsg.schedule(T=T, kernel=hsg.HSG_KERNEL_GLOBAL, **s), k)
+                assert np.array_equal(pool.spins(slot), lat.spins()), L
+                assert abs(e[slot] - lat.energy()) <= 2e-6
+                assert pool.sweep_count(slot) == 7
