@@ -226,7 +226,7 @@ uint32_t cta_threads(uint32_t L, uint32_t cluster) {
 uint32_t pool_cluster_size(uint32_t L, int total, int sm_count) {
   uint32_t c = cluster_size(L);
   if ((uint32_t)total * c <= (uint32_t)sm_count) return c;
-  if (c > 8) c = 8;
+  if (c > 8 && cta_threads(L, 8) <= kThreadsMax) c = 8;  // from L = 26 sixteen are needed
   while (c > 1 && cta_threads(L, c) < 192 && cta_threads(L, c / 2) <= kThreadsMax) c /= 2;
   return c;
 }
