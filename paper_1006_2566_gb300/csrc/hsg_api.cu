@@ -26,6 +26,7 @@ constexpr int kMaxL = 1624;    // L^3 < 2^32: site indices are 32-bit Philox cou
 constexpr int kElogInit = 64;
 constexpr int kCounters = 4;   // words at hsg_ctx::d_ctr
 constexpr long long kMaxGraphPeriod = 64;  // longest sweep period captured as one graph
+constexpr int kGraphSweeps = 16;           // sweeps in one graph without cadences
 
 thread_local std::string g_thread_error;
 int g_fail_alloc_countdown = 0;  // test hook: k-th allocation from now fails
@@ -85,6 +86,9 @@ struct hsg_ctx {
   hsg_schedule gsched{};
   int gvariant = 0, gperiod = 0, glaunches = 0;
   double* gelog = nullptr;
+  // While a period is captured: the sweep's number in it (the counter kernel
+  // then runs once, at the period's end); -1 otherwise.
+  int captured = -1;
   float4* gspins = nullptr;  // current spin buffer when the period was captured
   std::string err;
 };
@@ -208,6 +212,7 @@ void release(hsg_ctx* c) {
 
 hsg::SweepArgs sweep_args(hsg_ctx* c, int colour, float beta, float step, int hits) {
   hsg::SweepArgs a{};
+  a.sweep_add = c->captured > 0 ? (uint32_t)c->captured : 0u;
   const int o = 1 - colour;
   a.own = c->spins + colour * c->Nh;
   a.oth = c->spins + o * c->Nh;
@@ -227,7 +232,7 @@ hsg::SweepArgs sweep_args(hsg_ctx* c, int colour, float beta, float step, int hi
   a.sweep_hi = (uint32_t)(c->sweep >> 32);
   a.beta = beta;
   a.step = step;
-  a.sweep_ptr = c->d_ctr;  // the device counter equals c->sweep in stream order
+  a.sweep_ptr = c->d_ctr;  // the device counter (plus sweep_add) equals c->sweep in stream order
   if (c->packed) {
     float* base = reinterpret_cast<float*>(c->spins);
     a.own = reinterpret_cast<float4*>(base + 3 * colour * c->Nh);
@@ -390,8 +395,9 @@ hsg_status run_energy(hsg_ctx* c, bool logged) {
   return launch(c, HSG_PROF_ENERGY, logged ? 2 : 1, "energy kernel", [&] { return hsg::launch_energy(a, c->stream); });
 }
 
-hsg_status run_advance(hsg_ctx* c) {
-  return launch(c, HSG_PROF_LAYOUT, 1, "counter kernel", [&] { return hsg::launch_add_u64(c->d_ctr, 1, c->stream); });
+hsg_status run_advance(hsg_ctx* c, uint64_t sweeps) {
+  return launch(c, HSG_PROF_LAYOUT, 1, "counter kernel",
+                [&] { return hsg::launch_add_u64(c->d_ctr, sweeps, c->stream); });
 }
 
 hsg_status run_renorm(hsg_ctx* c) {
@@ -420,7 +426,7 @@ hsg_status enqueue_one_sweep(hsg_ctx* c, const hsg_schedule* s) {
     for (int colour = 0; colour < 2; ++colour)
       if ((st = run_half_sweep(c, s, HSG_OVERRELAX, colour)) != HSG_OK) return st;
   }
-  if ((st = run_advance(c)) != HSG_OK) return st;
+  if (c->captured < 0 && (st = run_advance(c, 1)) != HSG_OK) return st;
   c->sweep += 1;
   if (renorm_due && !fuse_renorm)
     if ((st = run_renorm(c)) != HSG_OK) return st;
@@ -441,8 +447,23 @@ bool graph_matches(const hsg_ctx* c, const hsg_schedule* s, int variant, int per
          c->gelog == c->elog && c->gspins == c->spins;
 }
 
-// Capture `period` sweeps starting at the current counter (a multiple of
-// the period) into c->gexec.  Capturing runs nothing, so the host mirrors
+// Sweeps in one graph for a schedule without cadences, n of them asked for:
+// the largest divisor of n up to kGraphSweeps (a multiple of `unit`), or
+// kGraphSweeps if none is half as long; a graph that is there is kept unless
+// eight of it would be replayed.
+int free_period(const hsg_ctx* c, const hsg_schedule* s, int variant, int n, int unit) {
+  if (c->gexec && graph_matches(c, s, variant, c->gperiod) && c->gperiod % unit == 0 &&
+      (c->gperiod >= kGraphSweeps / 2 || n < 8 * c->gperiod))
+    return c->gperiod;
+  if (n < 2 * unit) return unit;
+  int best = unit;
+  for (int d = unit; d <= kGraphSweeps && d <= n; d += unit)
+    if (n % d == 0) best = d;
+  return best >= kGraphSweeps / 2 || n <= kGraphSweeps ? (n <= kGraphSweeps ? n / unit * unit : best) : kGraphSweeps;
+}
+
+// Capture `period` sweeps starting at the current counter (with cadences a
+// multiple of the period) into c->gexec.  Capturing runs nothing, so the host mirrors
 // are restored afterwards.
 hsg_status capture_period(hsg_ctx* c, const hsg_schedule* s, int variant, int period) {
   if (c->gexec) cudaGraphExecDestroy(c->gexec);
@@ -454,7 +475,12 @@ hsg_status capture_period(hsg_ctx* c, const hsg_schedule* s, int variant, int pe
   cudaError_t e = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return cuda_fail(c, e, "sweep capture");
   hsg_status st = HSG_OK;
-  for (int j = 0; j < period && st == HSG_OK; ++j) st = enqueue_one_sweep(c, s);
+  for (int j = 0; j < period && st == HSG_OK; ++j) {
+    c->captured = j;
+    st = enqueue_one_sweep(c, s);
+  }
+  c->captured = -1;
+  if (st == HSG_OK) st = run_advance(c, (uint64_t)period);
   cudaGraph_t g = nullptr;
   e = cudaStreamEndCapture(c->stream, &g);
   c->glaunches = (int)(c->launches - launches0);
@@ -737,22 +763,25 @@ hsg_status hsg_sweep(hsg_ctx* c, const hsg_schedule* s, int n_sweeps) {
   }
   if (swaps > 0 && (st = prepare_bond_boxes(c)) != HSG_OK) return st;
   SweepGroup group_guard(c);
-  // Sweeps run in periods of P = lcm(renorm_every, energy_every) sweeps
-  // (1 without cadences).  On a non-default stream and without the
+  // Sweeps run in periods of P = lcm(renorm_every, energy_every) sweeps.  On a non-default stream and without the
   // profiler, a period that starts at a multiple of P is captured once as a
   // CUDA graph (the kernels read the sweep counter and the energy-log
   // position from device memory) and replayed; other sweeps are launched
   // directly.  Both paths issue the same kernels in the same order.  A
   // captured period leaves the spins in the buffer it found them in (an even
-  // number of buffer swaps), so that the graph can be replayed.
+  // number of buffer swaps), so that the graph can be replayed.  Without
+  // cadences the period is as many sweeps as one graph is given: a graph of
+  // one sweep costs 4-8 us of launching each.
+  const bool cadence = s->renorm_every > 0 || s->energy_every > 0;
   long long period = 1;
   if (s->renorm_every > 0) period = std::lcm(period, (long long)s->renorm_every);
   if (s->energy_every > 0) period = std::lcm(period, (long long)s->energy_every);
   if ((period * swaps) % 2 == 1) period *= 2;
+  if (!cadence && n_sweeps > 0) period = free_period(c, s, variant, n_sweeps, (int)period);
   const bool graphs = c->stream != nullptr && !c->prof && period <= kMaxGraphPeriod;
   int k = 0;
   while (k < n_sweeps) {
-    if (graphs && c->sweep % (uint64_t)period == 0 && n_sweeps - k >= period) {
+    if (graphs && (!cadence || c->sweep % (uint64_t)period == 0) && n_sweeps - k >= period) {
       if (!graph_matches(c, s, variant, (int)period) && (st = capture_period(c, s, variant, (int)period)) != HSG_OK)
         return st;
       cudaError_t e = cudaGraphLaunch(c->gexec, c->stream);

@@ -96,9 +96,11 @@ struct SweepArgs {
   int L, Lh, colour, hits;
   uint32_t k0, k1, sweep_lo, sweep_hi;
   float beta, step;
-  // When set, the sweep counter is read from this device word instead of
-  // sweep_lo/sweep_hi (so that a captured graph can be replayed).
+  // When set, the sweep counter is this device word plus sweep_add instead of
+  // sweep_lo/sweep_hi (so that a captured graph can be replayed; sweep_add is
+  // the sweep's number in the captured period).
   const unsigned long long* sweep_ptr;
+  uint32_t sweep_add;
   // Packed layout: own / oth are then component-0 arrays of three fp32
   // arrays `stride` floats apart (global kernel only).
   bool packed;

@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(G_THREADS, MIN_BLOCKS)
   DrawArgs d{a.sweep_lo, a.sweep_hi, a.k0, a.k1, a.beta, a.step, a.hits, 0};
   if constexpr (U != U_OR) {
     if (a.sweep_ptr) {
-      const unsigned long long sw = *a.sweep_ptr;
+      const unsigned long long sw = *a.sweep_ptr + a.sweep_add;
       d.sweep_lo = (uint32_t)sw;
       d.sweep_hi = (uint32_t)(sw >> 32);
     }
@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(G_THREADS, 12) k_half_sweep_column(const Sweep
   if (xh >= Lh || y >= L) return;
   uint32_t sweep_lo = a.sweep_lo, sweep_hi = a.sweep_hi;
   if (a.sweep_ptr) {
-    const unsigned long long sw = *a.sweep_ptr;
+    const unsigned long long sw = *a.sweep_ptr + a.sweep_add;
     sweep_lo = (uint32_t)sw;
     sweep_hi = (uint32_t)(sw >> 32);
   }
@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(TX* SLAB_TY, slab_min_blocks<U>()) k_half_swee
   uint32_t sweep_lo = a.sweep_lo, sweep_hi = a.sweep_hi;
   if constexpr (U != U_OR) {
     if (a.sweep_ptr) {
-      const unsigned long long sw = *a.sweep_ptr;
+      const unsigned long long sw = *a.sweep_ptr + a.sweep_add;
       sweep_lo = (uint32_t)sw;
       sweep_hi = (uint32_t)(sw >> 32);
     }

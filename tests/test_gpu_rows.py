@@ -86,3 +86,29 @@ def test_overlapping_launches_equal_the_slab_kernel(hsg, L, use_stream):
                 outs.append((lat.spins(), lat.energy_log(), lat.energy()))
         for o in outs[1:]:
             assert all(np.array_equal(a, b) for a, b in zip(o, outs[0]))
+
+
+@pytest.mark.parametrize("kernel,n_or", [(1, 2), (3, 1), (3, 2)])
+def test_graphs_without_cadences_equal_direct_launches(hsg, kernel, n_or):
+    """Without cadences a graph holds as many sweeps as one call's number
+    allows: calls of other lengths, a change of schedule, new spins and a
+    counter set by hand in between."""
+    L = 40
+    outs = []
+    for stream in (torch.cuda.Stream(), None):
+        with hsg.Lattice(L, 13, stream=stream) as lat:
+            lat.generate_couplings()
+            sched = hsg.schedule(kind=hsg.HSG_HEATBATH, T=0.6, n_or=n_or, kernel=kernel)
+            other = hsg.schedule(kind=hsg.HSG_METROPOLIS, T=0.6, n_or=1, kernel=kernel)
+            got = []
+            for n, sc in ((1, sched), (5, sched), (5, sched), (3, sched), (50, sched), (20, other), (2, sched), (17, sched),
+                          (33, sched), (7, other), (7, other)):
+                lat.sweep(sc, n)
+                got.append((lat.energy(), lat.sweep_count))
+            lat.sweep_count = 2 ** 32 - 5
+            lat.sweep(sched, 12)
+            lat.set_spins(lat.spins()[::-1].copy())
+            lat.sweep(sched, 12)
+            outs.append((got, lat.sweep_count, lat.spins()))
+    assert outs[0][0] == outs[1][0] and outs[0][1] == outs[1][1]
+    assert np.array_equal(outs[0][2], outs[1][2])
