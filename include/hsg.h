@@ -86,7 +86,7 @@ enum {
                           * an energy in one launch where the lattice is small (L <=
                           * 32, few hits): the same results */
   HSG_KERNEL_GLOBAL = 1, /* one thread per one to four sites of a column, neighbours through L1/L2 (heat-bath from
-                          * L = 224: one thread per six-plane column, carrying its column's
+                          * L = 152: one thread per six-plane column, carrying its column's
                           * neighbours; the same results) */
   HSG_KERNEL_SLAB = 2,   /* z-marching tiles: other colour staged in shared memory */
   /* Temporally blocked over-relaxation: each over-relaxation sweep

@@ -40,7 +40,7 @@ __device__ __forceinline__ uint32_t site_number(int xh, int p, int y, int z, int
 //   L = 128  7.94 -> 6.66, 20.7 -> 20.5, 15.1 -> 12.3 us
 //   L = 130  11.0 -> 7.9, 32.8 -> 22.6, 17.5 -> 13.3 us
 //   L = 256  85.0 -> 83.5, 160.6 -> 154.4 us; heat-bath stays with the column
-//            kernel (93.2 us; 95.8 with two rows per thread)
+//            kernel (86.5 us; 95.8 with two rows per thread)
 //   packed, L = 130: 12.1 -> 7.7, 35.7 -> 23.6, 21.4 -> 13.9 us; L = 256: 89.6 ->
 //            84.3, 170.6 -> 165, 102.9 -> 94.1 us
 // Rows per thread (row_shape below): the own-column neighbour of one row is
@@ -110,12 +110,14 @@ __global__ void __launch_bounds__(G_THREADS, MIN_BLOCKS)
 // flushed); 32 x 4, 128 x 1, 8 x 16 and 256-thread blocks 89.9-91.1 us;
 // streaming (evict-first) stores of the new spins gained 0.2 us more.
 constexpr int ZM_PLANES = 6;
-// From here on the column march wins: 93.2 against 95.8 us at L = 256; below,
-// the rows kernel does (L = 192 43.6 against 43.2 us, L = 128 15.1 against 12.3,
-// L = 64 5.4 against 3.1 us: six planes per thread are too few threads).
-constexpr int ZM_MIN_L = 224;
+// 32-bit byte offsets up to L = 812: 86.5 against 88.6 us at L = 256, 40.8 against
+// 41.5 at L = 192.  From ZM_MIN_L on the column march wins over the rows kernel
+// (L = 160 23.9 against 25.9 us, 192 40.8 / 41.8, 222 60.2 / 63.9); below, six planes
+// per thread are too few threads (L = 128 13.8 against 12.4, L = 64 5.4 against 3.1).
+constexpr int ZM_MIN_L = 152;
 constexpr int ZM_BX = 16, ZM_BY = 8;
 
+template <class Off>
 __global__ void __launch_bounds__(G_THREADS, 12) k_half_sweep_column(const SweepArgs a) {
   const uint32_t xh = blockIdx.x * blockDim.x + threadIdx.x;
   const uint32_t y = blockIdx.y * blockDim.y + threadIdx.y;
@@ -135,30 +137,30 @@ __global__ void __launch_bounds__(G_THREADS, 12) k_half_sweep_column(const Sweep
   const uint32_t xm1 = xh == 0 ? Lh - 1 : xh - 1, xp1 = xh + 1 == Lh ? 0u : xh + 1;
   const float4* __restrict__ oth = a.oth;
   uint32_t zmo = (z0 == 0 ? L - 1 : z0 - 1) * plane, zo = z0 * plane;
-  float4 s_m = __ldg(oth + zmo + row + xh), s_0 = __ldg(oth + zo + row + xh);
+  float4 s_m = __ldg(elem<Off>(oth, zmo + row + xh)), s_0 = __ldg(elem<Off>(oth, zo + row + xh));
   for (uint32_t z = z0; z < z1; ++z) {
     const uint32_t zpo = z + 1 == L ? 0u : zo + plane;
     const uint32_t p = ((uint32_t)a.colour + y + z) & 1u;  // x = 2 xh + p
     const uint32_t q = zo + row + xh;
-    const float4 s_p = __ldg(oth + zpo + row + xh);
-    const float4 side = __ldg(oth + zo + row + (p ? xp1 : xm1));
+    const float4 s_p = __ldg(elem<Off>(oth, zpo + row + xh));
+    const float4 side = __ldg(elem<Off>(oth, zo + row + (p ? xp1 : xm1)));
     SiteInputs in;
     in.sxp = p ? side : s_0;
     in.sxm = p ? s_0 : side;
-    in.syp = __ldg(oth + zo + row_p + xh);
-    in.sym = __ldg(oth + zo + row_m + xh);
+    in.syp = __ldg(elem<Off>(oth, zo + row_p + xh));
+    in.sym = __ldg(elem<Off>(oth, zo + row_m + xh));
     in.szp = s_p;
     in.szm = s_m;
-    in.jxp = __ldg(a.jx_own + q);
-    in.jxm = __ldg(a.jx_oth + (p ? q : zo + row + xm1));
-    in.jyp = __ldg(a.jy_own + q);
-    in.jym = __ldg(a.jy_oth + zo + row_m + xh);
-    in.jzp = __ldg(a.jz_own + q);
-    in.jzm = __ldg(a.jz_oth + zmo + row + xh);
+    in.jxp = __ldg(elem<Off>(a.jx_own, q));
+    in.jxm = __ldg(elem<Off>(a.jx_oth, p ? q : zo + row + xm1));
+    in.jyp = __ldg(elem<Off>(a.jy_own, q));
+    in.jym = __ldg(elem<Off>(a.jy_oth, zo + row_m + xh));
+    in.jzp = __ldg(elem<Off>(a.jz_own, q));
+    in.jzm = __ldg(elem<Off>(a.jz_oth, zmo + row + xh));
     in.s = make_float3(0.0f, 0.0f, 0.0f);  // the heat-bath does not read the old spin
     in.q = q;
     in.site = (2 * xh + p) + y * L + z * L * L;
-    a.own[q] = site_result<U_HB>(in, (uint32_t)a.colour, sweep_lo, sweep_hi, a.k0, a.k1, a.beta, a.step, a.hits);
+    *elem<Off>(a.own, q) = site_result<U_HB>(in, (uint32_t)a.colour, sweep_lo, sweep_hi, a.k0, a.k1, a.beta, a.step, a.hits);
     s_m = s_0;
     s_0 = s_p;
     zmo = zo;
@@ -358,7 +360,10 @@ cudaError_t launch_kind(int variant, const SweepArgs& a, int sm_count, cudaStrea
   if constexpr (U == U_HB) {
     if (a.L >= ZM_MIN_L) {
       const dim3 grid(cdiv(a.Lh, ZM_BX), cdiv(a.L, ZM_BY), cdiv(a.L, ZM_PLANES));
-      k_half_sweep_column<<<grid, dim3(ZM_BX, ZM_BY), 0, s>>>(a);
+      if (a.L > kMaxOff32L)
+        k_half_sweep_column<unsigned long long><<<grid, dim3(ZM_BX, ZM_BY), 0, s>>>(a);
+      else
+        k_half_sweep_column<uint32_t><<<grid, dim3(ZM_BX, ZM_BY), 0, s>>>(a);
       return cudaGetLastError();
     }
   }
