@@ -533,7 +533,7 @@ hsg_status run_resident(hsg_ctx* c, const hsg_schedule* s, int n_sweeps) {
   for (int k = 0; k < n_sweeps;) {
     uint64_t m = (uint64_t)(n_sweeps - k);
     if (s->energy_every > 0) m = std::min(m, (uint64_t)s->energy_every - c->sweep % (uint64_t)s->energy_every);
-    hsg::ResidentArgs<1> a{};
+    hsg::ResidentArgs a{};
     a.L = (uint32_t)c->L;
     a.packed = c->packed;
     a.sweeps = (uint32_t)m;
@@ -543,8 +543,12 @@ hsg_status run_resident(hsg_ctx* c, const hsg_schedule* s, int n_sweeps) {
     a.hits = s->hits;
     a.sweep_ptr = c->d_ctr;
     a.n = 1;
-    a.lat[0] = {c->spins, c->J, 0, c->k0, c->k1, beta_of(s->T)};
-    st = launch(c, HSG_PROF_LAYOUT, 1, "resident sweeps kernel", [&] { return hsg::launch_resident(upd, a, c->stream); });
+    a.spins = c->spins;
+    a.J = c->J;
+    a.k0 = c->k0;
+    a.k1 = c->k1;
+    a.beta = beta_of(s->T);
+    st = launch(c, HSG_PROF_LAYOUT, 1, "resident sweeps kernel", [&] { return hsg::launch_resident(upd, a, c->sm_count, c->stream); });
     if (st != HSG_OK) return st;
     c->sweep += m;
     k += (int)m;

@@ -150,15 +150,24 @@ struct FastDiv {
   uint32_t m, s1, s2;
 };
 
-// Sweeps of small lattices in one launch (hsg_resident.cu).
-struct ResidentLattice {
-  float4* spins;    // S[2][N/2] (packed: [2][3][N/2] floats), read and written back
-  const float* J;   // J[3][2][N/2]
-  unsigned long long sweep;  // sweep counter (a pool's; a context's is on the device)
-  uint32_t k0, k1;
-  float beta;
+// One slot of a pool as the kernels see it (96 bytes).
+struct PoolDesc {
+  uint32_t L, Lh, nh, plane;          // side, side/2, sites per colour, per colour-plane
+  uint32_t k0, k1;                    // Philox key of (seed, sample, replica)
+  uint32_t sweep_lo, sweep_hi;        // the lattice's own sweep counter
+  float beta;                         // 1/T (0 for T = inf)
+  uint32_t active;                    // 1 while admitted
+  uint32_t tile_begin, tile_count;    // the slot's tiles in the work list
+  unsigned long long spin_off;        // float4 offset of colour 0 (colour 1 at + nh)
+  unsigned long long j_off;           // float offset of J[0][0] (J[d][c] at + (2d + c) nh)
+  FastDiv by_plane, by_lh;            // division of a site index by plane and by Lh
+  uint32_t pad[2];
 };
-template <int N>
+static_assert(sizeof(PoolDesc) == 96, "PoolDesc layout");
+
+// Sweeps of small lattices of one side in one launch (hsg_resident.cu): a
+// context's, given here, or n slots of a pool (slots not NULL), whose sweep
+// counters are read and not advanced.
 struct ResidentArgs {
   uint32_t L;
   bool packed;
@@ -166,25 +175,27 @@ struct ResidentArgs {
   uint32_t per_sweep;     // half-sweeps of a sweep, the main update's two first
   uint32_t renorm_every;  // 0 = never
   float step;
-  int hits;
-  unsigned long long* sweep_ptr;  // N = 1: the lattice's counter on the device, advanced by `sweeps`
-  int n;                          // lattices
-  ResidentLattice lat[N];
+  int hits, n;
+  float4* spins;   // S[2][N/2] (packed: [2][3][N/2] floats), read and written back
+  const float* J;  // J[3][2][N/2]
+  uint32_t k0, k1;
+  float beta;
+  unsigned long long* sweep_ptr;  // device sweep counter, advanced by `sweeps`
+  const PoolDesc* desc;
+  const uint32_t* slots;
+  char* arena;
   // set by the launcher
   size_t nh;
   uint32_t cluster, max_planes, Lh, plane;
   FastDiv by_plane, by_Lh;
 };
 constexpr int kResidentMaxL = 32;
-constexpr int kResidentPoolMax = 64;  // lattices of one L in one launch: 2.6 KB of parameters
-// Sites of a pool's small lattices up to which it takes them so.
+// Sites of a pool's small lattices up to which it takes them so (those from
+// L = 26 counted a quarter more).
 constexpr unsigned long long kResidentPoolSites = 640 * 1024;
 // `upd`: the main update's kind, or U_OR for over-relaxation only.
 bool resident_takes(int upd, int L, int hits);
-cudaError_t launch_resident(int upd, const ResidentArgs<1>& a, cudaStream_t s);
-// For a pool, whose `total` lattices of this L go in several such launches.
-cudaError_t launch_resident_pool(int upd, const ResidentArgs<kResidentPoolMax>& a, int total, int sm_count,
-                                 cudaStream_t s);
+cudaError_t launch_resident(int upd, const ResidentArgs& a, int sm_count, cudaStream_t s);
 
 // A batch of pool lattices swept by one launch per half-sweep (hsg_batch.cu),
 // handed over as kernel parameters.

@@ -31,24 +31,8 @@
 
 namespace {
 
-// One slot as the kernels see it (96 bytes).
-struct PoolDesc {
-  uint32_t L, Lh, nh, plane;          // side, side/2, sites per colour, per colour-plane
-  uint32_t k0, k1;                    // Philox key of (seed, sample, replica)
-  uint32_t sweep_lo, sweep_hi;        // the lattice's own sweep counter
-  float beta;                         // 1/T (0 for T = inf)
-  uint32_t active;                    // 1 while admitted
-  uint32_t tile_begin, tile_count;    // the slot's tiles in the work list
-  unsigned long long spin_off;        // float4 offset of colour 0 (colour 1 at + nh)
-  unsigned long long j_off;           // float offset of J[0][0] (J[d][c] at + (2d + c) nh)
-  hsg::FastDiv by_plane, by_lh;       // division of a site index by plane and by Lh
-  uint32_t pad[2];
-};
-static_assert(sizeof(PoolDesc) == 96, "PoolDesc layout");
-
-
 // Site index q -> (xh, y, z) of a slot.
-__device__ __forceinline__ void decode_site(const PoolDesc* d, uint32_t q, uint32_t& xh, uint32_t& y, uint32_t& z) {
+__device__ __forceinline__ void decode_site(const hsg::PoolDesc* d, uint32_t q, uint32_t& xh, uint32_t& y, uint32_t& z) {
   z = hsg::fast_div(q, d->by_plane);
   const uint32_t r = q - z * d->plane;
   y = hsg::fast_div(r, d->by_lh);
@@ -70,7 +54,7 @@ inline unsigned cdiv_u(unsigned long long a, unsigned long long b) { return (uns
 // two sites per thread, 243 us at 56 registers and one), and the Metropolis
 // pass runs fastest at the 64 registers its code wants.
 template <int U>
-__global__ void __launch_bounds__(256, 4) k_pool_half_sweep(const PoolDesc* __restrict__ desc,
+__global__ void __launch_bounds__(256, 4) k_pool_half_sweep(const hsg::PoolDesc* __restrict__ desc,
                                                          const uint2* __restrict__ tiles,
                                                          const uint32_t* __restrict__ n_tiles, float4* __restrict__ S,
                                                          const float* __restrict__ J, uint32_t colour, float step,
@@ -78,7 +62,7 @@ __global__ void __launch_bounds__(256, 4) k_pool_half_sweep(const PoolDesc* __re
   const uint32_t nt = *n_tiles;
   for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) {
     const uint2 tl = tiles[t];
-    const PoolDesc* d = desc + tl.x;
+    const hsg::PoolDesc* d = desc + tl.x;
     const uint32_t L = d->L, Lh = d->Lh, nh = d->nh;
     float4* base = S + d->spin_off;
     float4* own = base + (colour ? nh : 0);
@@ -101,7 +85,7 @@ __global__ void __launch_bounds__(256, 4) k_pool_half_sweep(const PoolDesc* __re
 
 // Counter advance of every active slot by `sweeps`, after the last half-sweep
 // of a sweep (or of all of them).
-__global__ void k_pool_advance(PoolDesc* __restrict__ desc, int n, uint32_t sweeps) {
+__global__ void k_pool_advance(hsg::PoolDesc* __restrict__ desc, int n, uint32_t sweeps) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     if (!desc[i].active) continue;
     const uint32_t lo = desc[i].sweep_lo + sweeps;
@@ -112,13 +96,13 @@ __global__ void k_pool_advance(PoolDesc* __restrict__ desc, int n, uint32_t swee
 
 // Renormalisation of the slots whose counter is a multiple of `every`
 // (the single-lattice rule: after the advance, when sweep % every == 0).
-__global__ void __launch_bounds__(256) k_pool_renorm(const PoolDesc* __restrict__ desc, const uint2* __restrict__ tiles,
+__global__ void __launch_bounds__(256) k_pool_renorm(const hsg::PoolDesc* __restrict__ desc, const uint2* __restrict__ tiles,
                                                      const uint32_t* __restrict__ n_tiles, float4* __restrict__ S,
                                                      uint32_t every, uint32_t tile_sites) {
   const uint32_t nt = *n_tiles;
   for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) {
     const uint2 tl = tiles[t];
-    const PoolDesc* d = desc + tl.x;
+    const hsg::PoolDesc* d = desc + tl.x;
     const unsigned long long sweep = ((unsigned long long)d->sweep_hi << 32) | d->sweep_lo;
     if (sweep % every != 0) continue;
     const uint32_t nh = d->nh;
@@ -155,7 +139,7 @@ __device__ __forceinline__ double block_sum(double v) {
 
 // Energy, first pass: per tile of colour-0 sites, sum of s . h (fp32 per
 // site, fp64 sums), written to partials[tile].
-__global__ void __launch_bounds__(256) k_pool_energy_partial(const PoolDesc* __restrict__ desc,
+__global__ void __launch_bounds__(256) k_pool_energy_partial(const hsg::PoolDesc* __restrict__ desc,
                                                              const uint2* __restrict__ tiles,
                                                              const uint32_t* __restrict__ n_tiles,
                                                              const float4* __restrict__ S, const float* __restrict__ J,
@@ -165,7 +149,7 @@ __global__ void __launch_bounds__(256) k_pool_energy_partial(const PoolDesc* __r
   for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) {
     const uint2 tl = tiles[t];
     if (sel && !sel[tl.x]) continue;  // slot not asked for
-    const PoolDesc* d = desc + tl.x;
+    const hsg::PoolDesc* d = desc + tl.x;
     const uint32_t L = d->L, Lh = d->Lh, nh = d->nh, plane = d->plane;
     const float4* s0 = S + d->spin_off;
     const float4* s1 = s0 + nh;
@@ -197,12 +181,12 @@ __global__ void __launch_bounds__(256) k_pool_energy_partial(const PoolDesc* __r
 
 // Energy, second pass: block per slot adds its tiles' partials in order;
 // E/N = -(sum)/N, NaN for inactive slots.
-__global__ void __launch_bounds__(256) k_pool_energy_final(const PoolDesc* __restrict__ desc, int n_slots,
+__global__ void __launch_bounds__(256) k_pool_energy_final(const hsg::PoolDesc* __restrict__ desc, int n_slots,
                                                            const uint8_t* __restrict__ sel,
                                                            const double* __restrict__ partials,
                                                            double* __restrict__ out) {
   for (int s = blockIdx.x; s < n_slots; s += gridDim.x) {
-    const PoolDesc* d = desc + s;
+    const hsg::PoolDesc* d = desc + s;
     if (!d->active || (sel && !sel[s])) {
       if (threadIdx.x == 0) out[s] = __longlong_as_double(0x7ff8000000000000ll);
       continue;
@@ -237,8 +221,8 @@ struct hsg_pool {
   // Device tables and two pinned host mirrors of each: a rebuild writes
   // the mirror whose last upload has completed (its event), so the host
   // never waits for the sweeps in flight.
-  PoolDesc* d_desc = nullptr;
-  PoolDesc* h_desc = nullptr;  // pinned, 2 x max_slots
+  hsg::PoolDesc* d_desc = nullptr;
+  hsg::PoolDesc* h_desc = nullptr;  // pinned, 2 x max_slots
   uint2* d_tiles = nullptr;
   uint2* h_tiles = nullptr;  // pinned, 2 x tiles_cap
   size_t tiles_cap = 0;
@@ -246,6 +230,11 @@ struct hsg_pool {
   // (word 1): the list holds the lattices of the batches last.
   uint32_t* d_ntiles = nullptr;
   uint32_t* h_ntiles = nullptr;  // pinned, 2 x 2
+  // Slots of the lattices under kBatchMinL, by side from the largest, and how
+  // many of each side: the resident kernel's list.
+  uint32_t* d_small = nullptr;
+  uint32_t* h_small = nullptr;  // pinned, 2 x max_slots
+  int small_count[hsg::kBatchMinL] = {};
   // Sweeping of the large lattices in batches (hsg_batch.cu): whether the
   // admitted lattices ask for it (set with the tables), whether others are left
   // to the persistent kernels, and the streams beside the pool's own, made on first use.
@@ -380,7 +369,7 @@ hsg_status sync_tables(hsg_pool* p) {
       return pcuda(p, e, "pool work list");
     p->tiles_cap = cap;
   }
-  PoolDesc* h_desc = p->h_desc + (size_t)b * p->max_slots;
+  hsg::PoolDesc* h_desc = p->h_desc + (size_t)b * p->max_slots;
   uint2* h_tiles = p->h_tiles + (size_t)b * p->tiles_cap;
   uint32_t* h_ntiles = p->h_ntiles + 2 * b;
   uint64_t large_sites = 0;
@@ -392,7 +381,7 @@ hsg_status sync_tables(hsg_pool* p) {
   for (int pass = 0; pass < 2; ++pass) {
     for (int i = 0; i < p->max_slots; ++i) {
       const Slot& s = p->slots[i];
-      PoolDesc& d = h_desc[i];
+      hsg::PoolDesc& d = h_desc[i];
       if (s.active && (p->batched && s.L >= hsg::kBatchMinL) != (pass == 1)) continue;
       memset(&d, 0, sizeof(d));
       if (!s.active) continue;
@@ -418,8 +407,19 @@ hsg_status sync_tables(hsg_pool* p) {
     h_ntiles[pass] = nt;
   }
   p->unbatched_left = h_ntiles[0] > 0;
-  if ((e = cudaMemcpyAsync(p->d_desc, h_desc, sizeof(PoolDesc) * p->max_slots, cudaMemcpyHostToDevice,
+  uint32_t* h_small = p->h_small + (size_t)b * p->max_slots;
+  uint32_t ns = 0;
+  std::fill(std::begin(p->small_count), std::end(p->small_count), 0);
+  for (const Slot& s : p->slots)
+    if (s.active && s.L < hsg::kBatchMinL) p->small_count[s.L] += 1;
+  for (int L = hsg::kBatchMinL - 2; L >= 4; L -= 2)
+    if (p->small_count[L] > 0)
+      for (int i = 0; i < p->max_slots; ++i)
+        if (p->slots[i].active && p->slots[i].L == L) h_small[ns++] = (uint32_t)i;
+  if ((e = cudaMemcpyAsync(p->d_desc, h_desc, sizeof(hsg::PoolDesc) * p->max_slots, cudaMemcpyHostToDevice,
                            p->stream)) != cudaSuccess ||
+      (ns && (e = cudaMemcpyAsync(p->d_small, h_small, sizeof(uint32_t) * ns, cudaMemcpyHostToDevice, p->stream)) !=
+                 cudaSuccess) ||
       (nt && (e = cudaMemcpyAsync(p->d_tiles, h_tiles, sizeof(uint2) * nt, cudaMemcpyHostToDevice, p->stream)) !=
                  cudaSuccess) ||
       (e = cudaMemcpyAsync(p->d_ntiles, h_ntiles, 2 * sizeof(uint32_t), cudaMemcpyHostToDevice, p->stream)) !=
@@ -440,7 +440,7 @@ cudaError_t launch_pool_half(hsg_pool* p, int upd, uint32_t colour, float step, 
   float4* S = const_cast<float4*>(S4);
   const float* J = reinterpret_cast<const float*>(p->arena);
   const uint32_t ts = (uint32_t)p->tile_sites;
-  const PoolDesc* D = p->d_desc;
+  const hsg::PoolDesc* D = p->d_desc;
   const uint2* T = p->d_tiles;
   const uint32_t* NT = p->d_ntiles;
   cudaStream_t st = p->stream;
@@ -552,7 +552,10 @@ cudaError_t join_lanes(hsg_pool* p, const bool (&used)[kLanes], cudaError_t e) {
 // Whether the small lattices take the resident kernel (hsg_resident.cu),
 // which then runs every sweep of a call in one launch per side.  All of
 // them or none: while the persistent kernels run for others anyway, a few small
-// lattices cost them nothing, and a launch of their own would come on top.
+// lattices cost them nothing, and a launch of their own would come on top.  Sites from
+// L = 26 count a quarter more: clusters of sixteen CTAs leave SMs idle
+// (29 x L = 28, 637k sites, heat-bath + 2 OR: 40.0 us against the persistent kernels'
+// 37.1, while 46 x L = 24, 636k sites, take 31.1 against 37.1).
 bool resident_pool(const hsg_pool* p, const hsg_schedule* s) {
   if (s->kind == HSG_NONE && s->n_or == 0) return false;
   if (main_passes(p, s) > 1) return false;  // the hits in passes, as configured
@@ -560,49 +563,44 @@ bool resident_pool(const hsg_pool* p, const hsg_schedule* s) {
   for (const Slot& sl : p->slots) {
     if (!sl.active) continue;
     if (sl.L >= hsg::kBatchMinL ? !p->batched : !hsg::resident_takes(main_update(s), sl.L, s->hits)) return false;
-    if (sl.L < hsg::kBatchMinL) sites += (uint64_t)sl.L * sl.L * sl.L;
+    if (sl.L >= hsg::kBatchMinL) continue;
+    const uint64_t n = (uint64_t)sl.L * sl.L * sl.L;
+    sites += sl.L < 26 ? n : n + n / 4;
   }
   return sites > 0 && sites <= hsg::kResidentPoolSites;
 }
 
-// n_sweeps sweeps of the small lattices, side by side: each side's launches on the
-// lane (the pool's stream and the side streams) with the fewest sites so far.
+// n_sweeps sweeps of the small lattices, side by side: each side's launch on the
+// lane (the pool's stream and the side streams) with the fewest sites so far.  It
+// reads the slots and the counters on the device: as kernel parameters, 64 lattices
+// to a launch, 1000 x L = 8 took 61 us a sweep for want of lattices in flight (1200 now 14).
 cudaError_t sweep_resident(hsg_pool* p, const hsg_schedule* s, int n_sweeps) {
-  int count[hsg::kBatchMinL] = {};
-  for (const Slot& sl : p->slots)
-    if (sl.active && sl.L < hsg::kBatchMinL) count[sl.L] += 1;
   const cudaStream_t st[kLanes] = {p->stream, p->side[0], p->side[1]};
   uint64_t load[kLanes] = {};
   bool used[kLanes] = {};
   cudaError_t e = cudaSuccess;
+  const uint32_t* slots = p->d_small;
   for (int L = hsg::kBatchMinL - 2; L >= 4 && e == cudaSuccess; L -= 2) {
-    if (count[L] == 0) continue;
+    const int n = p->small_count[L];
+    if (n == 0) continue;
     const int lane = (int)(std::min_element(load, load + kLanes) - load);
-    const uint64_t n = (uint64_t)L * L * L;
-    load[lane] += count[L] * n;
+    load[lane] += (uint64_t)n * L * L * L;
     if (lane > 0 && !used[lane]) e = cudaStreamWaitEvent(st[lane], p->fork_ev, 0);
     used[lane] = true;
-    hsg::ResidentArgs<hsg::kResidentPoolMax> a{};
+    hsg::ResidentArgs a{};
     a.L = (uint32_t)L;
     a.sweeps = (uint32_t)n_sweeps;
     a.per_sweep = (s->kind != HSG_NONE ? 2u : 0u) + 2u * (uint32_t)s->n_or;
     a.renorm_every = (uint32_t)s->renorm_every;
     a.step = s->step;
     a.hits = s->hits;
-    int left = count[L];
-    for (size_t i = 0; i < p->slots.size() && left > 0 && e == cudaSuccess; ++i) {
-      const Slot& sl = p->slots[i];
-      if (!sl.active || sl.L != L) continue;
-      a.lat[a.n++] = {reinterpret_cast<float4*>(p->arena + sl.off),
-                      reinterpret_cast<const float*>(p->arena + sl.off + sizeof(float4) * n),
-                      sl.sweep, key0(sl), key1(sl), beta_of(sl.T)};
-      left -= 1;
-      if (a.n == hsg::kResidentPoolMax || left == 0) {
-        e = hsg::launch_resident_pool(main_update(s), a, count[L], p->sm_count, st[lane]);
-        p->launches += 1;
-        a.n = 0;
-      }
-    }
+    a.n = n;
+    a.desc = p->d_desc;
+    a.slots = slots;
+    a.arena = p->arena;
+    if (e == cudaSuccess) e = hsg::launch_resident(main_update(s), a, p->sm_count, st[lane]);
+    p->launches += 1;
+    slots += n;
   }
   return join_lanes(p, used, e);
 }
@@ -745,10 +743,12 @@ hsg_status hsg_pool_create(hsg_pool** out, uint64_t budget_bytes, int max_slots,
   cudaError_t e = cudaGetDevice(&p->device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&p->sm_count, cudaDevAttrMultiProcessorCount, p->device);
   if (e == cudaSuccess) e = cudaMalloc(&p->arena, p->budget);
-  if (e == cudaSuccess) e = cudaMalloc(&p->d_desc, sizeof(PoolDesc) * max_slots);
-  if (e == cudaSuccess) e = cudaMallocHost(&p->h_desc, 2 * sizeof(PoolDesc) * max_slots);
+  if (e == cudaSuccess) e = cudaMalloc(&p->d_desc, sizeof(hsg::PoolDesc) * max_slots);
+  if (e == cudaSuccess) e = cudaMallocHost(&p->h_desc, 2 * sizeof(hsg::PoolDesc) * max_slots);
   if (e == cudaSuccess) e = cudaMalloc(&p->d_ntiles, 2 * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMallocHost(&p->h_ntiles, 4 * sizeof(uint32_t));
+  if (e == cudaSuccess) e = cudaMalloc(&p->d_small, sizeof(uint32_t) * max_slots);
+  if (e == cudaSuccess) e = cudaMallocHost(&p->h_small, 2 * sizeof(uint32_t) * max_slots);
   if (e == cudaSuccess) e = cudaMalloc(&p->d_energy, sizeof(double) * max_slots);
   if (e == cudaSuccess) e = cudaMallocHost(&p->h_energy, hsg_pool::kEnergyBufs * sizeof(double) * max_slots);
   if (e == cudaSuccess) e = cudaMallocHost(&p->h_sel, (size_t)hsg_pool::kEnergyBufs * max_slots);
@@ -780,6 +780,8 @@ hsg_status hsg_pool_destroy(hsg_pool* p) {
   cudaFreeHost(p->h_tiles);
   cudaFree(p->d_ntiles);
   cudaFreeHost(p->h_ntiles);
+  cudaFree(p->d_small);
+  cudaFreeHost(p->h_small);
   cudaFree(p->d_partials);
   cudaFree(p->d_energy);
   cudaFreeHost(p->h_energy);
@@ -921,7 +923,7 @@ hsg_status hsg_pool_sweep(hsg_pool* p, const hsg_schedule* sched, int n_sweeps) 
   // launches are issued directly.
   if (resident || (batch && !p->unbatched_left)) {
     if (resident) e = sweep_resident(p, sched, n_sweeps);
-    // the device's counters follow the host's
+    // the device's counters follow the host's (the resident kernel read them)
     if (e == cudaSuccess) {
       k_pool_advance<<<cdiv_u((unsigned)p->max_slots, 256), 256, 0, p->stream>>>(p->d_desc, p->max_slots,
                                                                                 (uint32_t)n_sweeps);

@@ -31,11 +31,12 @@
 //   L = 32   4 OR 20.3 -> 10.6 (13.1 -> 9.9), heat-bath 7.5 -> 5.5 (5.4 -> 4.6), 4 hits
 //            8.2 -> 8.3 (6.0 -> 7.3): there each hit costs 0.57 us against 0.19 on
 //            the whole GPU, hence the bound on the hits in resident_takes.
-// In a pool, one launch holds up to 64 lattices of one side, a cluster each, for
-// all the sweeps of a call (us per sweep, against the persistent kernels'
-// replayed graph): 8 x L = 16, 1 hit 10.6 -> 2.7; 128 x L = 16 16.4 -> 7.9; 64 x L = 16, 4 hits +
-// 2 OR 33 -> 13; 64 x L = 8 10.3 -> 2.3; with more work it is even (2048 x L = 16 131 -> 125)
-// or loses (64 x L = 24, 4 hits + 2 OR 56 -> 63), hence kResidentPoolSites.
+// In a pool, one launch holds all its lattices of one side, a cluster each, for all
+// the sweeps of a call (us per sweep of heat-bath + 2 OR, against the persistent
+// kernels' replayed graph): 64 x L = 8 18.6 -> 4.5, 1200 x 8 34.9 -> 13.8, 40 x L = 16
+// 22.7 -> 7.5, 150 x 16 30.9 -> 20.1, 46 x L = 24 37.1 -> 31.1, 16 x L = 28 29.0 -> 24.2;
+// with more work it is even (2048 x L = 16, 1 hit 131 -> 125) or loses (64 x L = 24, 4 hits
+// + 2 OR 56 -> 63), hence kResidentPoolSites.
 // A loop over sites with the indices formed and the bonds loaded for each
 // (so that larger lattices fit too): 7.9 us at L = 16, 24.9 against 14.0 at L = 40.
 #include "hsg_device.cuh"
@@ -93,8 +94,8 @@ struct KeptSite {
   float jxp, jxm, jyp, jym, jzp, jzm;
 };
 
-template <int U, int N>
-__global__ void __launch_bounds__(kThreadsMax, 1) k_resident(const __grid_constant__ ResidentArgs<N> a) {
+template <int U, bool POOL>
+__global__ void __launch_bounds__(kThreadsMax, 1) k_resident(const __grid_constant__ ResidentArgs a) {
   // sp[colour][plane][in-plane index]: plane 0 the halo below, 1 .. P this
   // CTA's own, P + 1 the halo above.
   extern __shared__ float4 sp[];
@@ -103,8 +104,22 @@ __global__ void __launch_bounds__(kThreadsMax, 1) k_resident(const __grid_consta
   const uint32_t z0 = rank * L / C, P = (rank + 1) * L / C - z0;
   const uint32_t part = (a.max_planes + 2) * plane;  // one colour's share of sp
   const uint32_t tid = threadIdx.x;
-  const ResidentLattice& lat = a.lat[N == 1 ? 0u : blockIdx.x / C];
-  const unsigned long long sweep0 = N == 1 ? *a.sweep_ptr : lat.sweep;
+  float4* spins = a.spins;
+  const float* J = a.J;
+  uint32_t k0 = a.k0, k1 = a.k1;
+  float beta = a.beta;
+  unsigned long long sweep0;
+  if constexpr (POOL) {
+    const PoolDesc& d = a.desc[a.slots[blockIdx.x / C]];
+    spins = reinterpret_cast<float4*>(a.arena) + d.spin_off;
+    J = reinterpret_cast<const float*>(a.arena) + d.j_off;
+    k0 = d.k0;
+    k1 = d.k1;
+    beta = d.beta;
+    sweep0 = (unsigned long long)d.sweep_hi << 32 | d.sweep_lo;
+  } else {
+    sweep0 = *a.sweep_ptr;
+  }
 
   // This thread's sites: in-plane index r of plane z, for tid < P * plane.
   const bool mine = tid < P * plane;
@@ -119,21 +134,21 @@ __global__ void __launch_bounds__(kThreadsMax, 1) k_resident(const __grid_consta
 #pragma unroll
   for (uint32_t c = 0; c < 2; ++c) {
     const uint32_t p = p0 ^ c, gzm = z == 0 ? g + (L - 1) * plane : g - plane;
-    const float *Jc = lat.J + c * a.nh, *Jo = lat.J + (1 - c) * a.nh;
+    const float *Jc = J + c * a.nh, *Jo = J + (1 - c) * a.nh;
     k[c].jxp = __ldg(Jc + g);
     k[c].jxm = __ldg(Jo + (p ? g : g + dxm));
     k[c].jyp = __ldg(Jc + 2 * a.nh + g);
     k[c].jym = __ldg(Jo + 2 * a.nh + (g + dym));
     k[c].jzp = __ldg(Jc + 4 * a.nh + g);
     k[c].jzm = __ldg(Jo + 4 * a.nh + gzm);
-    k[c].s = load_spin(lat.spins, a.packed, a.nh, c, g);
+    k[c].s = load_spin(spins, a.packed, a.nh, c, g);
     if (mine) sp[c * part + q] = k[c].s;
     for (uint32_t i = tid; i < 2 * plane; i += blockDim.x) {  // the halo planes z0 - 1 and z0 + P
       const bool lo = i < plane;
       const uint32_t ri = lo ? i : i - plane;
       const uint32_t zi = lo ? (z0 == 0 ? L - 1 : z0 - 1) : (z0 + P == L ? 0u : z0 + P);
       sp[c * part + (lo ? 0u : (P + 1) * plane) + ri] =
-          load_spin(lat.spins, a.packed, a.nh, c, zi * plane + ri);
+          load_spin(spins, a.packed, a.nh, c, zi * plane + ri);
     }
   }
   // Where the CTA below (above) keeps this CTA's first (last) plane.
@@ -172,7 +187,7 @@ __global__ void __launch_bounds__(kThreadsMax, 1) k_resident(const __grid_consta
           in.s = make_float3(k[c].s.x, k[c].s.y, k[c].s.z);
           in.q = 0;
           in.site = (2 * xh + p) + y * L + z * L * L;
-          k[c].s = main_update ? site_result<U>(in, c, lo, hi, lat.k0, lat.k1, lat.beta, a.step, a.hits)
+          k[c].s = main_update ? site_result<U>(in, c, lo, hi, k0, k1, beta, a.step, a.hits)
                                : site_result<U_OR>(in, c, 0u, 0u, 0u, 0u, 0.0f, 0.0f, 1);
           sp[c * part + q] = k[c].s;
           if (first) st_cluster(to_below + c * part * 16u, k[c].s);
@@ -197,11 +212,11 @@ __global__ void __launch_bounds__(kThreadsMax, 1) k_resident(const __grid_consta
     }
   }
   if (mine) {
-    store_spin(lat.spins, a.packed, a.nh, 0, g, k[0].s);
-    store_spin(lat.spins, a.packed, a.nh, 1, g, k[1].s);
+    store_spin(spins, a.packed, a.nh, 0, g, k[0].s);
+    store_spin(spins, a.packed, a.nh, 1, g, k[1].s);
   }
   // Every CTA read the counter before the first barrier.
-  if (N == 1 && rank == 0 && tid == 0) *a.sweep_ptr = sweep0 + a.sweeps;
+  if (!POOL && rank == 0 && tid == 0) *a.sweep_ptr = sweep0 + a.sweeps;
 }
 
 // CTAs in the cluster of an L lattice: as many as divide the work, at most
@@ -231,8 +246,8 @@ uint32_t pool_cluster_size(uint32_t L, int total, int sm_count) {
   return c;
 }
 
-template <int U, int N>
-cudaError_t launch_u(ResidentArgs<N> a, uint32_t cluster, cudaStream_t s) {
+template <int U, bool POOL>
+cudaError_t launch_u(ResidentArgs a, uint32_t cluster, cudaStream_t s) {
   static PerDevice configured;
   cudaError_t e = cudaSuccess;
   std::atomic<int>* slot = device_slot(configured, &e);
@@ -245,10 +260,10 @@ cudaError_t launch_u(ResidentArgs<N> a, uint32_t cluster, cudaStream_t s) {
   a.by_plane = make_fastdiv(a.plane);
   a.by_Lh = make_fastdiv(a.Lh);
   const uint32_t threads = cta_threads(a.L, cluster);
-  if (threads > kThreadsMax || a.n < 1 || a.n > N) return cudaErrorInvalidValue;
+  if (threads > kThreadsMax || a.n < 1) return cudaErrorInvalidValue;
   if (slot->load(std::memory_order_acquire) == 0) {
-    e = cudaFuncSetAttribute(k_resident<U, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_resident<U, N>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    e = cudaFuncSetAttribute(k_resident<U, POOL>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_resident<U, POOL>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     slot->store(1, std::memory_order_release);
   }
@@ -264,19 +279,18 @@ cudaError_t launch_u(ResidentArgs<N> a, uint32_t cluster, cudaStream_t s) {
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_resident<U, N>, a);
+  return cudaLaunchKernelEx(&cfg, k_resident<U, POOL>, a);
 }
 
-template <int N>
-cudaError_t launch_kinds(int upd, const ResidentArgs<N>& a, uint32_t cluster, cudaStream_t s) {
-  if (!resident_takes(upd, (int)a.L, a.hits)) return cudaErrorInvalidValue;
+template <bool POOL>
+cudaError_t launch_kinds(int upd, const ResidentArgs& a, uint32_t cluster, cudaStream_t s) {
   switch (upd) {
-    case U_OR: return launch_u<U_OR>(a, cluster, s);
-    case U_MET_SPHERE: return launch_u<U_MET_SPHERE>(a, cluster, s);
-    case U_MET_BALL: return launch_u<U_MET_BALL>(a, cluster, s);
-    case U_HB: return launch_u<U_HB>(a, cluster, s);
-    case U_MET_OR_SPHERE: return launch_u<U_MET_OR_SPHERE>(a, cluster, s);
-    case U_MET_OR_BALL: return launch_u<U_MET_OR_BALL>(a, cluster, s);
+    case U_OR: return launch_u<U_OR, POOL>(a, cluster, s);
+    case U_MET_SPHERE: return launch_u<U_MET_SPHERE, POOL>(a, cluster, s);
+    case U_MET_BALL: return launch_u<U_MET_BALL, POOL>(a, cluster, s);
+    case U_HB: return launch_u<U_HB, POOL>(a, cluster, s);
+    case U_MET_OR_SPHERE: return launch_u<U_MET_OR_SPHERE, POOL>(a, cluster, s);
+    case U_MET_OR_BALL: return launch_u<U_MET_OR_BALL, POOL>(a, cluster, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -292,13 +306,10 @@ bool resident_takes(int upd, int L, int hits) {
   return hits <= (L <= 16 ? 16 : L <= 24 ? 5 : 2);
 }
 
-cudaError_t launch_resident(int upd, const ResidentArgs<1>& a, cudaStream_t s) {
-  return launch_kinds(upd, a, cluster_size(a.L), s);
-}
-
-cudaError_t launch_resident_pool(int upd, const ResidentArgs<kResidentPoolMax>& a, int total, int sm_count,
-                                 cudaStream_t s) {
-  return launch_kinds(upd, a, pool_cluster_size(a.L, total, sm_count), s);
+cudaError_t launch_resident(int upd, const ResidentArgs& a, int sm_count, cudaStream_t s) {
+  if (!resident_takes(upd, (int)a.L, a.hits)) return cudaErrorInvalidValue;
+  return a.slots ? launch_kinds<true>(upd, a, pool_cluster_size(a.L, a.n, sm_count), s)
+                 : launch_kinds<false>(upd, a, cluster_size(a.L), s);
 }
 
 }  // namespace hsg

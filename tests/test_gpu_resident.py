@@ -86,11 +86,11 @@ def test_a_captured_sweep_replays_as_new_sweeps(hsg):
 
 
 # alone in their clusters, and too many for the GPU at once (smaller clusters)
-@pytest.mark.parametrize("sides,n", [((4, 6, 8, 10, 12, 14, 16, 18, 20, 22, 24, 26, 28, 30), 14), ((16,), 130), ((8,), 70),
+@pytest.mark.parametrize("sides,n", [((4, 6, 8, 10, 12, 14, 16, 18, 20, 22, 24, 26, 28, 30), 14), ((16,), 130), ((8,), 70), ((4, 8), 400),
                                      ((12, 20), 60), ((24,), 40), ((26, 28, 30), 30)])
 @pytest.mark.parametrize("use_stream", [True, False])
 def test_pools_of_small_lattices_equal_lattices_alone(hsg, sides, n, use_stream):
-    """All sweeps of a call in one launch per 64 lattices of a side; counters
+    """All sweeps of a call in one launch per side; counters
     stay right for the calls that take the half-sweep kernels."""
     kw = dict(kind=hsg.HSG_METROPOLIS, hits=2, proposal=hsg.HSG_PROP_BALL, n_or=1, renorm_every=3)
     many = dict(kw, hits=18)  # too many hits for the resident kernel
