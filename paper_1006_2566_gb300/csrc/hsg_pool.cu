@@ -12,7 +12,9 @@
 // and the slot table change, in device memory, between replays.
 //
 // From 2^17 sites of lattices of L >= 32 on, those lattices are swept in
-// batches instead (hsg_batch.cu), beside the persistent kernels of the others.
+// batches instead (hsg_batch.cu), beside the persistent kernels of the others; and
+// where the small lattices are few, the resident kernel (hsg_resident.cu) takes them
+// in place of the persistent ones.
 //
 // Every site is updated by half_sweep_site or update_rows, the same device code as
 // the single-lattice kernels, with the same key and counters: a lattice swept

@@ -43,7 +43,7 @@ __device__ __forceinline__ uint32_t site_number(int xh, int p, int y, int z, int
 //            kernel (86.5 us; 95.8 with two rows per thread)
 //   packed, L = 130: 12.1 -> 7.7, 35.7 -> 23.6, 21.4 -> 13.9 us; L = 256: 89.6 ->
 //            84.3, 170.6 -> 165, 102.9 -> 94.1 us
-// Rows per thread (row_shape below): the own-column neighbour of one row is
+// Rows per thread (launch_global below): the own-column neighbour of one row is
 // the y neighbour of the next, so R rows load 2 + 2/R + 1 neighbours each
 // instead of five; but R rows per thread leave 1/R of the threads, and below
 // about 10^6 sites those are too few (L = 64, 4-hit Metropolis: 4.1, 5.1,
@@ -56,14 +56,15 @@ constexpr int G_THREADS = 128;
 
 template <int U, int R, int MIN_BLOCKS, class Off, bool PACKED, bool OVERLAP>
 __global__ void __launch_bounds__(G_THREADS, MIN_BLOCKS)
-    k_half_sweep_rows(const SweepArgs a, FastDiv by_lh, uint32_t columns, bool early) {
+    k_half_sweep_rows(const SweepArgs a, FastDiv by_lh, uint32_t columns, bool early, bool down) {
   const uint32_t t = blockIdx.x * G_THREADS + threadIdx.x;
   if constexpr (OVERLAP) {
     if (early) let_next_start();
     wait_for_previous();
   }
   if (t >= columns) return;
-  const uint32_t g = fast_div(t, by_lh), xh = t - g * (uint32_t)a.Lh, y0 = g * R, z = blockIdx.y;
+  const uint32_t g = fast_div(t, by_lh), xh = t - g * (uint32_t)a.Lh, y0 = g * R;
+  const uint32_t z = down ? gridDim.y - 1 - blockIdx.y : blockIdx.y;
   const RowLattice<PACKED, OVERLAP> lat{a.own,    a.oth,    a.jx_own, a.jy_own,      a.jz_own,       a.jx_oth,
                                a.jy_oth, a.jz_oth, a.stride, (uint32_t)a.L, (uint32_t)a.Lh, (uint32_t)a.colour};
   DrawArgs d{a.sweep_lo, a.sweep_hi, a.k0, a.k1, a.beta, a.step, a.hits, 0};
@@ -96,7 +97,7 @@ __global__ void __launch_bounds__(G_THREADS, MIN_BLOCKS)
 // other colour's spins in the thread's own column on planes z-1 and z (the
 // site's -z neighbour and one of its x neighbours) are carried from the
 // plane before, so a site loads four neighbour spins instead of six; the
-// inputs and the site code are those of k_half_sweep_global, so the results
+// inputs and the site code are those of k_half_sweep_rows, so the results
 // are the same bit for bit.  Measured on the L = 256 heat-bath half-sweep:
 // 6 planes and 40 registers (12 blocks per SM) 94.0 us, against 100.9 us
 // for one site per thread at 32 registers; 8 planes 95.1, 4 planes 96.0,
@@ -118,7 +119,7 @@ constexpr int ZM_MIN_L = 152;
 constexpr int ZM_BX = 16, ZM_BY = 8;
 
 template <class Off>
-__global__ void __launch_bounds__(G_THREADS, 12) k_half_sweep_column(const SweepArgs a) {
+__global__ void __launch_bounds__(G_THREADS, 12) k_half_sweep_column(const SweepArgs a, bool down) {
   const uint32_t xh = blockIdx.x * blockDim.x + threadIdx.x;
   const uint32_t y = blockIdx.y * blockDim.y + threadIdx.y;
   const uint32_t L = a.L, Lh = a.Lh;
@@ -130,7 +131,7 @@ __global__ void __launch_bounds__(G_THREADS, 12) k_half_sweep_column(const Sweep
     sweep_hi = (uint32_t)(sw >> 32);
   }
   const uint32_t plane = L * Lh;
-  const uint32_t z0 = blockIdx.z * ZM_PLANES, z1 = min(z0 + ZM_PLANES, L);
+  const uint32_t z0 = (down ? gridDim.z - 1 - blockIdx.z : blockIdx.z) * ZM_PLANES, z1 = min(z0 + ZM_PLANES, L);
   // rows y, y+1, y-1 and columns xh+1, xh-1, wrapped (the layout comment of
   // hsg_device.cuh; the same indices as site_index)
   const uint32_t row = y * Lh, row_p = (y + 1 == L ? 0u : y + 1) * Lh, row_m = (y == 0 ? L - 1 : y - 1) * Lh;
@@ -285,18 +286,37 @@ Overlap overlap(int L) {
   return L <= 90 ? LATE : L <= 126 ? EARLY : NONE;
 }
 
+// Colour 1's CTAs take the planes from the top down (CTAs start in the order of
+// their index), where colour 0's went up: each half-sweep so begins on the planes that
+// the one before left in L2, where streaming them in the same order finds none.  us per
+// two half-sweeps, same order / reversed (126 MB L2; the state is 28 L^3 bytes, packed 24):
+//   OR         L = 136 16.8 / 17.0, 144 22.3 / 20.3, 152 33.0 / 26.5, 160 42.8 / 32.4, 176 58.1 / 48.3,
+//              192 73.4 / 64.4, 222 113 / 107, 256 168 / 162, 288 240 / 233
+//   heat-bath  L = 152 46.8 / 46.3, 192 85.0 / 83.3, 222 125.6 / 123.6, 256 180 / 180
+//   ball       L = 136 25.7 / 25.8, 144 32.3 / 30.3, 160 53.2 / 44.1, 192 87.1 / 80.7, 256 198 / 190;
+//              4 hits 160 84.8 / 81.9, 256 308 / 305
+//   packed OR  L = 144 21.5 / 21.4, 152 29.2 / 26.3, 160 45.6 / 33.9, 192 75.7 / 64.9, 256 169 / 159
+// At L = 400 OR 635 / 630, ball 735 / 728, heat-bath 686 / 688; at 512 1315 / 1312, 1534 /
+// 1524, sphere + OR 1548 / 1554, heat-bath 1381 / 1388.
+constexpr int kDownMinL = 144, kDownMaxL = 400, kDownMaxLHeatbath = 320;
+template <int U>
+bool downward(const SweepArgs& a) {
+  return a.colour == 1 && a.L >= kDownMinL && a.L <= (U == U_HB ? kDownMaxLHeatbath : kDownMaxL);
+}
+
 template <int U, int R, int MIN_BLOCKS, class Off, bool PACKED>
 cudaError_t launch_rows(const SweepArgs& a, cudaStream_t s) {
   const uint32_t columns = (uint32_t)a.Lh * (uint32_t)(a.L / R);
   const FastDiv by_lh = make_fastdiv((uint32_t)a.Lh);
   const dim3 grid(cdiv(columns, G_THREADS), (unsigned)a.L);
+  const bool down = downward<U>(a);
   if constexpr (sizeof(Off) == 4 && R < 4) {
     const Overlap o = overlap<U>(a.L);
     if (o != NONE)
       return launch_overlapped(k_half_sweep_rows<U, R, MIN_BLOCKS, Off, PACKED, true>, grid, dim3(G_THREADS), s, a, by_lh,
-                               columns, o == EARLY);
+                               columns, o == EARLY, down);
   }
-  k_half_sweep_rows<U, R, MIN_BLOCKS, Off, PACKED, false><<<grid, G_THREADS, 0, s>>>(a, by_lh, columns, false);
+  k_half_sweep_rows<U, R, MIN_BLOCKS, Off, PACKED, false><<<grid, G_THREADS, 0, s>>>(a, by_lh, columns, false, down);
   return cudaGetLastError();
 }
 
@@ -312,7 +332,7 @@ cudaError_t launch_rows(const SweepArgs& a, cudaStream_t s) {
 //                          [18.4 / 47 / 69 / 153]; R 1, B 12 1 hit 10.3 / 27.8 / 46.7 / 106
 //   ball       R 1, B 12   1 hit 10.3 / 25.5 / 42.2 / 96 [10.3 / 29.7 / 44.6 / 97] (R 4 10.9 / 25.7 / 47.1 / 102);
 //              R 4         4 hits 22.5 / 42.3 / 68.9 / 155 [20.5 / 50.2 / 71.5 / 161] (R 1, B 12 21.5 / 42.5 / 71.0 / 164)
-//   sphere+OR  R 1, B 14   1 hit 10.4 / 25.0 / 41.5 / 94 [10.3 / 27.0 / 41.8 / 91];
+//   sphere+OR  R 1, B 14   1 hit 10.4 / 22.6 / 40.7 / 93 [12.4 / 28.0 / 43.3 / 93] (R 2, B 12 10.3 / 25.4 / 44.8 / 99);
 //              R 2, B 8    4 hits 18.5 / 36.9 / 60.7 / 139 [18.5 / 45.1 / 65.1 / 143]
 //   ball+OR    R 2         1 hit 10.3 / 24.0 / 40.3 / 92 [10.3 / 33.1 / 50.0 / 107], 4 hits 21.5 / 40.3 / 67.7 / 155
 //                          [20.6 / 52.3 / 76.6 / 169]
@@ -360,10 +380,11 @@ cudaError_t launch_kind(int variant, const SweepArgs& a, int sm_count, cudaStrea
   if constexpr (U == U_HB) {
     if (a.L >= ZM_MIN_L) {
       const dim3 grid(cdiv(a.Lh, ZM_BX), cdiv(a.L, ZM_BY), cdiv(a.L, ZM_PLANES));
+      const bool down = downward<U>(a);
       if (a.L > kMaxOff32L)
-        k_half_sweep_column<unsigned long long><<<grid, dim3(ZM_BX, ZM_BY), 0, s>>>(a);
+        k_half_sweep_column<unsigned long long><<<grid, dim3(ZM_BX, ZM_BY), 0, s>>>(a, down);
       else
-        k_half_sweep_column<uint32_t><<<grid, dim3(ZM_BX, ZM_BY), 0, s>>>(a);
+        k_half_sweep_column<uint32_t><<<grid, dim3(ZM_BX, ZM_BY), 0, s>>>(a, down);
       return cudaGetLastError();
     }
   }

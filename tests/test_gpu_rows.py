@@ -33,9 +33,9 @@ def sweep_halves(hsg, lat, kernel):
             lat.half_sweep(hsg.schedule(T=0.7, hits=hits, proposal=prop, kernel=kernel), upd, colour)
 
 
-# 4, 6: the smallest; 94 | 96: one | two rows; 150 | 152, 154: the heat-bath's
+# 4, 6: the smallest; 94 | 96: one | two rows; 142 | 144: colour 1 from the top down; 150 | 152, 154: the heat-bath's
 # column march, four rows where 4 divides L; 158 | 160: packed two rows
-@pytest.mark.parametrize("L", [4, 6, 94, 96, 150, 152, 154, 158, 160, 226])
+@pytest.mark.parametrize("L", [4, 6, 94, 96, 142, 144, 150, 152, 154, 158, 160, 226])
 def test_global_kernels_equal_the_slab_kernel(hsg, L):
     outs = []
     for layout, kernel in ((hsg.HSG_LAYOUT_FLOAT4, hsg.HSG_KERNEL_SLAB), (hsg.HSG_LAYOUT_FLOAT4, hsg.HSG_KERNEL_GLOBAL),
