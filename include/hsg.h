@@ -80,8 +80,9 @@ enum { HSG_HOST = 0, HSG_DEVICE = 1 };
 /* Half-sweep kernel variant. */
 enum {
   HSG_KERNEL_AUTO = 0,   /* library's choice: HSG_KERNEL_WAVE when the lattice's
-                          * spins and bonds (28 N bytes) exceed three quarters of
-                          * the device's L2, so that the sweep streams much of it
+                          * spins and bonds (28 N bytes) exceed 1.2 times the
+                          * device's L2 (three quarters of it with renorm_every = 1,
+                          * which WAVE fuses), so that the sweep streams much of it
                           * from HBM; else GLOBAL.  hsg_sweep runs all sweeps up to
                           * an energy in one launch where the lattice is small (L <=
                           * 32, few hits): the same results */

@@ -3,7 +3,7 @@
 // Host code only: argument checks, stream-ordered device memory, the sweep
 // schedule (which kernels run in which order), the energy log and the
 // event-based profiler.  Every step of the Monte Carlo itself runs in the
-// kernels of hsg_sweep.cu and hsg_aux.cu.
+// kernels of hsg_sweep.cu, hsg_wave.cu, hsg_resident.cu and hsg_aux.cu.
 #include <algorithm>
 #include <atomic>
 #include <cmath>
@@ -266,17 +266,21 @@ hsg_status check_schedule(hsg_ctx* c, const hsg_schedule* s, bool need_kind) {
 float beta_of(double T) { return std::isinf(T) ? 0.0f : (float)(1.0 / T); }
 
 // HSG_KERNEL_AUTO: the temporally blocked over-relaxation once the spins
-// and bonds (16 + 12 bytes per site) exceed three quarters of L2 -- it
-// saves HBM traffic, and pays where the sweeps stream much of their state
-// from HBM.  Measured on GB300 (126 MB L2), whole sweeps of 4-hit
-// Metropolis + 1 OR sweep: L = 128 (59 MB) 73.6 against 66.4 us with the
-// global kernel, L = 144 (84 MB) 123-127 against 121-125 us, L = 152 (98
-// MB) 135-139 against 144-147 us, L = 160 157 against 167 us; at L = 256
-// one OR sweep 131.7 us against 2 x 87.9 us.
-int pick_variant(const hsg_ctx* c, int requested) {
-  if (requested == HSG_KERNEL_GLOBAL || requested == HSG_KERNEL_SLAB || requested == HSG_KERNEL_WAVE) return requested;
+// and bonds (16 + 12 bytes per site) exceed 1.2 times L2 -- it saves HBM
+// traffic, and pays where the sweeps stream most of their state from HBM; below,
+// two half-sweeps, the second from the top down, find enough of it in L2.
+// Measured on GB300 (126 MB L2), one OR sweep, global / wave: L = 152 (98 MB)
+// 26.5 / 32.5 us, 160 (115 MB) 32.4 / 38.1, 176 (153 MB) 48.3 / 55.6, 184 (174 MB)
+// 56.7 / 56.8, 192 64.4 / 60.7, 256 162 / 127.  Where a renormalisation is due
+// after every sweep, which the wave fuses and the global kernel does not, from
+// three quarters of L2: heat-bath + OR + renormalisation L = 154 93.9 / 89.8 us,
+// 160 101.6 / 96.6, 176 143.4 / 136.8.
+int pick_variant(const hsg_ctx* c, const hsg_schedule* s) {
+  if (s->kernel != HSG_KERNEL_AUTO) return s->kernel;
   if (c->packed) return hsg::V_GLOBAL;
-  return 4 * 28LL * c->N > 3 * c->l2_bytes ? hsg::V_WAVE : hsg::V_GLOBAL;
+  const long long state = 28LL * c->N;
+  const bool wave = s->renorm_every == 1 ? 4 * state > 3 * c->l2_bytes : 5 * state > 6 * c->l2_bytes;
+  return wave ? hsg::V_WAVE : hsg::V_GLOBAL;
 }
 
 // Temporally blocked launches of one sweep under schedule s with the wave
@@ -300,7 +304,7 @@ hsg_status run_half_sweep(hsg_ctx* c, const hsg_schedule* s, int update, int col
     kclass = HSG_PROF_HEATBATH;
   }
   const hsg::SweepArgs a = sweep_args(c, colour, beta_of(s->T), s->step, s->hits);
-  int variant = pick_variant(c, s->kernel);
+  int variant = pick_variant(c, s);
   if (variant == hsg::V_WAVE) variant = hsg::V_GLOBAL;  // a single colour: the plain kernel
   return launch(c, kclass, 1, "half-sweep kernel", [&] { return hsg::launch_half_sweep(upd, variant, a, c->sm_count, c->stream); });
 }
@@ -409,7 +413,7 @@ hsg_status run_renorm(hsg_ctx* c) {
 // counter and the energy-log position advance as the device ones will.
 hsg_status enqueue_one_sweep(hsg_ctx* c, const hsg_schedule* s) {
   hsg_status st;
-  const bool wave = pick_variant(c, s->kernel) == hsg::V_WAVE;
+  const bool wave = pick_variant(c, s) == hsg::V_WAVE;
   if (s->kind != HSG_NONE)
     for (int colour = 0; colour < 2; ++colour)
       if ((st = run_half_sweep(c, s, s->kind, colour)) != HSG_OK) return st;
@@ -759,7 +763,7 @@ hsg_status hsg_sweep(hsg_ctx* c, const hsg_schedule* s, int n_sweeps) {
     if (st != HSG_OK) return st;
   }
   if (use_resident(c, s)) return run_resident(c, s, n_sweeps);
-  const int variant = pick_variant(c, s->kernel);
+  const int variant = pick_variant(c, s);
   const int swaps = variant == hsg::V_WAVE ? wave_sweeps_per_sweep(s) : 0;
   if (swaps > 0 && !c->spins_alt) {
     cudaError_t e = dev_alloc(reinterpret_cast<void**>(&c->spins_alt), sizeof(float4) * (size_t)c->N, c->stream);
@@ -968,7 +972,7 @@ hsg_status hsg_kernel_for(hsg_ctx* c, const hsg_schedule* s, int* kernel) {
   if (!kernel) return fail(c, HSG_EINVAL, "kernel is NULL");
   hsg_status st = check_schedule(c, s, true);
   if (st != HSG_OK) return st;
-  *kernel = pick_variant(c, s->kernel);
+  *kernel = pick_variant(c, s);
   return HSG_OK;
 }
 
