@@ -331,7 +331,9 @@ cudaError_t launch_rows(const SweepArgs& a, cudaStream_t s) {
 //   sphere     R 2, B 10   1 hit 9.6 / 24.7 / 40.9 / 92 [10.2 / 30.7 / 46.9 / 101], 4 hits 18.4 / 35.1 / 58.9 / 133
 //                          [18.4 / 47 / 69 / 153]; R 1, B 12 1 hit 10.3 / 27.8 / 46.7 / 106
 //   ball       R 1, B 12   1 hit 10.3 / 25.5 / 42.2 / 96 [10.3 / 29.7 / 44.6 / 97] (R 4 10.9 / 25.7 / 47.1 / 102);
-//              R 4         4 hits 22.5 / 42.3 / 68.9 / 155 [20.5 / 50.2 / 71.5 / 161] (R 1, B 12 21.5 / 42.5 / 71.0 / 164)
+//              R 2, R 4    4 hits, each as a sweep of its own, R 1, B 12 / R 2 / R 4: L = 120 17.9 / 17.9, 128 21.3 / 20.9,
+//                          150 34.1 / 33.3, 160 - / 39.7 / 40.8, 192 - / 66.9 / 67.4, 208 - / 84.3 / 84.8, 222 109 / 102,
+//                          224 - / 104.1 / 103.9, 256 - / 154 / 153, 320 - / 298 / 294 [128 22.6, 150 46.2, 192 74.7, 256 164]
 //   sphere+OR  R 1, B 14   1 hit 10.4 / 22.6 / 40.7 / 93 [12.4 / 28.0 / 43.3 / 93] (R 2, B 12 10.3 / 25.4 / 44.8 / 99);
 //              R 2, B 8    4 hits 18.5 / 36.9 / 60.7 / 139 [18.5 / 45.1 / 65.1 / 143]
 //   ball+OR    R 2         1 hit 10.3 / 24.0 / 40.3 / 92 [10.3 / 33.1 / 50.0 / 107], 4 hits 21.5 / 40.3 / 67.7 / 155
@@ -356,7 +358,8 @@ cudaError_t launch_global(const SweepArgs& a, cudaStream_t s) {
     if constexpr (U == U_MET_SPHERE) {
       return launch_rows<U, 2, 10, uint32_t, PACKED>(a, s);
     } else if constexpr (U == U_MET_BALL) {
-      if (a.hits > 1 && a.L >= 152 && a.L % 4 == 0) return launch_rows<U, 4, 1, uint32_t, PACKED>(a, s);
+      if (a.hits > 1 && a.L >= 220 && a.L % 4 == 0) return launch_rows<U, 4, 1, uint32_t, PACKED>(a, s);
+      if (a.hits > 1 && a.L >= 124) return launch_rows<U, 2, 1, uint32_t, PACKED>(a, s);
       return launch_rows<U, 1, 12, uint32_t, PACKED>(a, s);
     } else if constexpr (U == U_MET_OR_SPHERE) {
       if (a.hits == 1) return launch_rows<U, 1, 14, uint32_t, PACKED>(a, s);

@@ -34,8 +34,8 @@ def sweep_halves(hsg, lat, kernel):
 
 
 # 4, 6: the smallest; 94 | 96: one | two rows; 142 | 144: colour 1 from the top down; 150 | 152, 154: the heat-bath's
-# column march, four rows where 4 divides L; 158 | 160: packed two rows
-@pytest.mark.parametrize("L", [4, 6, 94, 96, 142, 144, 150, 152, 154, 158, 160, 226])
+# column march; 122 | 124 | 224: ball, many hits, one | two | four rows; 158 | 160: packed two rows
+@pytest.mark.parametrize("L", [4, 6, 94, 96, 122, 124, 142, 144, 150, 152, 154, 158, 160, 224, 226])
 def test_global_kernels_equal_the_slab_kernel(hsg, L):
     outs = []
     for layout, kernel in ((hsg.HSG_LAYOUT_FLOAT4, hsg.HSG_KERNEL_SLAB), (hsg.HSG_LAYOUT_FLOAT4, hsg.HSG_KERNEL_GLOBAL),
