@@ -68,7 +68,8 @@ struct hsg_ctx {
   double* partials = nullptr;  // energy first-pass sums
   double* elog = nullptr;      // energy log
   int elog_cap = 0, elog_n = 0;
-  double* host_e = nullptr;  // pinned, 2 doubles: E/N and the bond-box wait flag
+  hsg::ResultWords words{};
+  double* host_e = nullptr;  // words.p, pinned: E/N and the bond-box wait flag
   bool prof = false;
   bool group = false;     // inside hsg_sweep: one event pair per run of same-class launches
   bool run_open = false;  // recs.back() still lacks its stop event
@@ -201,7 +202,7 @@ void release(hsg_ctx* c) {
   dev_free(c->d_ctr, s);
   cudaStreamSynchronize(s);
   if (c->gexec) cudaGraphExecDestroy(c->gexec);
-  hsg::give_result_words(c->host_e);
+  hsg::give_result_words(c->words);
   for (auto& r : c->recs) {
     cudaEventDestroy(r.start);
     if (r.stop) cudaEventDestroy(r.stop);
@@ -652,7 +653,8 @@ hsg_status hsg_create_layout(hsg_ctx** out, int L, uint64_t seed, uint32_t sampl
     release(c);
     return st;
   }
-  e = hsg::take_result_words(&c->host_e);
+  e = hsg::take_result_words(&c->words);
+  c->host_e = c->words.p;
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_ctr, 0, kCounters * sizeof(unsigned long long), c->stream);
   if (e != cudaSuccess) {
     st = cuda_fail(nullptr, e, "pinned host slot / counters");

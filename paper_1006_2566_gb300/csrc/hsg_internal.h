@@ -288,10 +288,15 @@ cudaError_t launch_add_u64(unsigned long long* p, unsigned long long d, cudaStre
 cudaError_t launch_renorm(void* S, bool packed, long long n, int sm_count, cudaStream_t s);
 
 // Stream-ordered device memory from the library's pool on the current device
-// (hsg_memory.cu; freed with cudaFreeAsync), and four pinned words for results.
+// (hsg_memory.cu; freed with cudaFreeAsync), and four pinned words for results
+// with the id of the CUDA context that they belong to (0: pages of their own).
 cudaError_t device_alloc(void** p, size_t bytes, cudaStream_t s);
-cudaError_t take_result_words(double** p);
-void give_result_words(double* p);
+struct ResultWords {
+  double* p;
+  unsigned long long ctx_id;
+};
+cudaError_t take_result_words(ResultWords* w);
+void give_result_words(const ResultWords& w);
 
 // Record the calling thread's last error message (read by hsg_last_error(NULL)).
 void set_thread_error(const std::string& msg);

@@ -10,8 +10,10 @@
 // up to kKeepBytes of freed memory for the next context (more is given back at the
 // next synchronisation, all of it before an allocation may fail), and the
 // result words are cut from pinned pages, given back once none of a page is
-// in use (the first page stays).  Both are kept per CUDA context (by its id, so that
-// nothing outlives a device reset) under one lock; stream order is CUDA's.
+// in use (the first page stays).  Both are kept per CUDA context under one lock, by
+// the context's id: after a device reset the handles and the addresses come back,
+// the ids do not.  Words are given back to the context that they came from; of
+// one that is gone nothing is touched.  Stream order is CUDA's.
 #include <cstdint>
 #include <mutex>
 
@@ -29,7 +31,8 @@ struct Page {
   uint64_t used[kSlots / 64];
 };
 struct Device {
-  unsigned long long ctx_id;
+  CUcontext ctx;
+  unsigned long long ctx_id;  // 1, 2, ... in CUDA's own count
   cudaMemPool_t pool;
   Page pages[kPages];
 };
@@ -53,24 +56,37 @@ F driver_function(const char* name) {
   return reinterpret_cast<F>(p);
 }
 
-// The current CUDA context's record (g_mu held), or nullptr: no such entry
-// points, or more contexts over the process's life than there are records.
-Device* current_device() {
+// The current CUDA context and its id; false: none, or no such entry points.
+bool current_context(CUcontext* ctx, unsigned long long* id) {
   static const CtxGetCurrentFn get_current = driver_function<CtxGetCurrentFn>("cuCtxGetCurrent");
   static const CtxGetIdFn get_id = driver_function<CtxGetIdFn>("cuCtxGetId");
-  if (!get_current || !get_id || cudaFree(nullptr) != cudaSuccess) return nullptr;
-  CUcontext ctx = nullptr;
-  unsigned long long id = 0;
-  if (get_current(&ctx) != CUDA_SUCCESS || !ctx || get_id(ctx, &id) != CUDA_SUCCESS) return nullptr;
+  *ctx = nullptr;
+  return get_current && get_id && get_current(ctx) == CUDA_SUCCESS && *ctx && get_id(*ctx, id) == CUDA_SUCCESS;
+}
+
+Device* find_device(unsigned long long id) {
   for (int i = 0; i < g_n; ++i)
     if (g_devices[i].ctx_id == id) return &g_devices[i];
-  int dev = 0;
-  if (g_n == kMaxDevices || cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+  return nullptr;
+}
+
+// The current CUDA context's record (g_mu held), or nullptr: no such entry
+// points, or more contexts at a time than there are records.  A record with
+// this context's handle and another id is of a context that is gone: reused.
+Device* current_device() {
+  CUcontext ctx = nullptr;
+  unsigned long long id = 0;
+  if (cudaFree(nullptr) != cudaSuccess || !current_context(&ctx, &id)) return nullptr;
+  if (Device* known = find_device(id)) return known;
+  int slot = 0, dev = 0;
+  while (slot < g_n && g_devices[slot].ctx != ctx) ++slot;
+  if (slot == kMaxDevices || cudaGetDevice(&dev) != cudaSuccess) return nullptr;
   cudaMemPoolProps props = {};
   props.allocType = cudaMemAllocationTypePinned;
   props.location.type = cudaMemLocationTypeDevice;
   props.location.id = dev;
   Device d = {};
+  d.ctx = ctx;
   d.ctx_id = id;
   unsigned long long keep = kKeepBytes;
   if (cudaMemPoolCreate(&d.pool, &props) != cudaSuccess ||
@@ -79,8 +95,9 @@ Device* current_device() {
     if (d.pool) cudaMemPoolDestroy(d.pool);
     return nullptr;
   }
-  g_devices[g_n] = d;
-  return &g_devices[g_n++];
+  g_devices[slot] = d;
+  if (slot == g_n) ++g_n;
+  return &g_devices[slot];
 }
 
 }  // namespace
@@ -101,8 +118,8 @@ cudaError_t device_alloc(void** p, size_t bytes, cudaStream_t s) {
   return e;
 }
 
-cudaError_t take_result_words(double** p) {
-  *p = nullptr;
+cudaError_t take_result_words(ResultWords* w) {
+  *w = ResultWords{};
   std::lock_guard<std::mutex> lock(g_mu);
   if (Device* d = current_device()) {
     for (Page& page : d->pages) {
@@ -118,33 +135,40 @@ cudaError_t take_result_words(double** p) {
         const uint64_t bit = 1ull << (k % 64);
         if (word & bit) continue;
         word |= bit;
-        *p = reinterpret_cast<double*>(page.base + k * kWordBytes);
+        w->p = reinterpret_cast<double*>(page.base + k * kWordBytes);
+        w->ctx_id = d->ctx_id;
         return cudaSuccess;
       }
     }
   }
-  return cudaMallocHost(reinterpret_cast<void**>(p), kWordBytes);
+  return cudaMallocHost(reinterpret_cast<void**>(&w->p), kWordBytes);
 }
 
-void give_result_words(double* p) {
-  if (!p) return;
-  const char* c = reinterpret_cast<const char*>(p);
+void give_result_words(const ResultWords& w) {
+  if (!w.p) return;
+  if (!w.ctx_id) {
+    cudaFreeHost(w.p);
+    return;
+  }
+  const char* c = reinterpret_cast<const char*>(w.p);
   std::lock_guard<std::mutex> lock(g_mu);
-  for (int i = 0; i < g_n; ++i)
-    for (int j = 0; j < kPages; ++j) {
-      Page& page = g_devices[i].pages[j];
-      if (!page.base || c < page.base || c >= page.base + kPageBytes) continue;
-      const int k = (int)((c - page.base) / kWordBytes);
-      page.used[k / 64] &= ~(1ull << (k % 64));
-      bool any = false;
-      for (uint64_t w : page.used) any |= w != 0;
-      if (!any && j > 0) {
-        cudaFreeHost(page.base);
-        page.base = nullptr;
-      }
-      return;
+  Device* d = find_device(w.ctx_id);
+  if (!d) return;  // that context is gone, and its pages with it
+  for (int j = 0; j < kPages; ++j) {
+    Page& page = d->pages[j];
+    if (!page.base || c < page.base || c >= page.base + kPageBytes) continue;
+    const int k = (int)((c - page.base) / kWordBytes);
+    page.used[k / 64] &= ~(1ull << (k % 64));
+    bool any = false;
+    for (uint64_t u : page.used) any |= u != 0;
+    CUcontext ctx = nullptr;
+    unsigned long long id = 0;
+    if (!any && j > 0 && current_context(&ctx, &id) && id == w.ctx_id) {
+      cudaFreeHost(page.base);
+      page.base = nullptr;
     }
-  cudaFreeHost(p);
+    return;
+  }
 }
 
 }  // namespace hsg
