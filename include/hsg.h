@@ -444,6 +444,14 @@ hsg_status hsg_test_fail_alloc(int k);
 hsg_status hsg_test_stall_tensor_loads(int on);
 
 /*
+ * For tests of small lattices on a device that cannot place their thread-block
+ * cluster (a partition of a GPU): on = 1 takes the device for one, so that they are
+ * swept by the half-sweep kernels (the same results); on = 0 restores;
+ * HSG_EINVAL otherwise.  Process-wide.  Library-specific.
+ */
+hsg_status hsg_test_no_clusters(int on);
+
+/*
  * E/N of a lattice held in the caller's own device memory, without any
  * allocation.  The paper has no counterpart: this entry point exists for
  * callers that cannot let a library allocate device memory -- applications

@@ -523,12 +523,14 @@ int main_update(const hsg_schedule* s) {
 // Whether hsg_sweep runs schedule s in the resident kernel
 // (hsg_resident.cu): AUTO only, and neither under the profiler, whose classes
 // are single half-sweeps, nor while the caller captures the stream (what a
-// capture takes, and what it refuses, stays with the half-sweep launches).
+// capture takes, and what it refuses, stays with the half-sweep launches),
+// and where the device can place its cluster.
 bool use_resident(const hsg_ctx* c, const hsg_schedule* s) {
   if (s->kernel != HSG_KERNEL_AUTO || c->prof || !hsg::resident_takes(main_update(s), c->L, s->hits)) return false;
   if (s->kind == HSG_NONE && s->n_or == 0) return false;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  return cudaStreamIsCapturing(c->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
+  return hsg::resident_fits(main_update(s), c->L, 1, false, c->sm_count);
 }
 
 // n_sweeps sweeps in the resident kernel, one launch up to each energy due.
@@ -1065,6 +1067,12 @@ hsg_status hsg_philox(uint64_t seed, uint32_t sample, uint32_t replica, uint32_t
 hsg_status hsg_test_stall_tensor_loads(int on) {
   if (on < 0 || on > 3) return fail(nullptr, HSG_EINVAL, "on must be 0 .. 3");
   g_test_stall_boxes.store(on);
+  return HSG_OK;
+}
+
+hsg_status hsg_test_no_clusters(int on) {
+  if (on != 0 && on != 1) return fail(nullptr, HSG_EINVAL, "on must be 0 or 1");
+  hsg::test_no_clusters(on == 1);
   return HSG_OK;
 }
 

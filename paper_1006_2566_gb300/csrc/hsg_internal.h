@@ -195,6 +195,10 @@ constexpr int kResidentMaxL = 32;
 constexpr unsigned long long kResidentPoolSites = 640 * 1024;
 // `upd`: the main update's kind, or U_OR for over-relaxation only.
 bool resident_takes(int upd, int L, int hits);
+// Whether the current device can place the cluster that a lattice of side L takes
+// (alone, or as one of a pool's n of this side); never under test_no_clusters.
+bool resident_fits(int upd, int L, int n, bool pool, int sm_count);
+void test_no_clusters(bool on);
 cudaError_t launch_resident(int upd, const ResidentArgs& a, int sm_count, cudaStream_t s);
 
 // A batch of pool lattices swept by one launch per half-sweep (hsg_batch.cu),

@@ -569,7 +569,10 @@ bool resident_pool(const hsg_pool* p, const hsg_schedule* s) {
     const uint64_t n = (uint64_t)sl.L * sl.L * sl.L;
     sites += sl.L < 26 ? n : n + n / 4;
   }
-  return sites > 0 && sites <= hsg::kResidentPoolSites;
+  if (sites == 0 || sites > hsg::kResidentPoolSites) return false;
+  for (int L = 4; L < hsg::kBatchMinL; L += 2)
+    if (p->small_count[L] > 0 && !hsg::resident_fits(main_update(s), L, p->small_count[L], true, p->sm_count)) return false;
+  return true;
 }
 
 // n_sweeps sweeps of the small lattices, side by side: each side's launch on the

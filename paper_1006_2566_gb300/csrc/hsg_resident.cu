@@ -39,6 +39,8 @@
 // + 2 OR 56 -> 63), hence kResidentPoolSites.
 // A loop over sites with the indices formed and the bonds loaded for each
 // (so that larger lattices fit too): 7.9 us at L = 16, 24.9 against 14.0 at L = 40.
+#include <atomic>
+
 #include "hsg_device.cuh"
 #include "hsg_internal.h"
 
@@ -48,6 +50,7 @@ namespace {
 // The lattices this kernel takes: every CTA's planes fit one thread per site
 // pair.  L = 32 is 1024 threads on each of 16 CTAs.
 constexpr uint32_t kThreadsMax = 1024;
+constexpr size_t kSharedMax = 96 * 1024;
 
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
@@ -246,12 +249,53 @@ uint32_t pool_cluster_size(uint32_t L, int total, int sm_count) {
   return c;
 }
 
+cudaLaunchAttribute cluster_attribute(uint32_t cluster) {
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = cluster;
+  at.val.clusterDim.y = 1;
+  at.val.clusterDim.z = 1;
+  return at;
+}
+
+std::atomic<bool> g_no_clusters{false};  // test hook: hsg_test_no_clusters
+
+// Sets the kernel's attributes and asks whether the device ever has room for a
+// cluster of this size (with the most threads and shared memory that a launch asks
+// for), once per kernel, size (a power of two up to 16) and device: a GPU whose
+// visible SMs come in smaller groups (a partition) has none for sixteen CTAs.
+template <int U, bool POOL>
+bool fits_u(uint32_t cluster) {
+  constexpr int kNo = 1, kYes = 2;
+  static PerDevice known[5];
+  int log2 = 0;
+  while ((1u << log2) < cluster) ++log2;
+  cudaError_t e = cudaSuccess;
+  std::atomic<int>* slot = device_slot(known[log2], &e);
+  if (!slot) return false;
+  int answer = slot->load(std::memory_order_acquire);
+  if (answer == 0) {
+    e = cudaFuncSetAttribute(k_resident<U, POOL>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSharedMax);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_resident<U, POOL>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaLaunchAttribute at = cluster_attribute(cluster);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(cluster);
+    cfg.blockDim = dim3(kThreadsMax);
+    cfg.dynamicSmemBytes = kSharedMax;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, k_resident<U, POOL>, &cfg);
+    if (e != cudaSuccess) cudaGetLastError();
+    answer = e == cudaSuccess && n > 0 ? kYes : kNo;
+    slot->store(answer, std::memory_order_release);
+  }
+  return answer == kYes;
+}
+
 template <int U, bool POOL>
 cudaError_t launch_u(ResidentArgs a, uint32_t cluster, cudaStream_t s) {
-  static PerDevice configured;
-  cudaError_t e = cudaSuccess;
-  std::atomic<int>* slot = device_slot(configured, &e);
-  if (!slot) return e;
+  if (!fits_u<U, POOL>(cluster)) return cudaErrorInvalidValue;
   a.cluster = cluster;
   a.max_planes = (a.L + cluster - 1) / cluster;
   a.Lh = a.L / 2;
@@ -261,23 +305,13 @@ cudaError_t launch_u(ResidentArgs a, uint32_t cluster, cudaStream_t s) {
   a.by_Lh = make_fastdiv(a.Lh);
   const uint32_t threads = cta_threads(a.L, cluster);
   if (threads > kThreadsMax || a.n < 1) return cudaErrorInvalidValue;
-  if (slot->load(std::memory_order_acquire) == 0) {
-    e = cudaFuncSetAttribute(k_resident<U, POOL>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_resident<U, POOL>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    slot->store(1, std::memory_order_release);
-  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(cluster * (uint32_t)a.n);
   cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = (size_t)2 * (a.max_planes + 2) * a.plane * sizeof(float4);
   cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = cluster;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
+  cudaLaunchAttribute at = cluster_attribute(cluster);
+  cfg.attrs = &at;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, k_resident<U, POOL>, a);
 }
@@ -295,6 +329,19 @@ cudaError_t launch_kinds(int upd, const ResidentArgs& a, uint32_t cluster, cudaS
   }
 }
 
+template <bool POOL>
+bool fits_kinds(int upd, uint32_t cluster) {
+  switch (upd) {
+    case U_OR: return fits_u<U_OR, POOL>(cluster);
+    case U_MET_SPHERE: return fits_u<U_MET_SPHERE, POOL>(cluster);
+    case U_MET_BALL: return fits_u<U_MET_BALL, POOL>(cluster);
+    case U_HB: return fits_u<U_HB, POOL>(cluster);
+    case U_MET_OR_SPHERE: return fits_u<U_MET_OR_SPHERE, POOL>(cluster);
+    case U_MET_OR_BALL: return fits_u<U_MET_OR_BALL, POOL>(cluster);
+    default: return false;
+  }
+}
+
 }  // namespace
 
 // Where sixteen SMs beat the whole GPU on one launch per half-sweep: a hit
@@ -305,6 +352,14 @@ bool resident_takes(int upd, int L, int hits) {
   if (upd == U_OR || upd == U_HB) return true;
   return hits <= (L <= 16 ? 16 : L <= 24 ? 5 : 2);
 }
+
+bool resident_fits(int upd, int L, int n, bool pool, int sm_count) {
+  if (g_no_clusters.load(std::memory_order_relaxed)) return false;
+  return pool ? fits_kinds<true>(upd, pool_cluster_size((uint32_t)L, n, sm_count))
+              : fits_kinds<false>(upd, cluster_size((uint32_t)L));
+}
+
+void test_no_clusters(bool on) { g_no_clusters.store(on); }
 
 cudaError_t launch_resident(int upd, const ResidentArgs& a, int sm_count, cudaStream_t s) {
   if (!resident_takes(upd, (int)a.L, a.hits)) return cudaErrorInvalidValue;

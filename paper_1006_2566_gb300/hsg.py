@@ -92,6 +92,7 @@ _SIGS = {
     "hsg_philox": ([_u64, _u32, _u32, _u32, _u32, _u32, _u32, _vp, _vp], _i),
     "hsg_test_fail_alloc": ([_i], _i),
     "hsg_test_stall_tensor_loads": ([_i], _i),
+    "hsg_test_no_clusters": ([_i], _i),
     "hsg_energy_noalloc": ([_i, _vp, _vp, _vp, _vp], _i),
     "hsg_pool_create": ([ctypes.POINTER(_vp), _u64, _i, _vp], _i),
     "hsg_pool_destroy": ([_vp], _i),
@@ -317,6 +318,11 @@ def hsg_test_fail_alloc(k: int) -> None:
 def hsg_test_stall_tensor_loads(on) -> None:
     """True / 1: the couplings' tensor loads; 2: the colour-1 planes' barriers; 3: both; False / 0: off."""
     _check(_lib.hsg_test_stall_tensor_loads(int(on)))
+
+
+def hsg_test_no_clusters(on) -> None:
+    """True: small lattices are swept as on a device that cannot place their cluster; False: off."""
+    _check(_lib.hsg_test_no_clusters(int(on)))
 
 
 def hsg_energy_noalloc(L: int, spins, J, e_out, stream=None) -> None:

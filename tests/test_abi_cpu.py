@@ -101,3 +101,11 @@ def test_create_without_a_device_reports_cuda_error(lib):
     with pytest.raises(hsg.HsgError) as e:
         hsg.hsg_create(8, seed=1)
     assert e.value.status == hsg.HSG_ECUDA
+
+
+def test_cluster_switch_arguments(lib):
+    from paper_1006_2566_gb300 import hsg
+
+    assert hsg._lib.hsg_test_no_clusters(2) == hsg.HSG_EINVAL
+    assert hsg._lib.hsg_test_no_clusters(-1) == hsg.HSG_EINVAL
+    assert hsg._lib.hsg_test_no_clusters(0) == hsg.HSG_OK

@@ -109,3 +109,24 @@ def test_pools_of_small_lattices_equal_lattices_alone(hsg, sides, n, use_stream)
                 assert np.array_equal(pool.spins(slot), lat.spins()), L
                 assert abs(e[slot] - lat.energy()) <= 2e-6
                 assert pool.sweep_count(slot) == 7
+
+
+@pytest.mark.parametrize("L", [8, 16, 32])
+def test_a_device_without_room_for_the_cluster_takes_half_sweeps(hsg, L):
+    kw = dict(kind=hsg.HSG_HEATBATH, n_or=1, renorm_every=2)
+    out = []
+    try:
+        for on in (0, 1):
+            hsg.hsg_test_no_clusters(on)
+            with hsg.Lattice(L, 3, stream=torch.cuda.Stream()) as lat, hsg.Pool(1 << 22, 2, torch.cuda.Stream()) as pool:
+                lat.generate_couplings()
+                slot = pool.admit(L, 3)
+                n, m = hsg.hsg_launch_count(lat.ctx), hsg.hsg_pool_launch_count(pool.pool)
+                lat.sweep(hsg.schedule(**kw), 5)
+                pool.sweep(hsg.schedule(**kw), 5)
+                n, m = hsg.hsg_launch_count(lat.ctx) - n, hsg.hsg_pool_launch_count(pool.pool) - m
+                out.append((lat.spins(), pool.spins(slot), n, m))
+    finally:
+        hsg.hsg_test_no_clusters(0)
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+    assert out[0][2] == 1 and out[1][2] >= 20 and out[1][3] >= 20  # 5 x 4 half-sweeps and what goes with them
