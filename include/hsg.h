@@ -451,6 +451,10 @@ hsg_status hsg_test_stall_tensor_loads(int on);
  */
 hsg_status hsg_test_no_clusters(int on);
 
+/* For tests of the sweeps' CUDA graphs: how many graphs hsg_sweep has captured and how
+ * many it has launched on this context.  Errors: HSG_EINVAL (NULL argument). */
+hsg_status hsg_test_graph_counts(hsg_ctx* ctx, uint64_t* captured, uint64_t* launched);
+
 /*
  * E/N of a lattice held in the caller's own device memory, without any
  * allocation.  The paper has no counterpart: this entry point exists for

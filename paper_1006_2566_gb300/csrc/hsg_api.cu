@@ -87,6 +87,7 @@ struct hsg_ctx {
   hsg_schedule gsched{};
   int gvariant = 0, gperiod = 0, glaunches = 0;
   double* gelog = nullptr;
+  uint64_t captures = 0, replays = 0;  // for hsg_test_graph_counts
   // While a period is captured: the sweep's number in it (the counter kernel
   // then runs once, at the period's end); -1 otherwise.
   int captured = -1;
@@ -447,9 +448,13 @@ bool same_schedule(const hsg_schedule& a, const hsg_schedule& b) {
          a.T == b.T && a.renorm_every == b.renorm_every && a.energy_every == b.energy_every && a.kernel == b.kernel;
 }
 
+// The captured graph is one of s, whichever spin buffer it starts from.
+bool same_graph(const hsg_ctx* c, const hsg_schedule* s, int variant) {
+  return c->gexec && same_schedule(c->gsched, *s) && c->gvariant == variant && c->gelog == c->elog;
+}
+
 bool graph_matches(const hsg_ctx* c, const hsg_schedule* s, int variant, int period) {
-  return c->gexec && same_schedule(c->gsched, *s) && c->gvariant == variant && c->gperiod == period &&
-         c->gelog == c->elog && c->gspins == c->spins;
+  return same_graph(c, s, variant) && c->gperiod == period && c->gspins == c->spins;
 }
 
 // Sweeps in one graph for a schedule without cadences, n of them asked for:
@@ -501,6 +506,7 @@ hsg_status capture_period(hsg_ctx* c, const hsg_schedule* s, int variant, int pe
     c->gexec = nullptr;
     return cuda_fail(c, e, "sweep graph");
   }
+  c->captures += 1;
   c->gsched = *s;
   c->gvariant = variant;
   c->gperiod = period;
@@ -775,6 +781,7 @@ hsg_status hsg_sweep(hsg_ctx* c, const hsg_schedule* s, int n_sweeps) {
   }
   if (swaps > 0 && (st = prepare_bond_boxes(c)) != HSG_OK) return st;
   SweepGroup group_guard(c);
+  int k = 0;
   // Sweeps run in periods of P = lcm(renorm_every, energy_every) sweeps.  On a non-default stream and without the
   // profiler, a period that starts at a multiple of P is captured once as a
   // CUDA graph (the kernels read the sweep counter and the energy-log
@@ -789,15 +796,23 @@ hsg_status hsg_sweep(hsg_ctx* c, const hsg_schedule* s, int n_sweeps) {
   if (s->renorm_every > 0) period = std::lcm(period, (long long)s->renorm_every);
   if (s->energy_every > 0) period = std::lcm(period, (long long)s->energy_every);
   if ((period * swaps) % 2 == 1) period *= 2;
-  if (!cadence && n_sweeps > 0) period = free_period(c, s, variant, n_sweeps, (int)period);
+  if (!cadence && n_sweeps > 0) {
+    // The graph there is starts from the other buffer (an odd number of swaps has
+    // been launched since): one direct sweep leads back to it.
+    if (swaps % 2 == 1 && !c->prof && same_graph(c, s, variant) && c->gspins == c->spins_alt) {
+      if ((st = enqueue_one_sweep(c, s)) != HSG_OK) return st;
+      k = 1;
+    }
+    period = free_period(c, s, variant, n_sweeps - k, (int)period);
+  }
   const bool graphs = c->stream != nullptr && !c->prof && period <= kMaxGraphPeriod;
-  int k = 0;
   while (k < n_sweeps) {
     if (graphs && (!cadence || c->sweep % (uint64_t)period == 0) && n_sweeps - k >= period) {
       if (!graph_matches(c, s, variant, (int)period) && (st = capture_period(c, s, variant, (int)period)) != HSG_OK)
         return st;
       cudaError_t e = cudaGraphLaunch(c->gexec, c->stream);
       if (e != cudaSuccess) return cuda_fail(c, e, "sweep graph launch");
+      c->replays += 1;
       c->launches += (uint64_t)c->glaunches;
       c->sweep += (uint64_t)period;
       if (s->energy_every > 0) c->elog_n += (int)(period / s->energy_every);
@@ -1067,6 +1082,13 @@ hsg_status hsg_philox(uint64_t seed, uint32_t sample, uint32_t replica, uint32_t
 hsg_status hsg_test_stall_tensor_loads(int on) {
   if (on < 0 || on > 3) return fail(nullptr, HSG_EINVAL, "on must be 0 .. 3");
   g_test_stall_boxes.store(on);
+  return HSG_OK;
+}
+
+hsg_status hsg_test_graph_counts(hsg_ctx* c, uint64_t* captured, uint64_t* launched) {
+  if (!c || !captured || !launched) return fail(c, HSG_EINVAL, "NULL argument");
+  *captured = c->captures;
+  *launched = c->replays;
   return HSG_OK;
 }
 

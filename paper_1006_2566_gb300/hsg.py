@@ -93,6 +93,7 @@ _SIGS = {
     "hsg_test_fail_alloc": ([_i], _i),
     "hsg_test_stall_tensor_loads": ([_i], _i),
     "hsg_test_no_clusters": ([_i], _i),
+    "hsg_test_graph_counts": ([_vp, ctypes.POINTER(_u64), ctypes.POINTER(_u64)], _i),
     "hsg_energy_noalloc": ([_i, _vp, _vp, _vp, _vp], _i),
     "hsg_pool_create": ([ctypes.POINTER(_vp), _u64, _i, _vp], _i),
     "hsg_pool_destroy": ([_vp], _i),
@@ -323,6 +324,13 @@ def hsg_test_stall_tensor_loads(on) -> None:
 def hsg_test_no_clusters(on) -> None:
     """True: small lattices are swept as on a device that cannot place their cluster; False: off."""
     _check(_lib.hsg_test_no_clusters(int(on)))
+
+
+def hsg_test_graph_counts(ctx):
+    """(graphs captured, graphs launched) by the sweeps of this context."""
+    a, b = _u64(0), _u64(0)
+    _check(_lib.hsg_test_graph_counts(ctx, ctypes.byref(a), ctypes.byref(b)), ctx)
+    return a.value, b.value
 
 
 def hsg_energy_noalloc(L: int, spins, J, e_out, stream=None) -> None:
