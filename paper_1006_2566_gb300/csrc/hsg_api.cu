@@ -26,7 +26,9 @@ constexpr int kMaxL = 1624;    // L^3 < 2^32: site indices are 32-bit Philox cou
 constexpr int kElogInit = 64;
 constexpr int kCounters = 4;   // words at hsg_ctx::d_ctr
 constexpr long long kMaxGraphPeriod = 64;  // longest sweep period captured as one graph
-constexpr int kGraphSweeps = 16;           // sweeps in one graph without cadences
+constexpr int kGraphSweeps = 16;           // most sweeps in one graph without cadences,
+constexpr int kGraphLaunches = 64;         // and most launches of more than one sweep
+constexpr int kOnceMaxL = 72;              // sides up to which a graph that runs once is not captured
 
 thread_local std::string g_thread_error;
 int g_fail_alloc_countdown = 0;  // test hook: k-th allocation from now fails
@@ -88,6 +90,8 @@ struct hsg_ctx {
   int gvariant = 0, gperiod = 0, glaunches = 0;
   double* gelog = nullptr;
   uint64_t captures = 0, replays = 0;  // for hsg_test_graph_counts
+  hsg_schedule last{};                 // of the last hsg_sweep
+  bool have_last = false;
   // While a period is captured: the sweep's number in it (the counter kernel
   // then runs once, at the period's end); -1 otherwise.
   int captured = -1;
@@ -457,19 +461,32 @@ bool graph_matches(const hsg_ctx* c, const hsg_schedule* s, int variant, int per
   return same_graph(c, s, variant) && c->gperiod == period && c->gspins == c->spins;
 }
 
+// Half-sweep and over-relaxation launches of one sweep (at least 1).
+int sweep_launches(const hsg_schedule* s, int variant) {
+  return std::max(1, (s->kind != HSG_NONE ? 2 : 0) + (variant == hsg::V_WAVE ? 1 : 2) * s->n_or);
+}
+
 // Sweeps in one graph for a schedule without cadences, n of them asked for:
-// the largest divisor of n up to kGraphSweeps (a multiple of `unit`), or
-// kGraphSweeps if none is half as long; a graph that is there is kept unless
-// eight of it would be replayed.
+// the largest divisor of n up to what one graph is given (a multiple of
+// `unit`), or that many if none is half as long; a graph that is there is kept
+// if it is half as long or n is less than eight of it.  One graph is given up to
+// kGraphSweeps sweeps, but no more than kGraphLaunches launches or an eighth of n:
+// capturing and instantiating costs 2.9 us a launch, which a schedule that is used
+// once (a temperature per call) does not earn back.  L = 40, heat-bath + 20 OR, a new T
+// for every 5, 10, 16 sweeps, us a call: 611, 1195, 1895 with all of them in a graph,
+// 307, 598, 947 with one each; sweep(31) again and again 1683 with 16, 1795 with one.
 int free_period(const hsg_ctx* c, const hsg_schedule* s, int variant, int n, int unit) {
-  if (c->gexec && graph_matches(c, s, variant, c->gperiod) && c->gperiod % unit == 0 &&
-      (c->gperiod >= kGraphSweeps / 2 || n < 8 * c->gperiod))
+  const int fit = std::max(kGraphLaunches / sweep_launches(s, variant), n / 8);
+  const int most = std::max(1, std::min(kGraphSweeps, fit) / unit) * unit;
+  if (graph_matches(c, s, variant, c->gperiod) && c->gperiod % unit == 0 &&
+      (2 * c->gperiod >= most || n < 8 * c->gperiod))
     return c->gperiod;
   if (n < 2 * unit) return unit;
+  if (n <= most) return n / unit * unit;
   int best = unit;
-  for (int d = unit; d <= kGraphSweeps && d <= n; d += unit)
+  for (int d = unit; d <= most; d += unit)
     if (n % d == 0) best = d;
-  return best >= kGraphSweeps / 2 || n <= kGraphSweeps ? (n <= kGraphSweeps ? n / unit * unit : best) : kGraphSweeps;
+  return 2 * best >= most ? best : most;
 }
 
 // Capture `period` sweeps starting at the current counter (with cadences a
@@ -526,6 +543,12 @@ int main_update(const hsg_schedule* s) {
   }
 }
 
+// Whether the caller captures the context's stream.
+bool stream_captured(const hsg_ctx* c) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+}
+
 // Whether hsg_sweep runs schedule s in the resident kernel
 // (hsg_resident.cu): AUTO only, and neither under the profiler, whose classes
 // are single half-sweeps, nor while the caller captures the stream (what a
@@ -534,8 +557,7 @@ int main_update(const hsg_schedule* s) {
 bool use_resident(const hsg_ctx* c, const hsg_schedule* s) {
   if (s->kernel != HSG_KERNEL_AUTO || c->prof || !hsg::resident_takes(main_update(s), c->L, s->hits)) return false;
   if (s->kind == HSG_NONE && s->n_or == 0) return false;
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
+  if (stream_captured(c)) return false;
   return hsg::resident_fits(main_update(s), c->L, 1, false, c->sm_count);
 }
 
@@ -805,7 +827,16 @@ hsg_status hsg_sweep(hsg_ctx* c, const hsg_schedule* s, int n_sweeps) {
     }
     period = free_period(c, s, variant, n_sweeps - k, (int)period);
   }
-  const bool graphs = c->stream != nullptr && !c->prof && period <= kMaxGraphPeriod;
+  bool graphs = c->stream != nullptr && !c->prof && period <= kMaxGraphPeriod;
+  // A new schedule's graph that this call would launch only once is not captured
+  // where the host cannot hide it behind the kernels: direct launches cost it 1.65 us
+  // each against 2.9.  A new T for each sweep of heat-bath + 20 OR, us, captured / direct:
+  // L = 40 132 / 75, 66 140 / 109, 100 200 / 266; + 2 OR: 32 / 16, 38 / 20, 45 / 44.
+  if (graphs && c->L <= kOnceMaxL && n_sweeps - k < 2 * period && !(c->have_last && same_schedule(c->last, *s)) &&
+      !same_graph(c, s, variant) && !stream_captured(c))
+    graphs = false;
+  c->last = *s;
+  c->have_last = true;
   while (k < n_sweeps) {
     if (graphs && (!cadence || c->sweep % (uint64_t)period == 0) && n_sweeps - k >= period) {
       if (!graph_matches(c, s, variant, (int)period) && (st = capture_period(c, s, variant, (int)period)) != HSG_OK)

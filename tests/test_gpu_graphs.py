@@ -32,6 +32,29 @@ def run(hsg, L, sched, calls, graphs=True):
 @pytest.mark.parametrize("calls,replayed", [((5,) * 8, 8), ((3,) * 8, 8), ((4, 1, 4, 1, 4), 2), ((5, 4, 5), 2)])
 def test_odd_calls_with_odd_buffer_swaps_keep_their_graph(hsg, calls, replayed):
     sched = hsg.schedule(kind=hsg.HSG_HEATBATH, T=0.5, n_or=1, kernel=hsg.HSG_KERNEL_WAVE)
-    spins, captured, launched = run(hsg, 36, sched, calls)
-    assert np.array_equal(spins, run(hsg, 36, sched, (sum(calls),), graphs=False)[0])
+    spins, captured, launched = run(hsg, 74, sched, calls)
+    assert np.array_equal(spins, run(hsg, 74, sched, (sum(calls),), graphs=False)[0])
     assert captured == 1 and launched >= replayed
+
+
+@pytest.mark.parametrize("L,n_or,n,captured,launched", [
+    (40, 20, 5, 1, 5),    # 42 launches a sweep: one sweep in a graph
+    (40, 20, 1, 0, 0),    # a graph that would run once is not captured
+    (40, 2, 10, 0, 0),
+    (40, 2, 20, 1, 2),    # 60 launches in a graph
+    (40, 0, 64, 1, 4),    # 16 sweeps
+    (34, 31, 3, 1, 3),    # 64 launches a sweep
+    (40, 20, 128, 1, 8),  # an eighth of the call
+    (74, 20, 1, 1, 1)])   # where the host is hidden
+def test_a_new_schedule_captures_no_more_than_it_replays(hsg, L, n_or, n, captured, launched):
+    sched = hsg.schedule(kind=hsg.HSG_HEATBATH, T=0.5, n_or=n_or)
+    spins, *counts = run(hsg, L, sched, (n,))
+    assert np.array_equal(spins, run(hsg, L, sched, (n,), graphs=False)[0])
+    assert counts == [captured, launched]
+
+
+def test_a_schedule_seen_twice_has_its_graph(hsg):
+    sched = hsg.schedule(kind=hsg.HSG_HEATBATH, T=0.5, n_or=2)
+    assert run(hsg, 40, sched, (5, 5, 5, 5))[1:] == (1, 3)
+    cadence = hsg.schedule(kind=hsg.HSG_HEATBATH, T=0.5, n_or=2, renorm_every=5, energy_every=5)
+    assert run(hsg, 40, cadence, (5, 5, 5, 5))[1:] == (1, 3)
