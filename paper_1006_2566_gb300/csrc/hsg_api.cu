@@ -44,6 +44,16 @@ struct ProfRec {
 
 }  // namespace
 
+// Some sweeps captured as a CUDA graph, replayed while the schedule, the kernel
+// variant, the energy log buffer and the spin buffer stay the same.
+struct SweepGraph {
+  cudaGraphExec_t exec = nullptr;
+  hsg_schedule sched{};
+  int variant = 0, period = 0, launches = 0;
+  double* elog = nullptr;
+  float4* spins = nullptr;  // current spin buffer when it was captured
+};
+
 struct hsg_ctx {
   int L = 0, Lh = 0;
   long long N = 0, Nh = 0;
@@ -83,19 +93,16 @@ struct hsg_ctx {
   // temporally blocked sweep whose bounded wait for a bond box gave up.  [3]
   // counts the energy kernel's blocks, zero between launches.
   unsigned long long* d_ctr = nullptr;
-  // One captured period of sweeps (see hsg_sweep), replayed while the
-  // schedule, the kernel variant and the energy log buffer stay the same.
-  cudaGraphExec_t gexec = nullptr;
-  hsg_schedule gsched{};
-  int gvariant = 0, gperiod = 0, glaunches = 0;
-  double* gelog = nullptr;
-  uint64_t captures = 0, replays = 0;  // for hsg_test_graph_counts
-  hsg_schedule last{};                 // of the last hsg_sweep
-  bool have_last = false;
+  // Captured sweeps (see hsg_sweep): one graph for the bulk of a call and, without
+  // cadences, one for what is left over or for calls shorter than the first.
+  SweepGraph graph, short_graph;
+  int short_want = 0;  // sweeps that the last call found no graph for (0: none)
   // While a period is captured: the sweep's number in it (the counter kernel
   // then runs once, at the period's end); -1 otherwise.
   int captured = -1;
-  float4* gspins = nullptr;  // current spin buffer when the period was captured
+  uint64_t captures = 0, replays = 0;  // for hsg_test_graph_counts
+  hsg_schedule last{};                 // of the last hsg_sweep
+  bool have_last = false;
   std::string err;
 };
 
@@ -206,7 +213,8 @@ void release(hsg_ctx* c) {
   dev_free(c->elog, s);
   dev_free(c->d_ctr, s);
   cudaStreamSynchronize(s);
-  if (c->gexec) cudaGraphExecDestroy(c->gexec);
+  if (c->graph.exec) cudaGraphExecDestroy(c->graph.exec);
+  if (c->short_graph.exec) cudaGraphExecDestroy(c->short_graph.exec);
   hsg::give_result_words(c->words);
   for (auto& r : c->recs) {
     cudaEventDestroy(r.start);
@@ -452,13 +460,13 @@ bool same_schedule(const hsg_schedule& a, const hsg_schedule& b) {
          a.T == b.T && a.renorm_every == b.renorm_every && a.energy_every == b.energy_every && a.kernel == b.kernel;
 }
 
-// The captured graph is one of s, whichever spin buffer it starts from.
-bool same_graph(const hsg_ctx* c, const hsg_schedule* s, int variant) {
-  return c->gexec && same_schedule(c->gsched, *s) && c->gvariant == variant && c->gelog == c->elog;
+// Graph g is one of s, whichever spin buffer it starts from.
+bool same_graph(const hsg_ctx* c, const SweepGraph& g, const hsg_schedule* s, int variant) {
+  return g.exec && same_schedule(g.sched, *s) && g.variant == variant && g.elog == c->elog;
 }
 
-bool graph_matches(const hsg_ctx* c, const hsg_schedule* s, int variant, int period) {
-  return same_graph(c, s, variant) && c->gperiod == period && c->gspins == c->spins;
+bool graph_matches(const hsg_ctx* c, const SweepGraph& g, const hsg_schedule* s, int variant) {
+  return same_graph(c, g, s, variant) && g.spins == c->spins;
 }
 
 // Half-sweep and over-relaxation launches of one sweep (at least 1).
@@ -478,9 +486,8 @@ int sweep_launches(const hsg_schedule* s, int variant) {
 int free_period(const hsg_ctx* c, const hsg_schedule* s, int variant, int n, int unit) {
   const int fit = std::max(kGraphLaunches / sweep_launches(s, variant), n / 8);
   const int most = std::max(1, std::min(kGraphSweeps, fit) / unit) * unit;
-  if (graph_matches(c, s, variant, c->gperiod) && c->gperiod % unit == 0 &&
-      (2 * c->gperiod >= most || n < 8 * c->gperiod))
-    return c->gperiod;
+  const int there = graph_matches(c, c->graph, s, variant) ? c->graph.period : 0;
+  if (there > 0 && there % unit == 0 && (2 * there >= most || n < 8 * there)) return there;
   if (n < 2 * unit) return unit;
   if (n <= most) return n / unit * unit;
   int best = unit;
@@ -490,11 +497,11 @@ int free_period(const hsg_ctx* c, const hsg_schedule* s, int variant, int n, int
 }
 
 // Capture `period` sweeps starting at the current counter (with cadences a
-// multiple of the period) into c->gexec.  Capturing runs nothing, so the host mirrors
+// multiple of the period) into *g.  Capturing runs nothing, so the host mirrors
 // are restored afterwards.
-hsg_status capture_period(hsg_ctx* c, const hsg_schedule* s, int variant, int period) {
-  if (c->gexec) cudaGraphExecDestroy(c->gexec);
-  c->gexec = nullptr;
+hsg_status capture_period(hsg_ctx* c, const hsg_schedule* s, int variant, int period, SweepGraph* g) {
+  if (g->exec) cudaGraphExecDestroy(g->exec);
+  g->exec = nullptr;
   const uint64_t sweep0 = c->sweep, launches0 = c->launches;
   const int elog0 = c->elog_n;
   float4* const spins0 = c->spins;
@@ -508,27 +515,53 @@ hsg_status capture_period(hsg_ctx* c, const hsg_schedule* s, int variant, int pe
   }
   c->captured = -1;
   if (st == HSG_OK) st = run_advance(c, (uint64_t)period);
-  cudaGraph_t g = nullptr;
-  e = cudaStreamEndCapture(c->stream, &g);
-  c->glaunches = (int)(c->launches - launches0);
+  cudaGraph_t captured = nullptr;
+  e = cudaStreamEndCapture(c->stream, &captured);
+  const int launches = (int)(c->launches - launches0);
   c->launches = launches0;
   c->sweep = sweep0;
   c->elog_n = elog0;
   c->spins = spins0;
   c->spins_alt = alt0;
-  if (st == HSG_OK && e == cudaSuccess) e = cudaGraphInstantiate(&c->gexec, g, 0);
-  if (g) cudaGraphDestroy(g);
+  if (st == HSG_OK && e == cudaSuccess) e = cudaGraphInstantiate(&g->exec, captured, 0);
+  if (captured) cudaGraphDestroy(captured);
   if (st != HSG_OK) return st;
   if (e != cudaSuccess) {
-    c->gexec = nullptr;
+    g->exec = nullptr;
     return cuda_fail(c, e, "sweep graph");
   }
   c->captures += 1;
-  c->gsched = *s;
-  c->gvariant = variant;
-  c->gperiod = period;
-  c->gelog = c->elog;
-  c->gspins = spins0;
+  g->sched = *s;
+  g->variant = variant;
+  g->period = period;
+  g->launches = launches;
+  g->elog = c->elog;
+  g->spins = spins0;
+  return HSG_OK;
+}
+
+// The graph for the last `left` sweeps of a call without cadences, fewer than the
+// bulk's graph holds: the short graph that is there, or, where the call before
+// had as many left, one captured now; else nullptr (they are launched directly).
+// Calls of changing lengths so end up with a graph that divides what they leave.
+// us a call of sweep(n) and energy() after a long call, direct launches / short graph,
+// heat-bath + n_or over-relaxation sweeps:
+//   n_or = 0   n = 1: L = 40 23.9 / 23.0, 66 29.5 / 27.4, 128 54.2 / 51.2; n = 3: 33.4 / 29.9, 43.5 / 40.0, 115 / 101
+//   n_or = 2   n = 1: 29.5 / 27.7, 38.9 / 37.0, 88 / 79; n = 5: 74 / 62, 107 / 94, 350 / 287
+//   n_or = 20  n = 1: 88 / 73, 129 / 113, 394 / 319; n = 5: 367 / 288, 552 / 471, 1864 / 1486
+hsg_status pick_short(hsg_ctx* c, const hsg_schedule* s, int variant, int left, int unit, SweepGraph** g) {
+  *g = nullptr;
+  const int len = left / unit * unit;
+  if (len == 0) return HSG_OK;
+  if (graph_matches(c, c->short_graph, s, variant) && c->short_graph.period <= left) {
+    *g = &c->short_graph;
+  } else if (c->short_want == len) {
+    const hsg_status st = capture_period(c, s, variant, len, &c->short_graph);
+    if (st != HSG_OK) return st;
+    *g = &c->short_graph;
+  } else {
+    c->short_want = len;
+  }
   return HSG_OK;
 }
 
@@ -811,43 +844,56 @@ hsg_status hsg_sweep(hsg_ctx* c, const hsg_schedule* s, int n_sweeps) {
   // directly.  Both paths issue the same kernels in the same order.  A
   // captured period leaves the spins in the buffer it found them in (an even
   // number of buffer swaps), so that the graph can be replayed.  Without
-  // cadences the period is as many sweeps as one graph is given: a graph of
-  // one sweep costs 4-8 us of launching each.
+  // cadences the period is as many sweeps as one graph is given (free_period: a
+  // graph of one sweep costs 4-8 us of launching each), and what is left over may have
+  // a graph of its own (pick_short).
   const bool cadence = s->renorm_every > 0 || s->energy_every > 0;
   long long period = 1;
   if (s->renorm_every > 0) period = std::lcm(period, (long long)s->renorm_every);
   if (s->energy_every > 0) period = std::lcm(period, (long long)s->energy_every);
   if ((period * swaps) % 2 == 1) period *= 2;
+  const int unit = cadence ? 1 : (int)period;  // without cadences: 1, or 2 with an odd number of swaps
   if (!cadence && n_sweeps > 0) {
     // The graph there is starts from the other buffer (an odd number of swaps has
     // been launched since): one direct sweep leads back to it.
-    if (swaps % 2 == 1 && !c->prof && same_graph(c, s, variant) && c->gspins == c->spins_alt) {
+    if (swaps % 2 == 1 && !c->prof && same_graph(c, c->graph, s, variant) && c->graph.spins == c->spins_alt) {
       if ((st = enqueue_one_sweep(c, s)) != HSG_OK) return st;
       k = 1;
     }
-    period = free_period(c, s, variant, n_sweeps - k, (int)period);
+    period = free_period(c, s, variant, n_sweeps - k, unit);
   }
+  const bool seen = c->have_last && same_schedule(c->last, *s);
+  if (!seen) c->short_want = 0;
   bool graphs = c->stream != nullptr && !c->prof && period <= kMaxGraphPeriod;
   // A new schedule's graph that this call would launch only once is not captured
   // where the host cannot hide it behind the kernels: direct launches cost it 1.65 us
   // each against 2.9.  A new T for each sweep of heat-bath + 20 OR, us, captured / direct:
   // L = 40 132 / 75, 66 140 / 109, 100 200 / 266; + 2 OR: 32 / 16, 38 / 20, 45 / 44.
-  if (graphs && c->L <= kOnceMaxL && n_sweeps - k < 2 * period && !(c->have_last && same_schedule(c->last, *s)) &&
-      !same_graph(c, s, variant) && !stream_captured(c))
+  if (graphs && c->L <= kOnceMaxL && n_sweeps - k < 2 * period && !seen &&
+      !same_graph(c, c->graph, s, variant) && !stream_captured(c))
     graphs = false;
   c->last = *s;
   c->have_last = true;
+  bool look_short = graphs && !cadence;  // asked once a call where there is none
   while (k < n_sweeps) {
+    SweepGraph* g = nullptr;
     if (graphs && (!cadence || c->sweep % (uint64_t)period == 0) && n_sweeps - k >= period) {
-      if (!graph_matches(c, s, variant, (int)period) && (st = capture_period(c, s, variant, (int)period)) != HSG_OK)
+      g = &c->graph;
+      if ((g->period != period || !graph_matches(c, *g, s, variant)) &&
+          (st = capture_period(c, s, variant, (int)period, g)) != HSG_OK)
         return st;
-      cudaError_t e = cudaGraphLaunch(c->gexec, c->stream);
+    } else if (look_short) {
+      if ((st = pick_short(c, s, variant, n_sweeps - k, unit, &g)) != HSG_OK) return st;
+      look_short = g != nullptr;
+    }
+    if (g) {
+      cudaError_t e = cudaGraphLaunch(g->exec, c->stream);
       if (e != cudaSuccess) return cuda_fail(c, e, "sweep graph launch");
       c->replays += 1;
-      c->launches += (uint64_t)c->glaunches;
-      c->sweep += (uint64_t)period;
-      if (s->energy_every > 0) c->elog_n += (int)(period / s->energy_every);
-      k += (int)period;
+      c->launches += (uint64_t)g->launches;
+      c->sweep += (uint64_t)g->period;
+      if (s->energy_every > 0) c->elog_n += g->period / s->energy_every;
+      k += g->period;
     } else {
       if ((st = enqueue_one_sweep(c, s)) != HSG_OK) return st;
       k += 1;

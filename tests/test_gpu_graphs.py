@@ -58,3 +58,23 @@ def test_a_schedule_seen_twice_has_its_graph(hsg):
     assert run(hsg, 40, sched, (5, 5, 5, 5))[1:] == (1, 3)
     cadence = hsg.schedule(kind=hsg.HSG_HEATBATH, T=0.5, n_or=2, renorm_every=5, energy_every=5)
     assert run(hsg, 40, cadence, (5, 5, 5, 5))[1:] == (1, 3)
+
+
+# calls shorter than the first, remainders, lengths in turn: after two calls alike a
+# graph of that length, in the end one that divides them
+@pytest.mark.parametrize("n_or,calls,captured,launched", [
+    (5, (50, 1, 1, 1, 1), 2, 10 + 3),
+    (5, (50, 13, 13, 13), 2, 10 + 2 + 3 + 3),
+    (3, (64, 5, 3, 5, 3, 3, 5, 3, 5, 3), 3, 8 + 0 + 0 + 0 + 0 + 1 + 1 + 1 + 2 + 1),
+    (0, (64, 1, 1, 1), 2, 4 + 0 + 1 + 1)])
+@pytest.mark.parametrize("kernel", ["AUTO", "WAVE"])
+def test_short_calls_get_a_graph(hsg, n_or, calls, captured, launched, kernel):
+    k = getattr(hsg, "HSG_KERNEL_" + kernel)
+    sched = hsg.schedule(kind=hsg.HSG_METROPOLIS, hits=2, T=0.5, n_or=n_or, kernel=k)
+    spins, *counts = run(hsg, 40, sched, calls)
+    want = hsg.schedule(kind=hsg.HSG_METROPOLIS, hits=2, T=0.5, n_or=n_or, kernel=hsg.HSG_KERNEL_GLOBAL)
+    assert np.array_equal(spins, run(hsg, 40, want, (sum(calls),), graphs=False)[0])
+    if kernel == "AUTO":
+        assert counts == [captured, launched]
+    else:  # other launches a sweep, buffers that swap
+        assert counts[0] <= 4
