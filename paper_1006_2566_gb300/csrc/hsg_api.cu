@@ -354,7 +354,7 @@ hsg_status prepare_bond_boxes(hsg_ctx* c) {
   if (!c->Jpad) {
     const size_t bytes = sizeof(float) * hsg::padded_bonds_elems(c->L);
     size_t free_b = 0, total_b = 0;
-    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || free_b < bytes + ((size_t)1 << 30)) {
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || free_b + hsg::kept_bytes() < bytes + ((size_t)1 << 30)) {
       cudaGetLastError();
       return HSG_OK;  // no room: register loads
     }

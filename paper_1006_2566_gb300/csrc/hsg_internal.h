@@ -295,6 +295,8 @@ cudaError_t launch_renorm(void* S, bool packed, long long n, int sm_count, cudaS
 // (hsg_memory.cu; freed with cudaFreeAsync), and four pinned words for results
 // with the id of the CUDA context that they belong to (0: pages of their own).
 cudaError_t device_alloc(void** p, size_t bytes, cudaStream_t s);
+// Bytes that the pool holds and nobody uses, which cudaMemGetInfo does not count as free.
+size_t kept_bytes();
 struct ResultWords {
   double* p;
   unsigned long long ctx_id;

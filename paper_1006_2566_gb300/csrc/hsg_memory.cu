@@ -118,6 +118,18 @@ cudaError_t device_alloc(void** p, size_t bytes, cudaStream_t s) {
   return e;
 }
 
+size_t kept_bytes() {
+  std::lock_guard<std::mutex> lock(g_mu);
+  Device* d = current_device();
+  unsigned long long reserved = 0, used = 0;
+  if (!d || cudaMemPoolGetAttribute(d->pool, cudaMemPoolAttrReservedMemCurrent, &reserved) != cudaSuccess ||
+      cudaMemPoolGetAttribute(d->pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return reserved > used ? (size_t)(reserved - used) : 0;
+}
+
 cudaError_t take_result_words(ResultWords* w) {
   *w = ResultWords{};
   std::lock_guard<std::mutex> lock(g_mu);

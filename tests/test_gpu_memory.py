@@ -83,3 +83,28 @@ def test_released_memory_is_kept_within_its_bound(hsg):
         for lat in lats:
             lat.close()
     assert used() - before <= (512 + 64) << 20
+
+
+def test_kept_memory_counts_as_room(hsg):
+    """With less than the margin of 1 GiB free, but more of it kept by the
+    library, the wave sweep still takes its padded couplings (one launch)."""
+    def launches():
+        with hsg.Lattice(64, 1, stream=torch.cuda.Stream()) as lat:
+            lat.generate_couplings()
+            n = hsg.hsg_launch_count(lat.ctx)
+            lat.sweep(hsg.schedule(n_or=1, kernel=hsg.HSG_KERNEL_WAVE), 1)
+            lat.energy()
+            return hsg.hsg_launch_count(lat.ctx) - n
+
+    want = launches()
+    torch.cuda.empty_cache()
+    hsg.Lattice(192, 1).close()  # 198 MB, of which the library keeps all
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    block = torch.empty(free - (1 << 30) + (100 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        assert torch.cuda.mem_get_info()[0] < 1 << 30
+        assert launches() == want
+    finally:
+        del block
+        torch.cuda.empty_cache()
