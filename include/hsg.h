@@ -28,9 +28,10 @@
  *     then restores the caller's, so objects of several devices can be used
  *     from one thread in any order.
  *   - Device memory is owned by the context (stream-ordered allocations),
- *     released by hsg_destroy.  The library keeps up to 512 MB of released
- *     memory per device for its next contexts.  Caller arrays are copied,
- *     never retained.
+ *     released by hsg_destroy.  The library keeps released memory for its
+ *     next contexts, up to 1/512 of the device's (555 MiB on GB300), until
+ *     hsg_release_memory or until an allocation of this process would fail for
+ *     want of it.  Caller arrays are copied, never retained.
  *   - hsg_last_error() gives a message for the last failure.
  *   - A context is not thread-safe; distinct contexts are independent.
  */
@@ -198,6 +199,12 @@ hsg_status hsg_create_layout(hsg_ctx** out, int L, uint64_t seed, uint32_t sampl
 /* Release everything the context owns; waits for its stream.  NULL is a
  * no-op returning HSG_OK. */
 hsg_status hsg_destroy(hsg_ctx* ctx);
+
+/* Give the released memory that the library keeps on the current device back to
+ * the operating system (for other processes: allocations of this one are
+ * given it anyway).  Contexts are not touched; the next one pays for mapping its
+ * memory anew.  Library-specific.  Errors: HSG_ECUDA. */
+hsg_status hsg_release_memory(void);
 
 /*
  * Set the couplings (Eq. 1: Gaussian J_ij on nearest-neighbour bonds).

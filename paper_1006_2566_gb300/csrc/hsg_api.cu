@@ -740,6 +740,11 @@ hsg_status hsg_destroy(hsg_ctx* ctx) {
   return HSG_OK;
 }
 
+hsg_status hsg_release_memory(void) {
+  const cudaError_t e = hsg::release_kept();
+  return e == cudaSuccess ? HSG_OK : cuda_fail(nullptr, e, "memory release");
+}
+
 hsg_status hsg_set_couplings(hsg_ctx* c, const void* J, int dtype, int where) {
   if (!c) return fail(nullptr, HSG_EINVAL, "ctx is NULL");
   const hsg::DeviceGuard device_guard(c->device);

@@ -297,6 +297,7 @@ cudaError_t launch_renorm(void* S, bool packed, long long n, int sm_count, cudaS
 cudaError_t device_alloc(void** p, size_t bytes, cudaStream_t s);
 // Bytes that the pool holds and nobody uses, which cudaMemGetInfo does not count as free.
 size_t kept_bytes();
+cudaError_t release_kept();  // to the operating system
 struct ResultWords {
   double* p;
   unsigned long long ctx_id;

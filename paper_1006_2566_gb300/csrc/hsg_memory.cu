@@ -7,8 +7,12 @@
 // cudaMallocHost for two result words, that cost more than the sweeps of a
 // small lattice: creation 255 us and destruction 277 us at L = 48, 421 and 890 us
 // at L = 192.  So each device has one memory pool of the library's own, which keeps
-// up to kKeepBytes of freed memory for the next context (more is given back at the
-// next synchronisation, all of it before an allocation may fail), and the
+// freed memory for the next context, up to one part in kKeepShare of the device's
+// (555 MiB of GB300's 278 GiB: what a program does not miss; what a larger context frees
+// beyond it is given back at the next synchronisation and mapped anew by the next).
+// All of it goes back when an allocation would fail for want of it -- ours trim
+// the pool, the driver takes it for everyone else's in this process (a pool, torch and
+// cudaMallocAsync were each given more than was free) -- or by hsg_release_memory.  The
 // result words are cut from pinned pages, given back once none of a page is
 // in use (the first page stays).  Both are kept per CUDA context under one lock, by
 // the context's id: after a device reset the handles and the addresses come back,
@@ -22,7 +26,7 @@
 namespace hsg {
 namespace {
 
-constexpr unsigned long long kKeepBytes = 512ull << 20;  // an L = 192 context and its uploads: 490 MB
+constexpr unsigned long long kKeepShare = 512;
 constexpr int kWordBytes = 32, kPageBytes = 4096, kSlots = kPageBytes / kWordBytes;
 constexpr int kPages = 64;
 
@@ -88,7 +92,12 @@ Device* current_device() {
   Device d = {};
   d.ctx = ctx;
   d.ctx_id = id;
-  unsigned long long keep = kKeepBytes;
+  size_t free_b = 0, total_b = 0;
+  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  unsigned long long keep = total_b / kKeepShare;
   if (cudaMemPoolCreate(&d.pool, &props) != cudaSuccess ||
       cudaMemPoolSetAttribute(d.pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
     cudaGetLastError();
@@ -128,6 +137,12 @@ size_t kept_bytes() {
     return 0;
   }
   return reserved > used ? (size_t)(reserved - used) : 0;
+}
+
+cudaError_t release_kept() {
+  std::lock_guard<std::mutex> lock(g_mu);
+  Device* d = current_device();
+  return d ? cudaMemPoolTrimTo(d->pool, 0) : cudaSuccess;
 }
 
 cudaError_t take_result_words(ResultWords* w) {

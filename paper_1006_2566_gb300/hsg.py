@@ -67,6 +67,7 @@ _SIGS = {
     "hsg_create": ([ctypes.POINTER(_vp), _i, _u64, _u32, _u32, _vp], _i),
     "hsg_create_layout": ([ctypes.POINTER(_vp), _i, _u64, _u32, _u32, _vp, _i], _i),
     "hsg_destroy": ([_vp], _i),
+    "hsg_release_memory": ([], _i),
     "hsg_set_couplings": ([_vp, _vp, _i, _i], _i),
     "hsg_generate_couplings": ([_vp], _i),
     "hsg_get_couplings": ([_vp, _vp, _i], _i),
@@ -179,6 +180,11 @@ def hsg_create_layout(L: int, seed: int, sample: int = 0, replica: int = 0, stre
 
 def hsg_destroy(ctx) -> None:
     _check(_lib.hsg_destroy(ctx))
+
+
+def hsg_release_memory() -> None:
+    """Give back the memory that the library keeps on the current device."""
+    _check(_lib.hsg_release_memory())
 
 
 def hsg_set_couplings(ctx, J) -> None:

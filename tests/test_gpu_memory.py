@@ -108,3 +108,24 @@ def test_kept_memory_counts_as_room(hsg):
     finally:
         del block
         torch.cuda.empty_cache()
+
+
+def test_kept_memory_is_given_back_when_asked(hsg):
+    def used():
+        torch.cuda.synchronize()
+        free, total = torch.cuda.mem_get_info()
+        return total - free
+
+    with hsg.Lattice(16, 1) as lat:
+        lat.generate_couplings()
+        hsg.hsg_release_memory()
+        before = used()
+        e = lat.energy()
+        with hsg.Lattice(160, 2) as big:  # 115 MB
+            big.generate_couplings()
+            big.energy()
+        # the pool maps 32 MiB at a time: as much of the 115 MB may fall in what `lat` had mapped
+        assert used() - before >= 115_000_000 - (32 << 20)
+        hsg.hsg_release_memory()
+        assert used() - before <= 32 << 20
+        assert lat.energy() == e
