@@ -345,7 +345,7 @@ hsg_status hsg_philox(uint64_t seed, uint32_t sample, uint32_t replica, uint32_t
  * and replayed (on a non-default stream) while lattices come and go; lattices of
  * L >= 32 are swept in batches that fit in L2, one launch per half-sweep of a
  * batch, partly on streams of the pool's own between the work queued before and
- * after on the pool's stream.  Each lattice keeps its own side, Philox key, temperature and
+ * after on the pool's stream (and of its priority).  Each lattice keeps its own side, Philox key, temperature and
  * sweep counter, and is updated by the same device code with the same
  * random numbers as a single-lattice context: its spins are bit-identical
  * to those of the same lattice swept alone with hsg_sweep.
@@ -461,6 +461,11 @@ hsg_status hsg_test_no_clusters(int on);
 /* For tests of the sweeps' CUDA graphs: how many graphs hsg_sweep has captured and how
  * many it has launched on this context.  Errors: HSG_EINVAL (NULL argument). */
 hsg_status hsg_test_graph_counts(hsg_ctx* ctx, uint64_t* captured, uint64_t* launched);
+
+/* For tests of a pool's own streams: the priority of the pool's stream, and those of
+ * the up to n streams that it has made beside it (*n_side of them).  Errors: HSG_EINVAL,
+ * HSG_ECUDA. */
+hsg_status hsg_test_pool_priorities(hsg_pool* pool, int* own, int* side, int n, int* n_side);
 
 /*
  * E/N of a lattice held in the caller's own device memory, without any

@@ -528,12 +528,14 @@ int main_update(const hsg_schedule* s) {
 // lattices are swept side by side.
 constexpr int kLanes = 1 + hsg_pool::kSide;
 
-// The side streams and events, made once.
+// The side streams, of the pool's stream's priority, and events, made once.
 cudaError_t make_side_streams(hsg_pool* p) {
-  cudaError_t e = cudaSuccess;
+  int priority = 0;
+  cudaError_t e = cudaStreamGetPriority(p->stream, &priority);
+  if (e != cudaSuccess) return e;
   if (!p->fork_ev) e = cudaEventCreateWithFlags(&p->fork_ev, cudaEventDisableTiming);
   for (int i = 0; i < hsg_pool::kSide && e == cudaSuccess; ++i) {
-    if (!p->side[i]) e = cudaStreamCreateWithFlags(&p->side[i], cudaStreamNonBlocking);
+    if (!p->side[i]) e = cudaStreamCreateWithPriority(&p->side[i], cudaStreamNonBlocking, priority);
     if (e == cudaSuccess && !p->join_ev[i]) e = cudaEventCreateWithFlags(&p->join_ev[i], cudaEventDisableTiming);
   }
   return e;
@@ -1205,6 +1207,17 @@ hsg_status hsg_pool_launch_count(hsg_pool* p, uint64_t* launches) {
   if (!p || !launches) return pfail(p, HSG_EINVAL, "NULL argument");
   *launches = p->launches;
   return HSG_OK;
+}
+
+hsg_status hsg_test_pool_priorities(hsg_pool* p, int* own, int* side, int n, int* n_side) {
+  if (!p || !own || !side || !n_side || n < 0) return pfail(p, HSG_EINVAL, "NULL argument");
+  const hsg::DeviceGuard device_guard(p->device);
+  if (device_guard.status() != cudaSuccess) return pcuda(p, device_guard.status(), "cudaSetDevice");
+  *n_side = 0;
+  cudaError_t e = cudaStreamGetPriority(p->stream, own);
+  for (cudaStream_t st : p->side)
+    if (st && *n_side < n && e == cudaSuccess) e = cudaStreamGetPriority(st, side + (*n_side)++);
+  return e == cudaSuccess ? HSG_OK : pcuda(p, e, "stream priority");
 }
 
 const char* hsg_pool_last_error(const hsg_pool* p) { return p ? p->err.c_str() : ""; }

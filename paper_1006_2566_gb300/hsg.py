@@ -94,6 +94,7 @@ _SIGS = {
     "hsg_test_fail_alloc": ([_i], _i),
     "hsg_test_stall_tensor_loads": ([_i], _i),
     "hsg_test_no_clusters": ([_i], _i),
+    "hsg_test_pool_priorities": ([_vp, ctypes.POINTER(_i), ctypes.POINTER(_i), _i, ctypes.POINTER(_i)], _i),
     "hsg_test_graph_counts": ([_vp, ctypes.POINTER(_u64), ctypes.POINTER(_u64)], _i),
     "hsg_energy_noalloc": ([_i, _vp, _vp, _vp, _vp], _i),
     "hsg_pool_create": ([ctypes.POINTER(_vp), _u64, _i, _vp], _i),
@@ -337,6 +338,13 @@ def hsg_test_graph_counts(ctx):
     a, b = _u64(0), _u64(0)
     _check(_lib.hsg_test_graph_counts(ctx, ctypes.byref(a), ctypes.byref(b)), ctx)
     return a.value, b.value
+
+
+def hsg_test_pool_priorities(pool):
+    """(priority of the pool's stream, those of the streams it has made beside it)."""
+    own, side, n = _i(0), (_i * 8)(), _i(0)
+    _pcheck(_lib.hsg_test_pool_priorities(pool, ctypes.byref(own), side, 8, ctypes.byref(n)), pool)
+    return own.value, list(side[:n.value])
 
 
 def hsg_energy_noalloc(L: int, spins, J, e_out, stream=None) -> None:

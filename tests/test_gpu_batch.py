@@ -124,3 +124,13 @@ def test_a_lattice_beyond_32_bit_offsets(hsg):
         hsg.hsg_get_spins(lat.ctx, ref)
         torch.cuda.synchronize()
     assert torch.equal(out, ref)
+
+
+@pytest.mark.parametrize("priority", [0, -1])
+def test_side_streams_have_the_pools_priority(hsg, priority):
+    with hsg.Pool(1 << 27, 4, torch.cuda.Stream(priority=priority)) as pool:
+        pool.admit(64, 7)
+        pool.sweep(hsg.schedule(kind=hsg.HSG_HEATBATH), 1)
+        own, side = hsg.hsg_test_pool_priorities(pool.pool)
+        assert len(side) == 2 and side == [own, own]
+        assert (own < 0) == (priority < 0)
