@@ -377,7 +377,10 @@ hsg_status hsg_pool_retire(hsg_pool* pool, int slot);
 
 /* n_sweeps sweeps of every admitted lattice, each at its own temperature
  * (schedule.T and schedule.kernel are ignored; energy_every must be 0;
- * renorm_every applies to each lattice's own counter).  Asynchronous. */
+ * renorm_every applies to each lattice's own counter).  Asynchronous: the host
+ * queues one to a few CUDA graphs a sweep (in calls of fewer than eight sweeps each
+ * launch of the lattices of L >= 32: up to half of the time that the sweeps take) and waits
+ * only where the device's queue is full. */
 hsg_status hsg_pool_sweep(hsg_pool* pool, const hsg_schedule* schedule, int n_sweeps);
 
 /* E/N of every slot into out[0..n) (NaN for free slots); FP32 site terms,

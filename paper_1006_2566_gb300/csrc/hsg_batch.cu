@@ -39,7 +39,7 @@ __device__ __forceinline__ int batch_find(const BatchArgs& a, uint32_t b) {
   return lo;
 }
 
-template <int U, int R, int MIN_BLOCKS, class Off>
+template <int U, int R, int MIN_BLOCKS, class Off, bool COUNTED>
 __global__ void __launch_bounds__(B_THREADS, MIN_BLOCKS)
     k_batch_half(const __grid_constant__ BatchArgs a, uint32_t colour, int hits, int hit0, float step,
                  uint32_t sweep_add) {
@@ -64,12 +64,25 @@ __global__ void __launch_bounds__(B_THREADS, MIN_BLOCKS)
                               L,
                               Lh,
                               colour};
-  const unsigned long long sw = l.sweep + sweep_add;
+  // The count is advanced first by the sphere proposals' kernels and last by the others:
+  // where the store stands moves the compiler's registers.  us a sweep of 36 lattices of
+  // L = 64, first / last: sphere 1 hit 85.0 / 88.5, sphere + OR 88.0 / 96.0; ball 1 hit 90.9 / 85.4,
+  // ball + OR 90.5 / 88.8, heat-bath 112.9 / 109.1 (not counted: 84.8, 90.9, 85.8, 91.7, 107.7).
+  constexpr bool FIRST = U == U_MET_SPHERE || U == U_MET_OR_SPHERE;
+  unsigned long long sw = l.sweep + sweep_add;
+  if constexpr (COUNTED) {
+    const unsigned long long count = a.done[colour];
+    sw = l.sweep + count;
+    if (FIRST && blockIdx.x == 0 && threadIdx.x == 0) a.done[o] = count + colour;
+  }
   const DrawArgs d{(uint32_t)sw, (uint32_t)(sw >> 32), l.k0, l.k1, l.beta, step, hits, hit0};
   update_rows<U, R, Off>(lat, xh, y0, z, (colour + y0 + z) & 1u, d);  // z differs within a CTA
+  if constexpr (COUNTED && !FIRST) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.done[o] = a.done[colour] + colour;
+  }
 }
 
-template <int U, int R, int MIN_BLOCKS>
+template <int U, int R, int MIN_BLOCKS, bool COUNTED>
 void launch_r(BatchArgs& a, uint32_t colour, int hits, int hit0, float step, uint32_t sweep_add, cudaStream_t s) {
   uint32_t ctas = 0;
   bool wide = false;
@@ -81,9 +94,18 @@ void launch_r(BatchArgs& a, uint32_t colour, int hits, int hit0, float step, uin
     wide |= l.L > (uint32_t)kMaxOff32L;
   }
   if (wide)
-    k_batch_half<U, R, MIN_BLOCKS, unsigned long long><<<ctas, B_THREADS, 0, s>>>(a, colour, hits, hit0, step, sweep_add);
+    k_batch_half<U, R, MIN_BLOCKS, unsigned long long, COUNTED><<<ctas, B_THREADS, 0, s>>>(a, colour, hits, hit0, step, sweep_add);
   else
-    k_batch_half<U, R, MIN_BLOCKS, uint32_t><<<ctas, B_THREADS, 0, s>>>(a, colour, hits, hit0, step, sweep_add);
+    k_batch_half<U, R, MIN_BLOCKS, uint32_t, COUNTED><<<ctas, B_THREADS, 0, s>>>(a, colour, hits, hit0, step, sweep_add);
+}
+
+template <int U, int R, int MIN_BLOCKS, int MIN_BLOCKS_COUNTED>
+void launch_kind(bool counted, BatchArgs& a, uint32_t colour, int hits, int hit0, float step, uint32_t sweep_add,
+                 cudaStream_t s) {
+  if (counted)
+    launch_r<U, R, MIN_BLOCKS_COUNTED, true>(a, colour, hits, hit0, step, 0u, s);
+  else
+    launch_r<U, R, MIN_BLOCKS, false>(a, colour, hits, hit0, step, sweep_add, s);
 }
 
 __global__ void __launch_bounds__(256) k_batch_renorm(const __grid_constant__ BatchArgs a) {
@@ -96,18 +118,19 @@ __global__ void __launch_bounds__(256) k_batch_renorm(const __grid_constant__ Ba
 
 }  // namespace
 
-cudaError_t launch_batch_half(int upd, BatchArgs& a, uint32_t colour, int hits, int hit0, float step,
+cudaError_t launch_batch_half(int upd, bool counted, BatchArgs& a, uint32_t colour, int hits, int hit0, float step,
                               uint32_t sweep_add, cudaStream_t s) {
   // Rows per thread and registers as in the single-lattice launches
   // (hsg_sweep.cu), measured here for OR (one row 47 us, two 53-70), the
-  // heat-bath (two rows 75, one 80) and the ball proposal (two 129, one 133).
+  // heat-bath (two rows 75, one 80) and the ball proposal (two 129, one 133).  The counted
+  // ones are held to the registers of the others (64 and 56, not 96 and 80).
   switch (upd) {
-    case U_OR: launch_r<U_OR, 1, 12>(a, colour, hits, hit0, step, sweep_add, s); break;
-    case U_MET_SPHERE: launch_r<U_MET_SPHERE, 2, 10>(a, colour, hits, hit0, step, sweep_add, s); break;
-    case U_MET_BALL: launch_r<U_MET_BALL, 2, 8>(a, colour, hits, hit0, step, sweep_add, s); break;
-    case U_HB: launch_r<U_HB, 2, 1>(a, colour, hits, hit0, step, sweep_add, s); break;
-    case U_MET_OR_SPHERE: launch_r<U_MET_OR_SPHERE, 2, 8>(a, colour, hits, hit0, step, sweep_add, s); break;
-    case U_MET_OR_BALL: launch_r<U_MET_OR_BALL, 2, 1>(a, colour, hits, hit0, step, sweep_add, s); break;
+    case U_OR: launch_r<U_OR, 1, 12, false>(a, colour, hits, hit0, step, sweep_add, s); break;
+    case U_MET_SPHERE: launch_kind<U_MET_SPHERE, 2, 10, 10>(counted, a, colour, hits, hit0, step, sweep_add, s); break;
+    case U_MET_BALL: launch_kind<U_MET_BALL, 2, 8, 8>(counted, a, colour, hits, hit0, step, sweep_add, s); break;
+    case U_HB: launch_kind<U_HB, 2, 1, 8>(counted, a, colour, hits, hit0, step, sweep_add, s); break;
+    case U_MET_OR_SPHERE: launch_kind<U_MET_OR_SPHERE, 2, 8, 8>(counted, a, colour, hits, hit0, step, sweep_add, s); break;
+    case U_MET_OR_BALL: launch_kind<U_MET_OR_BALL, 2, 1, 9>(counted, a, colour, hits, hit0, step, sweep_add, s); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();

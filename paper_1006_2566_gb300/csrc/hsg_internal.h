@@ -215,14 +215,19 @@ struct BatchLattice {
 };
 constexpr int kBatchMax = 24;   // 2 KB of parameters: 3 us of host time per launch (40: 4 us)
 constexpr int kBatchMinL = 32;  // smaller lattices stay with the pool's persistent kernels
+// done, for counted launches: two words on the device, the sweeps since `sweep` was
+// written.  Colour 0's launches of the main update read done[0] and write done[1] =
+// done[0]; colour 1's read done[1] and write done[0] = done[1] + 1.  So each sweep
+// advances the count without a launch of its own, and none reads what it writes.
 struct BatchArgs {
   int n;
+  unsigned long long* done;
   BatchLattice lat[kBatchMax];
 };
 // Half-sweep `upd` of colour `colour` of every lattice of the batch, hits
-// hit0 .. hit0 + hits - 1, at its sweep counter plus sweep_add.
-cudaError_t launch_batch_half(int upd, BatchArgs& a, uint32_t colour, int hits, int hit0, float step, uint32_t sweep_add,
-                              cudaStream_t s);
+// hit0 .. hit0 + hits - 1, at its sweep counter plus sweep_add or (counted) the count.
+cudaError_t launch_batch_half(int upd, bool counted, BatchArgs& a, uint32_t colour, int hits, int hit0, float step,
+                              uint32_t sweep_add, cudaStream_t s);
 cudaError_t launch_batch_renorm(const BatchArgs& a, cudaStream_t s);
 
 // Halo-padded copy of the colour-split bonds, read by the sweep's tensor

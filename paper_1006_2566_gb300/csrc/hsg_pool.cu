@@ -47,6 +47,7 @@ constexpr size_t kAlign = 256;
 // lattices of L >= kBatchMinL from which they are worth their launches beside
 // the persistent kernels' (one L = 40 lattice among small ones is not).
 constexpr uint64_t kBatchBytes = 32ull << 20, kBatchMinSites = 1ull << 17;
+constexpr int kBatchGraphMin = 8;  // sweeps in a call from which the batches' are graphs
 
 inline unsigned cdiv_u(unsigned long long a, unsigned long long b) { return (unsigned)((a + b - 1) / b); }
 
@@ -200,6 +201,17 @@ __global__ void __launch_bounds__(256) k_pool_energy_final(const hsg::PoolDesc* 
   }
 }
 
+// A batch of larger lattices (hsg_batch.cu) and the lane that sweeps it.
+struct PoolBatch {
+  hsg::BatchArgs a;
+  int lane;
+};
+
+struct BatchGraph {
+  cudaGraphExec_t exec = nullptr;
+  bool stale = true;  // none yet, or one of other batches
+};
+
 struct Slot {
   bool active = false;
   int L = 0;
@@ -244,6 +256,14 @@ struct hsg_pool {
   static constexpr int kSide = 2;
   cudaStream_t side[kSide] = {nullptr, nullptr};
   cudaEvent_t fork_ev = nullptr, join_ev[kSide] = {nullptr, nullptr};
+  // The batches of the admitted lattices, with the lattices' counters as they were
+  // batch_swept sweeps ago, that many as the device last counted them (two words a
+  // batch at d_done), and one sweep of each as a graph, made when first needed.
+  std::vector<PoolBatch> batches;
+  bool batches_ok = false;
+  uint64_t batch_swept = 0, batch_counted = 0;
+  unsigned long long* d_done = nullptr;
+  std::vector<BatchGraph> batch_graphs;
   cudaEvent_t up_ev[2] = {nullptr, nullptr};
   bool up_rec[2] = {false, false};
   int up_buf = 0;
@@ -273,7 +293,7 @@ struct hsg_pool {
     bool operator==(const GraphKey& o) const { return memcmp(this, &o, sizeof(GraphKey)) == 0; }
   };
   bool have_graph = false;
-  GraphKey gkey{};
+  GraphKey gkey{}, batch_key{};
   cudaGraphExec_t gexec = nullptr;
   uint64_t launches = 0;
   std::string err;
@@ -378,6 +398,7 @@ hsg_status sync_tables(hsg_pool* p) {
   for (const Slot& s : p->slots)
     if (s.active && s.L >= hsg::kBatchMinL) large_sites += (uint64_t)s.L * s.L * s.L;
   p->batched = large_sites >= kBatchMinSites;
+  p->batches_ok = false;
   uint32_t nt = 0;
   // The slots of the persistent kernels first, those of the batches after them.
   for (int pass = 0; pass < 2; ++pass) {
@@ -612,16 +633,14 @@ cudaError_t sweep_resident(hsg_pool* p, const hsg_schedule* s, int n_sweeps) {
   return join_lanes(p, used, e);
 }
 
-// A batch and the lane that sweeps it.
-struct PoolBatch {
-  hsg::BatchArgs a;
-  int lane;
-};
 // The slots' lattices of L >= kBatchMinL in batches of about kBatchBytes, each
 // given to the lane with the fewest bytes so far (the pool's own stream
 // first sweeps the other lattices: counted twice, their kernels being slower).
-std::vector<PoolBatch> make_batches(const hsg_pool* p) {
-  std::vector<PoolBatch> out;
+void make_batches(hsg_pool* p) {
+  std::vector<PoolBatch>& out = p->batches;
+  out.clear();
+  p->batch_swept = 0;
+  p->batch_counted = ~0ull;
   uint64_t load[kLanes] = {};
   for (const Slot& sl : p->slots)
     if (sl.active && sl.L < hsg::kBatchMinL) load[0] += 2 * sl.bytes;
@@ -631,6 +650,7 @@ std::vector<PoolBatch> make_batches(const hsg_pool* p) {
     if (out.empty() || out.back().a.n == hsg::kBatchMax || bytes + sl.bytes > kBatchBytes) {
       out.emplace_back();
       out.back().a.n = 0;
+      out.back().a.done = p->d_done + 2 * (out.size() - 1);
       out.back().lane = (int)(std::min_element(load, load + kLanes) - load);
       bytes = 0;
     }
@@ -649,7 +669,7 @@ std::vector<PoolBatch> make_batches(const hsg_pool* p) {
     l.beta = beta_of(sl.T);
     l.by_lh = hsg::make_fastdiv(l.Lh);
   }
-  return out;
+  p->batches_ok = true;
 }
 
 // The launches of one sweep of a batch, in the single-lattice order.
@@ -663,55 +683,143 @@ struct BatchSweep {
     passes = main_passes(p, s);
     per = passes ? (s->hits + passes - 1) / passes : 0;
   }
-  int steps() const { return 2 * passes + 2 * s->n_or + (s->renorm_every > 0); }
-  cudaError_t launch(hsg::BatchArgs& a, int step, int sweep_add, cudaStream_t st) const {
-    if (step < 2 * passes) {
-      const int q = step % passes, j0 = q * per;
-      // the fused reflection follows the colour's last hit only
-      const int u = s->kind == HSG_METROPOLIS_OR && q + 1 < passes ? met : upd;
-      p->launches += 1;
-      return hsg::launch_batch_half(u, a, (uint32_t)(step / passes), std::min(per, s->hits - j0), j0, s->step,
-                                    (uint32_t)sweep_add, st);
-    }
-    step -= 2 * passes;
-    if (step < 2 * s->n_or) {
-      p->launches += 1;
-      return hsg::launch_batch_half(hsg::U_OR, a, (uint32_t)step & 1u, 1, 0, s->step, (uint32_t)sweep_add, st);
-    }
+  int half_sweeps() const { return 2 * passes + 2 * s->n_or; }
+  // Half-sweep `step` of the sweep `sweep_add` after the batch's counters, or of the
+  // next that the device counts.
+  cudaError_t half_sweep(hsg::BatchArgs& a, int step, bool counted, uint32_t sweep_add, cudaStream_t st) const {
+    p->launches += 1;
+    if (step >= 2 * passes)
+      return hsg::launch_batch_half(hsg::U_OR, false, a, (uint32_t)(step - 2 * passes) & 1u, 1, 0, s->step, 0u, st);
+    const int q = step % passes, j0 = q * per;
+    // the fused reflection follows the colour's last hit only
+    const int u = s->kind == HSG_METROPOLIS_OR && q + 1 < passes ? met : upd;
+    return hsg::launch_batch_half(u, counted, a, (uint32_t)(step / passes), std::min(per, s->hits - j0), j0, s->step,
+                                  sweep_add, st);
+  }
+  // Renormalises the lattices of the batch that are due when it has made `done` sweeps.
+  cudaError_t renorm(const hsg::BatchArgs& a, uint64_t done, cudaStream_t st) const {
+    if (s->renorm_every == 0) return cudaSuccess;
     hsg::BatchArgs due;
     due.n = 0;
     for (int k = 0; k < a.n; ++k)
-      if ((a.lat[k].sweep + (uint64_t)sweep_add + 1) % (uint64_t)s->renorm_every == 0) due.lat[due.n++] = a.lat[k];
+      if ((a.lat[k].sweep + done) % (uint64_t)s->renorm_every == 0) due.lat[due.n++] = a.lat[k];
     if (due.n) p->launches += 1;
     return hsg::launch_batch_renorm(due, st);
   }
+  // One sweep of batch i as a graph; a graph that is there from other batches is
+  // given the new kernels' arguments where its shape allows.
+  cudaError_t capture(size_t i) const {
+    const cudaStream_t st = p->side[0];
+    const uint64_t launches = p->launches;
+    cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return e;
+    for (int k = 0; k < half_sweeps() && e == cudaSuccess; ++k) e = half_sweep(p->batches[i].a, k, true, 0u, st);
+    p->launches = launches;
+    cudaGraph_t g = nullptr;
+    const cudaError_t end = cudaStreamEndCapture(st, &g);
+    if (e == cudaSuccess) e = end;
+    BatchGraph& b = p->batch_graphs[i];
+    cudaGraphExecUpdateResultInfo info;
+    if (e == cudaSuccess && b.exec && cudaGraphExecUpdate(b.exec, g, &info) != cudaSuccess) {
+      cudaGetLastError();
+      cudaGraphExecDestroy(b.exec);
+      b.exec = nullptr;
+    }
+    if (e == cudaSuccess && !b.exec && (e = cudaGraphInstantiate(&b.exec, g, 0)) != cudaSuccess) b.exec = nullptr;
+    if (g) cudaGraphDestroy(g);
+    b.stale = e != cudaSuccess;
+    return e;
+  }
 };
+
+__global__ void k_set_done(unsigned long long* done, int n, unsigned long long v) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) done[i] = v;
+}
+
+// Before the side streams start: the batches of the admitted lattices and, for a call
+// whose sweeps the device counts, the count.
+cudaError_t prepare_batches(hsg_pool* p, const hsg_pool::GraphKey& key, bool counted) {
+  const bool ok = p->batches_ok && p->batch_swept < 1u << 30;
+  if (!ok || !(p->batch_key == key)) {
+    p->batches_ok = false;  // until there are graphs for them
+    if (!ok) make_batches(p);
+    for (size_t i = p->batches.size(); i < p->batch_graphs.size(); ++i)
+      if (p->batch_graphs[i].exec) cudaGraphExecDestroy(p->batch_graphs[i].exec);
+    p->batch_graphs.resize(p->batches.size());
+    for (BatchGraph& b : p->batch_graphs) b.stale = true;
+    p->batch_key = key;
+    p->batches_ok = true;
+  }
+  if (!counted || p->batch_counted == p->batch_swept) return cudaSuccess;
+  const int n = 2 * (int)p->batches.size();
+  k_set_done<<<cdiv_u((unsigned)n, 256), 256, 0, p->stream>>>(p->d_done, n, p->batch_swept);
+  p->launches += 1;
+  p->batch_counted = p->batch_swept;
+  return cudaGetLastError();
+}
 
 // n_sweeps sweeps of the batches, each batch all of its sweeps on its lane,
 // the lanes' launches interleaved.  The side streams start after what the
 // pool's stream held at fork_ev, and the pool's stream then waits for them.
-cudaError_t sweep_batches(hsg_pool* p, const hsg_schedule* s, int n_sweeps, std::vector<PoolBatch>& batches) {
+//
+// In a call of kBatchGraphMin sweeps or more a sweep of a batch is a graph, so that the
+// call returns long before the sweeps end: six launches with 2 KB of arguments each take
+// the host 16 us, a graph 1.2 us, and launches ahead of the GPU fill their queue (from some
+// 1000 a lane on the host waits).  us a sweep of 4-hit Metropolis + 2 OR in calls of 40, host
+// time / until the end, launches and graphs:
+//   24 lattices of L = 64 to 96   185 / 445   17 / 419
+//   256 of 16 to 48                94 / 389   10 / 384
+//   128 of 32 and 48               96 / 332    9 / 329
+//   4 of 64, 6 of 160         11 / 58, 68 / 944   1.2 / 47, 6 / 930
+// Without over-relaxation 288 of L = 32: heat-bath 107.1 / 108.0, 4 hits 176.5 / 178.0 until the end.
+// With five sweeps to a graph (128 of 32 and 48) 362, with a launch to count 342, with the sweep
+// set in the graph's nodes before each launch 361: the lanes' kernels then fall
+// into step, Metropolis beside Metropolis.  The first graphs of a call cost it some 25 us
+// more than launches, hence kBatchGraphMin; a new batch's graph is made while its lane
+// has a sweep to work on.
+cudaError_t sweep_batches(hsg_pool* p, const hsg_schedule* s, int n_sweeps, bool counted) {
   const cudaStream_t st[kLanes] = {p->stream, p->side[0], p->side[1]};
   const BatchSweep sweep(p, s);
+  const size_t n = p->batches.size();
   cudaError_t e = cudaSuccess;
   bool used[kLanes] = {};
-  for (const PoolBatch& b : batches) used[b.lane] = true;
+  for (const PoolBatch& b : p->batches) used[b.lane] = true;
   for (int l = 1; l < kLanes && e == cudaSuccess; ++l)
     if (used[l]) e = cudaStreamWaitEvent(st[l], p->fork_ev, 0);
-  size_t at[kLanes] = {};  // each lane's batch at hand
-  for (;;) {
-    bool any = false;
-    for (int l = 0; l < kLanes; ++l) {
-      while (at[l] < batches.size() && batches[at[l]].lane != l) ++at[l];
-      any |= at[l] < batches.size();
+  size_t at[kLanes] = {};  // each lane's batch at hand,
+  int k[kLanes] = {};      // its sweeps so far,
+  bool queued[kLanes] = {};  // and whether the lane has work
+  while (e == cudaSuccess) {
+    bool any = false, launches[kLanes] = {};
+    for (int l = 0; l < kLanes && e == cudaSuccess; ++l) {
+      while (at[l] < n && (p->batches[at[l]].lane != l || k[l] == n_sweeps)) {
+        ++at[l];
+        k[l] = 0;
+      }
+      if (at[l] == n) continue;
+      any = true;
+      BatchGraph& g = p->batch_graphs[at[l]];
+      launches[l] = !counted || (g.stale && !queued[l]) || sweep.half_sweeps() == 0;
+      if (launches[l]) continue;
+      if (g.stale) e = sweep.capture(at[l]);
+      if (e == cudaSuccess) e = cudaGraphLaunch(g.exec, st[l]);
+      p->launches += (uint64_t)sweep.half_sweeps();
     }
-    if (!any || e != cudaSuccess) break;
-    for (int k = 0; k < n_sweeps && e == cudaSuccess; ++k)
-      for (int i = 0; i < sweep.steps() && e == cudaSuccess; ++i)
-        for (int l = 0; l < kLanes && e == cudaSuccess; ++l)
-          if (at[l] < batches.size()) e = sweep.launch(batches[at[l]].a, i, k, st[l]);
-    for (size_t& i : at) ++i;
+    if (!any) break;
+    for (int i = 0; i < sweep.half_sweeps() && e == cudaSuccess; ++i)
+      for (int l = 0; l < kLanes && e == cudaSuccess; ++l)
+        if (launches[l])
+          e = sweep.half_sweep(p->batches[at[l]].a, i, counted, (uint32_t)p->batch_swept + (uint32_t)k[l], st[l]);
+    for (int l = 0; l < kLanes && e == cudaSuccess; ++l) {
+      if (at[l] == n) continue;
+      k[l] += 1;
+      queued[l] = true;
+      e = sweep.renorm(p->batches[at[l]].a, p->batch_swept + (uint64_t)k[l], st[l]);
+    }
   }
+  p->batch_swept += (uint64_t)n_sweeps;
+  if (counted && s->kind != HSG_NONE) p->batch_counted = p->batch_swept;  // (over-relaxation alone counts nothing)
+  if (e != cudaSuccess) p->batches_ok = false;
   return join_lanes(p, used, e);
 }
 
@@ -755,6 +863,7 @@ hsg_status hsg_pool_create(hsg_pool** out, uint64_t budget_bytes, int max_slots,
   if (e == cudaSuccess) e = cudaMalloc(&p->d_ntiles, 2 * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMallocHost(&p->h_ntiles, 4 * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc(&p->d_small, sizeof(uint32_t) * max_slots);
+  if (e == cudaSuccess) e = cudaMalloc(&p->d_done, 2 * sizeof(unsigned long long) * max_slots);
   if (e == cudaSuccess) e = cudaMallocHost(&p->h_small, 2 * sizeof(uint32_t) * max_slots);
   if (e == cudaSuccess) e = cudaMalloc(&p->d_energy, sizeof(double) * max_slots);
   if (e == cudaSuccess) e = cudaMallocHost(&p->h_energy, hsg_pool::kEnergyBufs * sizeof(double) * max_slots);
@@ -788,6 +897,9 @@ hsg_status hsg_pool_destroy(hsg_pool* p) {
   cudaFree(p->d_ntiles);
   cudaFreeHost(p->h_ntiles);
   cudaFree(p->d_small);
+  cudaFree(p->d_done);
+  for (BatchGraph& b : p->batch_graphs)
+    if (b.exec) cudaGraphExecDestroy(b.exec);
   cudaFreeHost(p->h_small);
   cudaFree(p->d_partials);
   cudaFree(p->d_energy);
@@ -912,17 +1024,18 @@ hsg_status hsg_pool_sweep(hsg_pool* p, const hsg_schedule* sched, int n_sweeps) 
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if ((e = cudaStreamIsCapturing(p->stream, &cap)) != cudaSuccess) return pcuda(p, e, "pool sweep");
   const bool batch = p->batched && cap == cudaStreamCaptureStatusNone;
+  const bool counted = n_sweeps >= kBatchGraphMin;  // the batches' sweeps as graphs
   const bool resident = cap == cudaStreamCaptureStatusNone && resident_pool(p, sched);
-  std::vector<PoolBatch> batches;
-  if (batch) {
-    try {
-      batches = make_batches(p);
-    } catch (const std::bad_alloc&) {
-      return pfail(p, HSG_ENOMEM, "host allocation failed");
-    }
-  }
   if (batch || resident) {
-    if ((e = make_side_streams(p)) == cudaSuccess) e = cudaEventRecord(p->fork_ev, p->stream);
+    e = make_side_streams(p);
+    if (e == cudaSuccess && batch) {
+      try {
+        e = prepare_batches(p, key, counted);
+      } catch (const std::bad_alloc&) {
+        return pfail(p, HSG_ENOMEM, "host allocation failed");
+      }
+    }
+    if (e == cudaSuccess) e = cudaEventRecord(p->fork_ev, p->stream);
     if (e != cudaSuccess) return pcuda(p, e, "pool streams");
   }
   // One sweep is captured once per (schedule, launch configuration) and
@@ -963,7 +1076,7 @@ hsg_status hsg_pool_sweep(hsg_pool* p, const hsg_schedule* sched, int n_sweeps) 
   } else {
     for (int k = 0; k < n_sweeps && e == cudaSuccess; ++k) e = enqueue_sweep(p, sched);
   }
-  if (batch && e == cudaSuccess) e = sweep_batches(p, sched, n_sweeps, batches);
+  if (batch && e == cudaSuccess) e = sweep_batches(p, sched, n_sweeps, counted);
   if (e != cudaSuccess) return pcuda(p, e, "pool sweep");
   for (Slot& s : p->slots)
     if (s.active) s.sweep += (uint64_t)n_sweeps;

@@ -134,3 +134,69 @@ def test_side_streams_have_the_pools_priority(hsg, priority):
         own, side = hsg.hsg_test_pool_priorities(pool.pool)
         assert len(side) == 2 and side == [own, own]
         assert (own < 0) == (priority < 0)
+
+
+@pytest.mark.parametrize("k", range(6))
+@pytest.mark.parametrize("use_stream", [True, False])
+def test_long_calls_equal_lattices_alone(hsg, k, use_stream):
+    """Calls long enough for graphs, whose sweeps the device counts, among short
+    ones and over-relaxation alone, which it does not; several batches a lane."""
+    kw = kinds(hsg)[k]
+    alone_or = dict(kind=hsg.HSG_NONE, n_or=1)
+    specs = SPECS + [(96, 7, 10 + j, j & 1, 0.4 + 0.1 * j) for j in range(6)]
+    first = [(kw, 9), (kw, 3), (alone_or, 8), (kw, 10)]
+    then = [(kw, 8), (kw, 8)]
+    with hsg.Pool(1 << 28, 20, torch.cuda.Stream() if use_stream else None) as pool:
+        slots = [pool.admit(*s) for s in specs]
+        if k % 2:
+            hsg.hsg_pool_config(pool.pool, 128, 256, 4, 1)  # one hit per pass
+        for s, n in first:
+            pool.sweep(hsg.schedule(**s), n)
+        pool.retire(slots[2])
+        late = pool.admit(40, 7, 90, 0, 0.8)
+        for s, n in then:
+            pool.sweep(hsg.schedule(**s), n)
+        for slot, spec, calls in [(s, x, first + then) for s, x in zip(slots, specs) if x[0] != 108] + [(late, (40, 7, 90, 0, 0.8), then)]:
+            L, seed, sample, replica, T = spec
+            with hsg.Lattice(L, seed, sample, replica) as lat:
+                lat.generate_couplings()
+                for s, n in calls:
+                    lat.sweep(hsg.schedule(T=T, kernel=hsg.HSG_KERNEL_GLOBAL, **s), n)
+                assert np.array_equal(pool.spins(slot), lat.spins()), (L, kw)
+                assert pool.sweep_count(slot) == lat.sweep_count
+
+
+def test_a_long_call_does_not_wait_for_its_sweeps(hsg):
+    import time
+
+    with hsg.Pool(1 << 26, 4, torch.cuda.Stream()) as pool:
+        for k in range(4):
+            pool.admit(64, 7, k)
+        sched = hsg.schedule(kind=hsg.HSG_METROPOLIS, hits=4, proposal=hsg.HSG_PROP_BALL, n_or=2)
+        pool.sweep(sched, 10)
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        pool.sweep(sched, 1000)  # 6000 half-sweeps
+        returned = time.perf_counter() - t0
+        torch.cuda.synchronize()
+        assert returned < 0.5 * (time.perf_counter() - t0)
+
+
+@pytest.mark.parametrize("kind,proposal", [("HEATBATH", 0), ("METROPOLIS", 0), ("METROPOLIS_OR", 1)])
+def test_a_lattice_beyond_32_bit_offsets_in_a_long_call(hsg, kind, proposal):
+    if torch.cuda.mem_get_info()[0] < 60 << 30:
+        pytest.skip("needs 60 GB of device memory")
+    L, kw = 814, dict(kind=getattr(hsg, "HSG_" + kind), hits=1, proposal=proposal)
+    out = torch.empty(3 * L ** 3, device="cuda")
+    with hsg.Pool(28 * L ** 3 + 256, 1, torch.cuda.Stream()) as pool:
+        slot = pool.admit(L, 1, 0, 0, 0.5)
+        pool.sweep(hsg.schedule(**kw), 8)
+        hsg.hsg_pool_get_spins(pool.pool, slot, out)
+        torch.cuda.synchronize()
+    ref = torch.empty_like(out)
+    with hsg.Lattice(L, 1) as lat:
+        lat.generate_couplings()
+        lat.sweep(hsg.schedule(T=0.5, kernel=hsg.HSG_KERNEL_GLOBAL, **kw), 8)
+        hsg.hsg_get_spins(lat.ctx, ref)
+        torch.cuda.synchronize()
+    assert torch.equal(out, ref)
