@@ -339,13 +339,15 @@ hsg_status hsg_philox(uint64_t seed, uint32_t sample, uint32_t replica, uint32_t
 
 /*
  * Pools: many independent lattices (disorder samples, replicas, requests) of
- * uneven L in one device arena, swept together.  Every half-sweep of the
- * small lattices is ONE persistent kernel over a work list of (lattice,
- * site-range) tiles, and a sweep's launches are captured once in a CUDA graph
- * and replayed (on a non-default stream) while lattices come and go; lattices of
- * L >= 32 are swept in batches that fit in L2, one launch per half-sweep of a
- * batch, partly on streams of the pool's own between the work queued before and
- * after on the pool's stream (and of its priority).  Each lattice keeps its own side, Philox key, temperature and
+ * uneven L in one device arena, swept together.  Lattices of L >= 32 are swept in
+ * batches that fit in L2, one launch per half-sweep of a batch; few lattices below (640 K
+ * sites in all, few hits) by one launch per side for all the sweeps of a call, with a
+ * thread-block cluster for each; more of them by one persistent kernel per half-sweep
+ * over a work list of (lattice, site-range) tiles.  A sweep's launches are captured in
+ * CUDA graphs and replayed (the persistent kernels' on a non-default stream) while
+ * lattices come and go.  Part of the work runs on streams of the pool's own (of its
+ * stream's priority), between the work queued before and after on its stream.
+ * Each lattice keeps its own side, Philox key, temperature and
  * sweep counter, and is updated by the same device code with the same
  * random numbers as a single-lattice context: its spins are bit-identical
  * to those of the same lattice swept alone with hsg_sweep.
@@ -418,12 +420,16 @@ hsg_status hsg_pool_usage(hsg_pool* pool, uint64_t* bytes_used, uint64_t* bytes_
  * launch that reads and writes the colour again -- the neighbours are fixed
  * for the whole half-sweep and hit j draws the Philox numbers keyed by j,
  * so the result is the same; Table 3 of the paper runs the hits in one
- * pass).  hsg_pool_autotune times every launch shape with all hits in one
- * pass, then the best shape with 1, 2, 4, ... hits per pass (Metropolis
- * schedules with more than one hit), on the admitted lattices (one warm-up
- * and two timed sweeps each), restores the lattices and counters
- * afterwards, keeps the fastest configuration and reports it.  Results do
- * not depend on the configuration.  Errors: HSG_EINVAL (NULL pool, values
+ * pass).  The shape is that of the kernels that sweep the lattices of L < 32 of
+ * pools with more of them than a few (above); hits per pass h > 0 apply to all, and
+ * few small lattices too then take those kernels.  hsg_pool_autotune times
+ * these kernels in every launch shape, with all hits in one pass, on the lattices of L < 32 (one
+ * warm-up and two timed sweeps each; a pool without any keeps its shape), then that shape with all
+ * hits and with 1, 2, 4, ... hits per pass (Metropolis schedules with more than one hit; ten
+ * sweeps twice each), on the admitted lattices, restores the lattices and
+ * counters afterwards, keeps the fastest configuration and reports it.  Results
+ * do not depend on the configuration but for the last bits of the energies, whose
+ * fp64 sums run tile by tile.  Errors: HSG_EINVAL (NULL pool, values
  * out of range; autotune with no lattice admitted or on the legacy default
  * stream). */
 hsg_status hsg_pool_config(hsg_pool* pool, int threads, int tile_sites, int blocks_per_sm, int hits_per_pass);

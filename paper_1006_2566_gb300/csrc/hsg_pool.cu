@@ -285,6 +285,7 @@ struct hsg_pool {
   size_t stage_bytes = 0;
   bool dirty = true;
   int threads = 256, tile_sites = 512, blocks_per_sm = 8;
+  bool tuning_shape = false;  // the autotuner times the persistent kernels, and nothing beside them
   // Metropolis hits per pass over a colour (0: all of them in one pass).
   int hits_per_pass = 0;
   struct GraphKey {
@@ -1023,9 +1024,9 @@ hsg_status hsg_pool_sweep(hsg_pool* p, const hsg_schedule* sched, int n_sweeps) 
   // path below, as the sweep's own graph can be neither captured nor launched in it.
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if ((e = cudaStreamIsCapturing(p->stream, &cap)) != cudaSuccess) return pcuda(p, e, "pool sweep");
-  const bool batch = p->batched && cap == cudaStreamCaptureStatusNone;
+  const bool batch = p->batched && !p->tuning_shape && cap == cudaStreamCaptureStatusNone;
   const bool counted = n_sweeps >= kBatchGraphMin;  // the batches' sweeps as graphs
-  const bool resident = cap == cudaStreamCaptureStatusNone && resident_pool(p, sched);
+  const bool resident = !p->tuning_shape && cap == cudaStreamCaptureStatusNone && resident_pool(p, sched);
   if (batch || resident) {
     e = make_side_streams(p);
     if (e == cudaSuccess && batch) {
@@ -1263,12 +1264,12 @@ hsg_status hsg_pool_autotune(hsg_pool* p, const hsg_schedule* sched, int* thread
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
-  // One warm-up sweep (it also captures the graph), then two timed ones.
-  auto trial = [&](int t, int ts, int b, int h) {
+  // n timed sweeps in one call, after a call that captures the graphs.
+  auto trial = [&](int t, int ts, int b, int h, int warm_up, int n) {
     if (hsg_pool_config(p, t, ts, b, h) != HSG_OK) return true;
-    if ((st = hsg_pool_sweep(p, sched, 1)) != HSG_OK) return false;
+    if ((st = hsg_pool_sweep(p, sched, warm_up)) != HSG_OK) return false;
     cudaEventRecord(e0, p->stream);
-    if ((st = hsg_pool_sweep(p, sched, 2)) != HSG_OK) return false;
+    if ((st = hsg_pool_sweep(p, sched, n)) != HSG_OK) return false;
     cudaEventRecord(e1, p->stream);
     cudaEventSynchronize(e1);
     float ms = 0.0f;
@@ -1282,19 +1283,27 @@ hsg_status hsg_pool_autotune(hsg_pool* p, const hsg_schedule* sched, int* thread
     }
     return true;
   };
-  // Launch shape with every Metropolis hit in one pass, then, on that
-  // shape, the hits split over passes of 1, 2, 4, ... hits.
+  // Launch shape with every Metropolis hit in one pass, of the persistent kernels
+  // alone, on the lattices that they sweep once there are enough of them; then, on that
+  // shape, the hits split over passes of 1, 2, 4, ... hits, as a call runs them.
   const int cand_t[] = {128, 256};
   const int cand_ts[] = {256, 512, 1024, 2048};
   const int cand_b[] = {4, 8, 16};
-  bool ok = true;
-  for (int t : cand_t)
-    for (int ts : cand_ts)
-      for (int b : cand_b)
-        if (ok) ok = trial(t, ts, b, 0);
+  bool ok = hsg_pool_config(p, old_t, old_ts, old_b, 0) == HSG_OK && (st = sync_tables(p)) == HSG_OK;
+  best_h = 0;
+  if (ok && p->unbatched_left) {
+    p->tuning_shape = true;
+    for (int t : cand_t)
+      for (int ts : cand_ts)
+        for (int b : cand_b)
+          if (ok) ok = trial(t, ts, b, 0, 1, 2);
+    p->tuning_shape = false;
+  }
   const bool multi_hit = sched->kind == HSG_METROPOLIS || sched->kind == HSG_METROPOLIS_OR;
   const int shape_t = best_t, shape_ts = best_ts, shape_b = best_b;
-  for (int h = 1; ok && multi_hit && h < sched->hits; h *= 2) ok = trial(shape_t, shape_ts, shape_b, h);
+  best_ms = 1e30f;
+  for (int h = 0; ok && multi_hit && h < sched->hits && sched->hits > 1; h = h ? 2 * h : 1)
+    ok = trial(shape_t, shape_ts, shape_b, h, 10, 10);
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   // Restore the lattices and counters; keep the fastest configuration.

@@ -366,3 +366,24 @@ def test_pooled_l16_metropolis_matches_oracle_layer_by_layer(hsg):
                                   proposal=hsg.HSG_PROP_SPHERE)
                 check_one_sweep(L, Js[spec], before[slot], pool.spins(slot), oracle.MET, p,
                                 label=f"pooled L=16 sample {sample} sweep {n}")
+
+
+def test_autotune_keeps_a_shape_that_no_kernel_uses(hsg):
+    """All lattices in batches."""
+    with hsg.Pool(1 << 26, 16, torch.cuda.Stream()) as pool:
+        for k, L in enumerate((64, 66)):
+            pool.admit(L, 3, k)
+        hsg.hsg_pool_config(pool.pool, 64, 576, 5, 0)
+        for kw in (dict(kind=hsg.HSG_METROPOLIS, hits=4, proposal=1, n_or=1), dict(kind=hsg.HSG_HEATBATH)):
+            assert hsg.hsg_pool_autotune(pool.pool, hsg.schedule(**kw))[:3] == (64, 576, 5)
+
+
+def test_autotune_times_the_kernels_that_the_shape_is_for(hsg):
+    """Few small lattices take other kernels, all sweeps in one launch: the 24
+    shapes are timed on the persistent ones, three launches a sweep."""
+    with hsg.Pool(1 << 24, 16, torch.cuda.Stream()) as pool:
+        for k in range(8):
+            pool.admit(16, 3, k)
+        n = hsg.hsg_pool_launch_count(pool.pool)
+        hsg.hsg_pool_autotune(pool.pool, hsg.schedule(kind=hsg.HSG_HEATBATH))
+        assert hsg.hsg_pool_launch_count(pool.pool) - n == 24 * 3 * 3
