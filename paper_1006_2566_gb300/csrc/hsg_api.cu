@@ -594,12 +594,13 @@ bool use_resident(const hsg_ctx* c, const hsg_schedule* s) {
   return hsg::resident_fits(main_update(s), c->L, 1, false, c->sm_count);
 }
 
-// n_sweeps sweeps in the resident kernel, one launch up to each energy due.
+// n_sweeps sweeps in the resident kernel, a launch for as many as it takes at a time
+// or up to an energy due.
 hsg_status run_resident(hsg_ctx* c, const hsg_schedule* s, int n_sweeps) {
   const int upd = main_update(s);
   hsg_status st;
   for (int k = 0; k < n_sweeps;) {
-    uint64_t m = (uint64_t)(n_sweeps - k);
+    uint64_t m = (uint64_t)std::min(n_sweeps - k, hsg::kResidentSweeps);
     if (s->energy_every > 0) m = std::min(m, (uint64_t)s->energy_every - c->sweep % (uint64_t)s->energy_every);
     hsg::ResidentArgs a{};
     a.L = (uint32_t)c->L;

@@ -190,6 +190,11 @@ struct ResidentArgs {
   FastDiv by_plane, by_Lh;
 };
 constexpr int kResidentMaxL = 32;
+// Sweeps per launch: a pool's launch can hold every SM, and other streams' work, of
+// whatever priority, is let in between launches.  Beside 3000 heat-bath + 2 OR sweeps of 1200
+// L = 8 (39.1 ms) another stream's kernel waited 14.4 ms for one launch of all, now 1.3 ms; the
+// sweeps take 39.3 ms.
+constexpr int kResidentSweeps = 256;
 // Sites of a pool's small lattices up to which it takes them so (those from
 // L = 26 counted a quarter more).
 constexpr unsigned long long kResidentPoolSites = 640 * 1024;

@@ -1043,13 +1043,16 @@ hsg_status hsg_pool_sweep(hsg_pool* p, const hsg_schedule* sched, int n_sweeps) 
   // replayed; the legacy default stream cannot be captured, so there the
   // launches are issued directly.
   if (resident || (batch && !p->unbatched_left)) {
-    if (resident) e = sweep_resident(p, sched, n_sweeps);
-    // the device's counters follow the host's (the resident kernel read them)
-    if (e == cudaSuccess) {
-      k_pool_advance<<<cdiv_u((unsigned)p->max_slots, 256), 256, 0, p->stream>>>(p->d_desc, p->max_slots,
-                                                                                (uint32_t)n_sweeps);
+    for (int k = 0; k < n_sweeps && e == cudaSuccess;) {
+      const int m = resident ? std::min(n_sweeps - k, hsg::kResidentSweeps) : n_sweeps;
+      if (resident && k > 0) e = cudaEventRecord(p->fork_ev, p->stream);
+      if (resident && e == cudaSuccess) e = sweep_resident(p, sched, m);
+      if (e != cudaSuccess) break;
+      // the device's counters follow the host's (the resident kernel read them)
+      k_pool_advance<<<cdiv_u((unsigned)p->max_slots, 256), 256, 0, p->stream>>>(p->d_desc, p->max_slots, (uint32_t)m);
       p->launches += 1;
       e = cudaGetLastError();
+      k += m;
     }
   } else if (p->stream != nullptr) {
     if (!p->have_graph || !(p->gkey == key)) {

@@ -130,3 +130,42 @@ def test_a_device_without_room_for_the_cluster_takes_half_sweeps(hsg, L):
         hsg.hsg_test_no_clusters(0)
     assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
     assert out[0][2] == 1 and out[1][2] >= 20 and out[1][3] >= 20  # 5 x 4 half-sweeps and what goes with them
+
+
+def test_long_calls_let_other_streams_in(hsg):
+    """A pool's launch can hold every SM (here with one CTA a lattice, in more
+    than one wave); a call of many sweeps is several launches, between which
+    another stream's kernel runs.  The counters and the renormalisations go on
+    from launch to launch."""
+    kw = dict(kind=hsg.HSG_HEATBATH, n_or=2, renorm_every=100)
+    L, lattices, n = 8, 1200, 2000
+    with hsg.Pool(1 << 26, lattices, torch.cuda.Stream()) as pool, hsg.Lattice(L, 3, 700, stream=torch.cuda.Stream()) as lat:
+        slots = [pool.admit(L, 3, k, 0, 0.5) for k in range(lattices)]
+        lat.generate_couplings()
+        x = torch.zeros(1 << 20, device="cuda")
+        other = torch.cuda.Stream()
+        with torch.cuda.stream(other):
+            x += 1.0  # loads its kernel, which waits for the device
+        pool.sweep(hsg.schedule(**kw), 1)
+        pool.energies()
+        lat.sweep(hsg.schedule(T=0.5, **kw), 1)
+        torch.cuda.synchronize()
+        t = [torch.cuda.Event(enable_timing=True) for _ in range(3)]
+        t[0].record(other)
+        pool.sweep(hsg.schedule(**kw), n)
+        with torch.cuda.stream(other):
+            x += 1.0
+        t[1].record(other)
+        pool.energies()
+        t[2].record(other)
+        torch.cuda.synchronize()
+        # an eighth of the call is one launch, of which the first wave has to end
+        assert t[0].elapsed_time(t[1]) < 0.2 * t[0].elapsed_time(t[2])
+        launches = hsg.hsg_launch_count(lat.ctx)
+        lat.sweep(hsg.schedule(T=0.5, **kw), n)
+        assert hsg.hsg_launch_count(lat.ctx) - launches == 8  # 256 sweeps each
+        assert np.array_equal(pool.spins(slots[700]), lat.spins())
+        with hsg.Lattice(L, 3, 700, stream=torch.cuda.Stream()) as ref:
+            ref.generate_couplings()
+            ref.sweep(hsg.schedule(T=0.5, kernel=hsg.HSG_KERNEL_GLOBAL, **kw), 1 + n)
+            assert np.array_equal(lat.spins(), ref.spins())
