@@ -281,7 +281,7 @@ int slab_zc(int L, unsigned tiles, int sm_count) {
 //   4 hits     L = 40 3.06 / 2.04 / 2.06, 80 7.12 / 6.19 / 6.18, 110 15.3 / 14.8 / 14.4, 128 20.6 / 20.5 / 20.4
 enum Overlap { NONE, EARLY, LATE };
 template <int U>
-Overlap overlap(int L) {
+constexpr Overlap overlap(int L) {
   if (U == U_OR) return L <= 72 ? LATE : NONE;
   return L <= 90 ? LATE : L <= 126 ? EARLY : NONE;
 }
@@ -304,13 +304,14 @@ bool downward(const SweepArgs& a) {
   return a.colour == 1 && a.L >= kDownMinL && a.L <= (U == U_HB ? kDownMaxLHeatbath : kDownMaxL);
 }
 
-template <int U, int R, int MIN_BLOCKS, class Off, bool PACKED>
+// FROM: the smallest L that takes this shape.
+template <int U, int R, int MIN_BLOCKS, class Off, bool PACKED, int FROM = 0>
 cudaError_t launch_rows(const SweepArgs& a, cudaStream_t s) {
   const uint32_t columns = (uint32_t)a.Lh * (uint32_t)(a.L / R);
   const FastDiv by_lh = make_fastdiv((uint32_t)a.Lh);
   const dim3 grid(cdiv(columns, G_THREADS), (unsigned)a.L);
   const bool down = downward<U>(a);
-  if constexpr (sizeof(Off) == 4 && R < 4) {
+  if constexpr (overlap<U>(FROM) != NONE) {
     const Overlap o = overlap<U>(a.L);
     if (o != NONE)
       return launch_overlapped(k_half_sweep_rows<U, R, MIN_BLOCKS, Off, PACKED, true>, grid, dim3(G_THREADS), s, a, by_lh,
@@ -343,29 +344,34 @@ cudaError_t launch_rows(const SweepArgs& a, cudaStream_t s) {
 template <int U, bool PACKED>
 cudaError_t launch_global(const SweepArgs& a, cudaStream_t s) {
   constexpr bool MET = U != U_OR && U != U_HB;
-  if (a.L > kMaxOff32L) return launch_rows<U, 1, MET ? 1 : 12, unsigned long long, PACKED>(a, s);
+  static_assert(ZM_MIN_L <= kMaxOff32L, "the column march takes the float4 heat-bath beyond");
+  if constexpr (U != U_HB || PACKED) {
+    if (a.L > kMaxOff32L) return launch_rows<U, 1, MET ? 1 : 12, unsigned long long, PACKED, kMaxOff32L + 2>(a, s);
+  }
   if constexpr (U == U_OR) {
-    if (PACKED && a.L >= 160) return launch_rows<U, 2, 10, uint32_t, PACKED>(a, s);
+    if constexpr (PACKED) {
+      if (a.L >= 160) return launch_rows<U, 2, 10, uint32_t, PACKED, 160>(a, s);
+    }
     return launch_rows<U, 1, 12, uint32_t, PACKED>(a, s);
   } else if constexpr (U == U_HB) {
     if (a.L < 96) return launch_rows<U, 1, 12, uint32_t, PACKED>(a, s);
-    return launch_rows<U, 2, PACKED ? 10 : 16, uint32_t, PACKED>(a, s);
+    return launch_rows<U, 2, PACKED ? 10 : 16, uint32_t, PACKED, 96>(a, s);
   } else if constexpr (PACKED) {
-    if (a.L >= 160) return launch_rows<U, 2, 1, uint32_t, PACKED>(a, s);
+    if (a.L >= 160) return launch_rows<U, 2, 1, uint32_t, PACKED, 160>(a, s);
     return launch_rows<U, 1, 1, uint32_t, PACKED>(a, s);
   } else {
     if (a.L < 96) return launch_rows<U, 1, 1, uint32_t, PACKED>(a, s);
     if constexpr (U == U_MET_SPHERE) {
-      return launch_rows<U, 2, 10, uint32_t, PACKED>(a, s);
+      return launch_rows<U, 2, 10, uint32_t, PACKED, 96>(a, s);
     } else if constexpr (U == U_MET_BALL) {
-      if (a.hits > 1 && a.L >= 220 && a.L % 4 == 0) return launch_rows<U, 4, 1, uint32_t, PACKED>(a, s);
-      if (a.hits > 1 && a.L >= 124) return launch_rows<U, 2, 1, uint32_t, PACKED>(a, s);
-      return launch_rows<U, 1, 12, uint32_t, PACKED>(a, s);
+      if (a.hits > 1 && a.L >= 220 && a.L % 4 == 0) return launch_rows<U, 4, 1, uint32_t, PACKED, 220>(a, s);
+      if (a.hits > 1 && a.L >= 124) return launch_rows<U, 2, 1, uint32_t, PACKED, 124>(a, s);
+      return launch_rows<U, 1, 12, uint32_t, PACKED, 96>(a, s);
     } else if constexpr (U == U_MET_OR_SPHERE) {
-      if (a.hits == 1) return launch_rows<U, 1, 14, uint32_t, PACKED>(a, s);
-      return launch_rows<U, 2, 8, uint32_t, PACKED>(a, s);
+      if (a.hits == 1) return launch_rows<U, 1, 14, uint32_t, PACKED, 96>(a, s);
+      return launch_rows<U, 2, 8, uint32_t, PACKED, 96>(a, s);
     } else {
-      return launch_rows<U, 2, 1, uint32_t, PACKED>(a, s);
+      return launch_rows<U, 2, 1, uint32_t, PACKED, 96>(a, s);
     }
   }
 }
