@@ -829,7 +829,7 @@ BATCH = dict(samples=512, replicas=2, sides=(16, 24, 32, 48), seed=4, hits=4, pr
              renorm_every=10, sweeps_per_step=10, T=None,
              desc=("batched: 512 samples x 2 replicas, L uniform in {16,24,32,48} (seeded), T_s = 0.2 + 0.8 s/511, "
                    "Gaussian J per sample (device Philox + Box-Muller), 4-hit Metropolis (ball, 0.5) + 2 OR per "
-                   "sweep, renorm every 10; one pool, one graph replay per sweep; 1 step = 10 sweeps"))
+                   "sweep, renorm every 10; one pool, graph-replayed sweeps; 1 step = 10 sweeps"))
 # The L = 16 single-lattice workload (l16_met: 1-hit Metropolis, uniform-
 # sphere proposal, T = 1) as it is meant to run: many independent samples
 # in one pool.

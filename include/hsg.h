@@ -85,8 +85,9 @@ enum {
                           * device's L2 (three quarters of it with renorm_every = 1,
                           * which WAVE fuses), so that the sweep streams much of it
                           * from HBM; else GLOBAL.  hsg_sweep runs all sweeps up to
-                          * an energy in one launch where the lattice is small (L <=
-                          * 32, few hits): the same results */
+                          * an energy (256 at most) in one launch where the lattice is
+                          * small (L <= 32, few hits) and the device can place its
+                          * thread-block cluster: the same results */
   HSG_KERNEL_GLOBAL = 1, /* one thread per one to four sites of a column, neighbours through L1/L2 (heat-bath from
                           * L = 152: one thread per six-plane column, carrying its column's
                           * neighbours; the same results) */
@@ -308,7 +309,10 @@ hsg_status hsg_kernel_for(hsg_ctx* ctx, const hsg_schedule* schedule, int* kerne
  * by CUDA events on its stream.  hsg_profile_read synchronises, adds the
  * elapsed time (ms) and the number of launches of class `kclass`
  * (HSG_PROF_*) recorded since the last reset, and hsg_profile_reset
- * clears the records.  hsg_launch_count counts every kernel launch of the
+ * clears the records.  The launches are then those of single half-sweeps, and issued
+ * one by one: no CUDA graphs, and none that runs all the sweeps of a small lattice
+ * (HSG_KERNEL_AUTO, L <= 32), whose time per sweep the records do not show.
+ * hsg_launch_count counts every kernel launch of the
  * context since creation, profiled or not.
  */
 hsg_status hsg_profile(hsg_ctx* ctx, int on);

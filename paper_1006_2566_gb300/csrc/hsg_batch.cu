@@ -12,11 +12,11 @@
 // (bound by memory).  The lattices are kernel parameters: the constant bank gives
 // every CTA its lattice without dependent loads, and there is no table to upload.
 //
-// Measured on GB300, 4-hit Metropolis + 2 OR, us per sweep, against the
-// persistent kernels: 128 lattices of L = 32 and 48 469 -> 320; 24 of 64 to 96
-// 650 -> 457; 45 of 32 to 96 771 -> 531.  Per half-sweep of the 24: OR 86.6 -> 47, 4 hits
-// 143.7 -> 129, heat-bath 101.5 -> 75.  By batch size and streams (the 24): 1000 MB, 1:
-// 550; 64 MB, 1: 600; 64, 2: 486; 48, 2: 468; 32, 3: 457; 24, 4: 459; 128, 2: 559.
+// Measured on GB300, 4-hit Metropolis + 2 OR, us per sweep in calls of 40, against the
+// persistent kernels: 128 lattices of L = 32 and 48 474 -> 329; 24 of 64 to 96
+// 659 -> 416; 45 of 32 to 96 767 -> 510.  Per half-sweep of the 24: OR 88 -> 42, 4 hits
+// 155 -> 125, heat-bath 110 -> 78.  By batch size and streams (the 24, launched one by one, then
+// 457): 1000 MB, 1: 550; 64 MB, 1: 600; 64, 2: 486; 48, 2: 468; 32, 3: 457; 24, 4: 459; 128, 2: 559.
 #include "hsg_device.cuh"
 #include "hsg_internal.h"
 
