@@ -880,7 +880,9 @@ hsg_status hsg_sweep(hsg_ctx* c, const hsg_schedule* s, int n_sweeps) {
     graphs = false;
   c->last = *s;
   c->have_last = true;
-  bool look_short = graphs && !cadence;  // asked once a call where there is none
+  // Asked once a call where there is none, and not while the caller captures: the
+  // direct launches can be part of its graph, a graph of ours can not.
+  bool look_short = graphs && !cadence && !stream_captured(c);
   while (k < n_sweeps) {
     SweepGraph* g = nullptr;
     if (graphs && (!cadence || c->sweep % (uint64_t)period == 0) && n_sweeps - k >= period) {

@@ -78,3 +78,27 @@ def test_short_calls_get_a_graph(hsg, n_or, calls, captured, launched, kernel):
         assert counts == [captured, launched]
     else:  # other launches a sweep, buffers that swap
         assert counts[0] <= 4
+
+
+def test_short_calls_stay_launches_in_the_callers_capture(hsg):
+    """What a long call leaves to direct launches can be captured by the caller,
+    also where a call like it has its own graph; each replay is new sweeps."""
+    kw = dict(kind=hsg.HSG_HEATBATH, T=0.5, n_or=5)
+    stream = torch.cuda.Stream()
+    with hsg.Lattice(40, 5, stream=stream) as lat, hsg.Lattice(40, 5) as ref:
+        for x in (lat, ref):
+            x.generate_couplings()
+        sched = hsg.schedule(**kw)
+        for n in (50, 2, 2, 2):
+            lat.sweep(sched, n)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=stream):
+            for n in (2, 3, 3):
+                lat.sweep(sched, n)
+        for _ in range(2):
+            with torch.cuda.stream(stream):
+                g.replay()
+        torch.cuda.synchronize()
+        ref.sweep(sched, 56 + 2 * 8)
+        assert np.array_equal(lat.spins(), ref.spins())
