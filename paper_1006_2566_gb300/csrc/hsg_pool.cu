@@ -1306,7 +1306,7 @@ hsg_status hsg_pool_autotune(hsg_pool* p, const hsg_schedule* sched, int* thread
   const int shape_t = best_t, shape_ts = best_ts, shape_b = best_b;
   best_ms = 1e30f;
   for (int h = 0; ok && multi_hit && h < sched->hits && sched->hits > 1; h = h ? 2 * h : 1)
-    ok = trial(shape_t, shape_ts, shape_b, h, 10, 10);
+    ok = trial(shape_t, shape_ts, shape_b, h, p->batched ? 10 : 1, 10);  // (the batches' graphs want a long call)
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   // Restore the lattices and counters; keep the fastest configuration.
