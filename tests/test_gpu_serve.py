@@ -28,7 +28,8 @@ def hsg():
 
 
 def test_each_result_is_the_same_alone_and_in_the_mix(hsg):
-    reqs = serve.poisson_trace(14, rate_per_s=300.0, seed=8, sides=(8, 12, 16, 20, 24), sweep_range=(4, 30))
+    # arriving faster than they are served (0.3 ms each), so that they share the pool
+    reqs = serve.poisson_trace(14, rate_per_s=20000.0, seed=8, sides=(8, 12, 16, 20, 24), sweep_range=(4, 30))
     kw = dict(kind=hsg.HSG_METROPOLIS, hits=4, proposal=hsg.HSG_PROP_BALL, step=0.5, n_or=2, renorm_every=10)
     budget = 3 * 28 * 24 ** 3  # room for three of the largest lattices: later arrivals must wait
     res, st = serve.serve(reqs, kw, budget, 6, torch.cuda.Stream(), tick_sweeps=4, keep_spins=True, autotune=False)
