@@ -427,10 +427,10 @@ hsg_status hsg_pool_usage(hsg_pool* pool, uint64_t* bytes_used, uint64_t* bytes_
  * pass).  The shape is that of the kernels that sweep the lattices of L < 32 of
  * pools with more of them than a few (above); hits per pass h > 0 apply to all, and
  * few small lattices too then take those kernels.  hsg_pool_autotune times
- * these kernels in every launch shape, with all hits in one pass, on the lattices of L < 32 (one
- * warm-up and two timed sweeps each; a pool without any keeps its shape), then that shape with all
- * hits and with 1, 2, 4, ... hits per pass (Metropolis schedules with more than one hit; a
- * warm-up call and ten timed sweeps each), on the admitted lattices, restores the lattices and
+ * calls with these kernels in every launch shape, with all hits in one pass (one
+ * warm-up and two timed sweeps each; a pool without lattices of L < 32 keeps its shape), then that shape with all
+ * hits and with 1, 2, 4, ... hits per pass (Metropolis schedules with more than one hit; one
+ * warm-up sweep and two timed ones each, ten where few small lattices are all there is below L = 32), on the admitted lattices, restores the lattices and
  * counters afterwards, keeps the fastest configuration and reports it.  Results
  * do not depend on the configuration but for the last bits of the energies, whose
  * fp64 sums run tile by tile.  Errors: HSG_EINVAL (NULL pool, values

@@ -285,7 +285,7 @@ struct hsg_pool {
   size_t stage_bytes = 0;
   bool dirty = true;
   int threads = 256, tile_sites = 512, blocks_per_sm = 8;
-  bool tuning_shape = false;  // the autotuner times the persistent kernels, and nothing beside them
+  bool tuning_shape = false;  // the autotuner times the persistent kernels' launch shape: none resident
   // Metropolis hits per pass over a colour (0: all of them in one pass).
   int hits_per_pass = 0;
   struct GraphKey {
@@ -1024,7 +1024,7 @@ hsg_status hsg_pool_sweep(hsg_pool* p, const hsg_schedule* sched, int n_sweeps) 
   // path below, as the sweep's own graph can be neither captured nor launched in it.
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if ((e = cudaStreamIsCapturing(p->stream, &cap)) != cudaSuccess) return pcuda(p, e, "pool sweep");
-  const bool batch = p->batched && !p->tuning_shape && cap == cudaStreamCaptureStatusNone;
+  const bool batch = p->batched && cap == cudaStreamCaptureStatusNone;
   const bool counted = n_sweeps >= kBatchGraphMin;  // the batches' sweeps as graphs
   const bool resident = !p->tuning_shape && cap == cudaStreamCaptureStatusNone && resident_pool(p, sched);
   if (batch || resident) {
@@ -1286,9 +1286,13 @@ hsg_status hsg_pool_autotune(hsg_pool* p, const hsg_schedule* sched, int* thread
     }
     return true;
   };
-  // Launch shape with every Metropolis hit in one pass, of the persistent kernels
-  // alone, on the lattices that they sweep once there are enough of them; then, on that
-  // shape, the hits split over passes of 1, 2, 4, ... hits, as a call runs them.
+  // Launch shape with every Metropolis hit in one pass, where there are lattices for
+  // the persistent kernels (few of them, which the resident kernel would take, are timed
+  // on these too: the shape is for when there are more).  Batches run beside them as
+  // in any call, since what is best alone is not best there: 256 lattices of L = 16 to 48, four
+  // shapes, those of 16 and 24 alone / the pool, us a sweep: (256, 1024, 16) 60.3 / 384.7, (128,
+  // 512, 8) 62.4 / 375.7, (128, 1024, 4) 66.4 / 371.2, (128, 2048, 4) 96 / 370.8.  Then, on
+  // that shape, the hits split over passes of 1, 2, 4, ... hits.
   const int cand_t[] = {128, 256};
   const int cand_ts[] = {256, 512, 1024, 2048};
   const int cand_b[] = {4, 8, 16};
@@ -1304,9 +1308,11 @@ hsg_status hsg_pool_autotune(hsg_pool* p, const hsg_schedule* sched, int* thread
   }
   const bool multi_hit = sched->kind == HSG_METROPOLIS || sched->kind == HSG_METROPOLIS_OR;
   const int shape_t = best_t, shape_ts = best_ts, shape_b = best_b;
+  // (with all hits in one launch few small lattices are resident, which pays off over a call)
+  const int timed = ok && resident_pool(p, sched) ? 10 : 2;
   best_ms = 1e30f;
   for (int h = 0; ok && multi_hit && h < sched->hits && sched->hits > 1; h = h ? 2 * h : 1)
-    ok = trial(shape_t, shape_ts, shape_b, h, p->batched ? 10 : 1, 10);  // (the batches' graphs want a long call)
+    ok = trial(shape_t, shape_ts, shape_b, h, 1, timed);
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   // Restore the lattices and counters; keep the fastest configuration.
