@@ -670,7 +670,6 @@ void make_batches(hsg_pool* p) {
     l.beta = beta_of(sl.T);
     l.by_lh = hsg::make_fastdiv(l.Lh);
   }
-  p->batches_ok = true;
 }
 
 // The launches of one sweep of a batch, in the single-lattice order.
@@ -742,7 +741,7 @@ __global__ void k_set_done(unsigned long long* done, int n, unsigned long long v
 cudaError_t prepare_batches(hsg_pool* p, const hsg_pool::GraphKey& key, bool counted) {
   const bool ok = p->batches_ok && p->batch_swept < 1u << 30;
   if (!ok || !(p->batch_key == key)) {
-    p->batches_ok = false;  // until there are graphs for them
+    p->batches_ok = false;  // until there is room for their graphs (either may run out of host memory)
     if (!ok) make_batches(p);
     for (size_t i = p->batches.size(); i < p->batch_graphs.size(); ++i)
       if (p->batch_graphs[i].exec) cudaGraphExecDestroy(p->batch_graphs[i].exec);
